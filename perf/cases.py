@@ -93,7 +93,7 @@ def draw(rng):
         return _solve_case(None, "poisson", 3, e + 1, levels, precision, 1e-8, m=m)
     if kind == "matrix_free":
         e, levels = _elements(rng, 16, 128, (4, 5, 6, 7), 2)
-        return _solve_case(None, "kappa", 3, e + 1, levels, MIXED, 1e-10, rng.choice([0x3F, 0x15, 0x1F]), True, m)
+        return _solve_case(None, "kappa", 3, e + 1, levels, MIXED, 1e-10, rng.choice([0x3F, 0x15, 0x1F]), True, min(m, WINDOW))
     if kind == "kappa2d":
         e, levels = _elements(rng, 64, 1024, (4, 5, 6, 7), 3)
         return _solve_case(None, "kappa", 2, e + 1, levels, MIXED, 1e-10, m=min(m, WINDOW))

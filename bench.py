@@ -98,11 +98,20 @@ def stencil_words(dim: int, w: int, vector: bool = False) -> int:
     return full // 2 + 1 if w == 4 else full
 
 
-def kernel_work(cls: str, n: int, C: int, cnt: int, w: int, S: int = 27):
+def kernel_work(cls: str, n: int, C: int, cnt: int, w: int, S: int = 27, recurrence: bool = True):
     """Algorithmic HBM bytes and flops of one launch on the fine grid (per
     unknown figures x n; cnt = blocks in the window at that launch; S =
     stored stencil coefficients per unknown, stencil_words).  The flops
-    count the full stencil's products whatever is stored."""
+    count the full stencil's products whatever is stored.  recurrence: A P
+    formed as A Z - sum A P_j beta_j within the orthogonalisation, with the
+    Gram sums; the library forms it by the block SpMM of P (False)."""
+    if cls == "orth_update" and not recurrence:      # read Z, P_j; write P
+        return (cnt * C + 2 * C) * w * n, 2 * cnt * C * C * n
+    if cls == "orth_gram" and not recurrence:        # read the new P, A P and r; upper triangle of P^T A P, P^T r
+        return (2 * C + 1) * w * n, 2 * (C * (C + 1) // 2 + C) * n
+    if cls == "spmm" and not recurrence:             # read stencil, P; write A P
+        taps = 81 if S == 81 else (27 if S > 9 else 9)
+        return (S + 2 * C) * w * n, 2 * taps * C * n
     if cls == "orth_update":      # read Z, AZ, P_j, AP_j, r; write P, AP; sym Gram + P^T r
         return (2 * cnt * C + 4 * C + 1) * w * n, 2 * (2 * cnt * C * C + C * (C + 1) + C) * n
     if cls == "gram_window":      # read AP_j, Z
@@ -176,7 +185,8 @@ def roofline(trace, ns, C, m, w, peaks, fp64_alu_peak_tflops, S=27, vector=False
         elif cls == "prolong":   # composite: write J fine columns, read every coarse correction once
             b, f = (J * ns[J] + sum(ns[:J])) * w, 2 * 8 * J * ns[J]
         elif cls in ("orth_update", "gram_window", "spmm", "update_xr", "orth_gram"):
-            b, f = kernel_work(cls, ns[J], C, cnt, w, s_fine if (s_fine is not None and cls == "spmm") else S)
+            b, f = kernel_work(cls, ns[J], C, cnt, w, s_fine if (s_fine is not None and cls == "spmm") else S,
+                               recurrence=False)
         if cls == dom:
             if b is not None:
                 bytes_sum += b
@@ -1095,8 +1105,8 @@ def amg_roofline(trace, ns, nnzA, nnzP, C, m, w, peaks):
             jp += 1
         elif cls == "spmm":
             b = nnzA[J] * (4 + w) + 2 * C * ns[J] * w
-        elif cls in ("orth_update", "gram_window", "update_xr"):
-            b, _ = kernel_work(cls, ns[J], C, cnt, w)
+        elif cls in ("orth_update", "gram_window", "update_xr", "orth_gram"):
+            b, _ = kernel_work(cls, ns[J], C, cnt, w, recurrence=False)
         if cls == dom:
             if b is not None:
                 bytes_sum += b

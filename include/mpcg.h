@@ -398,8 +398,8 @@ mpcg_status mg_get_operator(mg_hierarchy* h, int level, double* planes_dev);   /
  * in MPCG_NUM_KERNEL_CLASSES classes named by mpcg_kernel_class_name():
  * pack, residual, init, restrict, coarse_solve, prolong, jacobi, spmm,
  * gram_window, small_beta, orth_update, small_alpha, update_xr, check, aux,
- * net (the learned column) and orth_gram (the Gram partials of the new block
- * in double-word arithmetic, a kernel of its own there).
+ * net (the learned column) and orth_gram (the Gram sums P^T A P and P^T r of
+ * the new block).
  *
  * mpcg_solve_profiled runs mpcg_solve with direct kernel launches (no graph)
  * and a CUDA event pair around every launch on the hierarchy's stream; it

@@ -123,11 +123,11 @@ struct Solver {
   T* zc[kMaxLevels] = {};
   T* tmp[kMaxLevels] = {};
   T* tmp2[kMaxLevels] = {};
-  T *x = nullptr, *r = nullptr, *b = nullptr, *Z = nullptr, *AZ = nullptr;
+  T *x = nullptr, *r = nullptr, *b = nullptr, *Z = nullptr;
   T* Zmg = nullptr;   // the per-grid columns when they are summed into one
   Window<T> win = {};
   DevState* state = nullptr;
-  double *part_res = nullptr, *part_zaz = nullptr, *part_W = nullptr, *part_G = nullptr, *part_r = nullptr;
+  double *part_res = nullptr, *part_W = nullptr, *part_G = nullptr, *part_r = nullptr;
   double* small_scratch = nullptr;   // reduced values of the small solves
   unsigned* counters = nullptr;      // last-block counters of small_beta / small_alpha
   int* flag = nullptr;               // "some problem still running" (batched loop condition)
@@ -362,7 +362,6 @@ mpcg_status build_solver(mg_hierarchy* h, Solver<T>& S) {
   CKS(S.mem.get(&S.b, gf.cp, s));
   CKS(S.mem.get(&S.Z, (size_t)C * gf.cp, s));
   if (h->opt.sum_columns) CKS(S.mem.get(&S.Zmg, (size_t)h->levels * gf.cp, s));
-  CKS(S.mem.get(&S.AZ, (size_t)C * gf.cp, s));
   for (int j = 0; j < S.m; ++j) {
     CKS(S.mem.get(&S.win.P[j], (size_t)C * gf.cp, s));
     CKS(S.mem.get(&S.win.AP[j], (size_t)C * gf.cp, s));
@@ -383,7 +382,6 @@ mpcg_status build_solver(mg_hierarchy* h, Solver<T>& S) {
   // (the autotuner can change the shapes after the buffers exist)
   const size_t sbc = (size_t)stream_blocks_cap(gf), gcc = (size_t)gram_chunks_cap(gf);
   CKS(S.mem.get(&S.part_res, nb * 2 * sbc, s));
-  CKS(S.mem.get(&S.part_zaz, nb * C * sbc, s));
   CKS(S.mem.get(&S.part_W, nb * S.m * C * C * gcc, s));
   CKS(S.mem.get(&S.part_G, nb * (C * (C + 1) / 2 + C) * sbc, s));
   CKS(S.mem.get(&S.part_r, nb * sbc, s));
@@ -623,7 +621,7 @@ void enqueue_mg_algebraic(mg_hierarchy* h, Solver<T>& S, const T* r, T* Z, const
     const GridDesc& gf = h->lev[j].g;
     const GridDesc& gc = h->lev[j - 1].g;
     LAUNCH(h, K_RESTRICT, s,
-           launch_ell_spmm<T>(ell_of<T>(h->lev[j].eR), rj + gf.G, gf.cp, S.rlev[j - 1] + gc.G, gc.cp, 1, nullptr, 0,
+           launch_ell_spmm<T>(ell_of<T>(h->lev[j].eR), spmm_io<T>(rj + gf.G, S.rlev[j - 1] + gc.G), gf.cp, gc.cp, 1,
                               state, s));
     rj = S.rlev[j - 1];
     if (j - 1 >= 1) {
@@ -641,8 +639,8 @@ void enqueue_mg_algebraic(mg_hierarchy* h, Solver<T>& S, const T* r, T* Z, const
     const GridDesc& gk = h->lev[k].g;
     T* dst = k < J ? S.zc[k] : Z;
     LAUNCH(h, K_PROLONG, s,
-           launch_ell_spmm<T>(ell_of<T>(h->lev[k].eP), S.zc[k - 1] + gc.G, gc.cp, dst + gk.G, gk.cp, k, nullptr, 0,
-                              state, s));
+           launch_ell_spmm<T>(ell_of<T>(h->lev[k].eP), spmm_io<T>(S.zc[k - 1] + gc.G, dst + gk.G), gc.cp, gk.cp, k, state,
+                              s));
   }
   cudaStreamWaitEvent(s, h->ev_fine, 0);
 }
@@ -653,7 +651,8 @@ void launch_fine_residual(mg_hierarchy* h, const T* b, const T* x, T* r, double*
                           const int* xnz) {
   const Level& L = h->lev[h->levels - 1];
   if (h->algebraic)
-    launch_ell_residual<T>(ell_of<T>(L.eA), b + L.g.G, x + L.g.G, r + L.g.G, part, stream_blocks(L.g), s, xnz);
+    launch_ell_residual<T>(ell_of<T>(L.eA), b + L.g.G, x + L.g.G, r + L.g.G, part, stream_blocks(L.g),
+                           stream_threads(L.g), s, xnz);
   else
     launch_residual<T>(L.g, st_of<T>(L), b, x, r, part, s, xnz);
 }
@@ -723,7 +722,7 @@ void enqueue_vcycle(mg_hierarchy* h, Solver<T>& S, const T* r, T* out, const Dev
       LAUNCH(h, K_RESIDUAL, s,
              launch_ell_defect<T>(ell_of<T>(L.eA), rhs(j) + G, it(j) + G, S.tmp[j] + G, state, s));
       LAUNCH(h, K_RESTRICT, s,
-             launch_ell_spmm<T>(ell_of<T>(L.eR), S.tmp[j] + G, L.g.cp, S.rlev[j - 1] + gc.G, gc.cp, 1, nullptr, 0,
+             launch_ell_spmm<T>(ell_of<T>(L.eR), spmm_io<T>(S.tmp[j] + G, S.rlev[j - 1] + gc.G), L.g.cp, gc.cp, 1,
                                 state, s));
     } else {
       LAUNCH(h, K_RESIDUAL, s, launch_defect<T>(L.g, st_of<T>(L), rhs(j), it(j), S.tmp[j], state, s));
@@ -768,6 +767,30 @@ void enqueue_any(mg_hierarchy* h, Solver<T>& S, cudaGraphConditionalHandle cond,
   if (use_cond) LAUNCH(h, K_CHECK, s, launch_set_cond(S.flag, cond, s));
 }
 
+// A P of the block being built (the ring slot after the newest).
+template <typename T>
+void enqueue_block_spmm(mg_hierarchy* h, Solver<T>& S, cudaStream_t s) {
+  const Level& L = h->lev[h->levels - 1];
+  const int C = S.C;
+  if (h->algebraic) {
+    LAUNCH(h, K_SPMM, s,
+           launch_ell_spmm<T>(ell_of<T>(L.eA), spmm_ring(S.win, S.m, L.g.G), L.g.cp, L.g.cp, C, S.state, s));
+    return;
+  }
+  const SpmmIO<T> io = spmm_ring(S.win, S.m);
+  if constexpr (std::is_same<T, float>::value) {
+    if (L.kq32) {   // fine operator rebuilt from the element coefficients
+      LAUNCH(h, K_SPMM, s, launch_spmm_mf(L.g, L.kq32, io, C, spmm_blocks<T>(L.g, C), S.state, s));
+      return;
+    }
+    if (L.sth32) {   // the symmetric half of the stored stencil
+      LAUNCH(h, K_SPMM, s, launch_spmm_sym(L.g, L.sth32, io, C, S.state, s));
+      return;
+    }
+  }
+  LAUNCH(h, K_SPMM, s, launch_spmm<T>(L.g, st_of<T>(L), io, C, S.state, s));
+}
+
 template <typename T>
 void enqueue_body(mg_hierarchy* h, Solver<T>& S, cudaGraphConditionalHandle cond, int use_cond, cudaStream_t s) {
   const Level& L = h->lev[h->levels - 1];
@@ -790,31 +813,13 @@ void enqueue_body(mg_hierarchy* h, Solver<T>& S, cudaGraphConditionalHandle cond
              launch_net_infer<T>(L.g, 1, S.r, L.g.len, h->net_c, h->net_wtc, S.state, nullptr,
                                  S.Z + (size_t)(C - 1) * L.g.len, h->net_err, s));
   }
-  bool mf = false;
-  if (h->algebraic) {
-    LAUNCH(h, K_SPMM, s,
-           launch_ell_spmm<T>(ell_of<T>(L.eA), S.Z + L.g.G, L.g.cp, S.AZ + L.g.G, L.g.cp, C, S.part_zaz,
-                              spmm_blocks<T>(L.g, C), S.state, s));
-    mf = true;
-  }
-  if constexpr (std::is_same<T, float>::value) {
-    if (!mf && L.kq32 && C <= 12) {   // fine operator rebuilt from the element coefficients
-      LAUNCH(h, K_SPMM, s,
-             launch_spmm_mf(L.g, L.kq32, S.Z, S.AZ, C, spmm_blocks<T>(L.g, C), S.part_zaz, S.state, s));
-      mf = true;
-    } else if (!mf && L.sth32) {   // the symmetric half of the stored stencil
-      LAUNCH(h, K_SPMM, s, launch_spmm_sym(L.g, L.sth32, S.Z, S.AZ, C, S.part_zaz, S.state, s));
-      mf = true;
-    }
-  }
-  if (!mf) LAUNCH(h, K_SPMM, s, launch_spmm<T>(L.g, st_of<T>(L), S.Z, S.AZ, C, S.part_zaz, S.state, s));
   LAUNCH(h, K_GRAM, s, launch_gram_window<T>(L.g, S.win, S.Z, C, S.m, S.part_W, S.state, s));
-  LAUNCH(h, K_BETA, s, launch_small_beta(S.state, h->nb, S.part_W, gram_chunks(L.g), C, S.small_scratch, S.counters,
-                                         s));
-  LAUNCH(h, K_ORTH, s, launch_orth_update<T>(L.g, S.win, S.Z, S.AZ, S.r, C, S.part_G, S.state, s));
-  if constexpr (kIsDw<T>) LAUNCH(h, K_OGRAM, s, launch_orth_gram_dw(L.g, S.win, S.r, C, S.part_G, S.state, s));
-  LAUNCH(h, K_ALPHA, s, launch_small_alpha(S.state, h->nb, S.part_G, stream_blocks(L.g), S.part_zaz,
-                                          spmm_blocks<T>(L.g, C), spmm_blocks<T>(L.g, C), C, S.alpha_hist,
+  LAUNCH(h, K_BETA, s, launch_small_beta(S.state, h->nb, S.part_W, gram_shape<T>(L.g, C, S.m), C, S.small_scratch,
+                                         S.counters, s));
+  LAUNCH(h, K_ORTH, s, launch_orth_update<T>(L.g, S.win, S.Z, C, S.state, s));
+  enqueue_block_spmm<T>(h, S, s);
+  LAUNCH(h, K_OGRAM, s, launch_block_gram<T>(L.g, S.win, S.r, C, S.part_G, S.state, s));
+  LAUNCH(h, K_ALPHA, s, launch_small_alpha(S.state, h->nb, S.part_G, stream_blocks(L.g), C, S.alpha_hist,
                                           (long long)S.hist_cap * C, S.small_scratch, S.counters, s));
   LAUNCH(h, K_UPDATE, s, launch_update_xr<T>(L.g, S.win, S.x, S.r, C, S.part_r, S.state, s));
   LAUNCH(h, K_CHECK, s, launch_check(S.state, h->nb, S.part_r, stream_blocks(L.g), S.res_hist, S.hist_cap, cond,
@@ -2480,10 +2485,10 @@ mpcg_status mg_apply_operator(mg_hierarchy* h, int level, const double* X, doubl
     const int nc = ncols - c0 < chunk ? ncols - c0 : chunk;
     launch_pack<double, double>(L.g, X + (size_t)c0 * L.g.n, L.g.n, xp, nc, s);
     if (h->algebraic)
-      launch_ell_spmm<double>(ell_of<double>(L.eA), xp + L.g.G, L.g.len, yp + L.g.G, L.g.len, nc, nullptr, 0, nullptr,
-                              s);
+      launch_ell_spmm<double>(ell_of<double>(L.eA), spmm_io<double>(xp + L.g.G, yp + L.g.G), L.g.len, L.g.len, nc,
+                              nullptr, s);
     else
-      launch_spmm<double>(L.g, L.st64, xp, yp, nc, nullptr, nullptr, s);
+      launch_spmm<double>(L.g, L.st64, spmm_io<double>(xp, yp), nc, nullptr, s);
     launch_unpack<double, double>(L.g, yp, Y + (size_t)c0 * L.g.n, L.g.n, nc, s);
   }
   cudaError_t e = cudaStreamSynchronize(s);
@@ -2542,8 +2547,8 @@ mpcg_status mg_apply_operator_f32(mg_hierarchy* h, int level, const double* X, d
   for (int c0 = 0; c0 < ncols; c0 += chunk) {
     const int nc = ncols - c0 < chunk ? ncols - c0 : chunk;
     launch_pack<double, float>(L.g, X + (size_t)c0 * L.g.n, L.g.n, xp, nc, s);
-    if (L.sth32) launch_spmm_sym(L.g, L.sth32, xp, yp, nc, nullptr, nullptr, s);
-    else launch_spmm<float>(L.g, L.st32, xp, yp, nc, nullptr, nullptr, s);
+    if (L.sth32) launch_spmm_sym(L.g, L.sth32, spmm_io<float>(xp, yp), nc, nullptr, s);
+    else launch_spmm<float>(L.g, L.st32, spmm_io<float>(xp, yp), nc, nullptr, s);
     launch_unpack<float, double>(L.g, yp, Y + (size_t)c0 * L.g.n, L.g.n, nc, s);
   }
   cudaError_t e = cudaStreamSynchronize(s);
@@ -2739,7 +2744,7 @@ void net_batch_step(NetBatch& nb, const GridDesc& g, int nimg, const float* c, c
     launch_net_infer<float>(g, nimg, nb.rb, g.len, c, nb.wtc, nullptr, nb.y, (float*)nullptr, nb.terr, s, nullptr,
                             nb.a);
   }
-  launch_spmm<float>(g, st32, nb.y, nb.ay, nimg, nullptr, nullptr, s);
+  launch_spmm<float>(g, st32, spmm_io<float>(nb.y, nb.ay), nimg, nullptr, s);
   launch_net_loss_grad(g, nimg, nb.y, nb.ay, nb.eb, nb.aeb, nb.dots, nb.coef, loss_sum, nb.dy, s);
   if (nb.net3) launch_net3_backward(g, nimg, nb.wtc, nb.a, nb.dy, nb.gr, nb.d4, nb.terr, s);
   else launch_net_backward(g, nimg, wq, nb.a, nb.dy, nb.gr, nb.terr, s);
@@ -2969,7 +2974,7 @@ mpcg_status mg_learned_grad(mg_hierarchy* h, const float* params, const float* r
   launch_pack<float, float>(g, rhat_dev, g.n, nbt.rb, nimg, s);
   launch_pack<float, float>(g, e_dev, g.n, nbt.eb, nimg, s);
   const float* st32 = h->lev[h->levels - 1].st32;
-  launch_spmm<float>(g, st32, nbt.eb, nbt.aeb, nimg, nullptr, nullptr, s);
+  launch_spmm<float>(g, st32, spmm_io<float>(nbt.eb, nbt.aeb), nimg, nullptr, s);
   cudaMemsetAsync(lsum, 0, sizeof(double), s);
   net_batch_step(nbt, g, nimg, h->net_c, st32, wq, lsum, s);
   launch_net_grad_sum(nbt.parts_dev, net_batch_blocks(nbt, g, nimg), net3 ? 1 : 0, gd, s);
@@ -3067,7 +3072,7 @@ mpcg_status mg_learned_train(mg_hierarchy* const* hs, int nprob, const int* pair
   launch_pack<float, float>(g, e_dev, g.n, E, npairs, s);
   for (int i = 0; i < npairs; ++i) {
     const Level& Lp = hs[pair_prob[i]]->lev[hs[pair_prob[i]]->levels - 1];
-    launch_spmm<float>(g, Lp.st32, E + (size_t)i * L, AE + (size_t)i * L, 1, nullptr, nullptr, s);
+    launch_spmm<float>(g, Lp.st32, spmm_io<float>(E + (size_t)i * L, AE + (size_t)i * L), 1, nullptr, s);
   }
   // batches: pairs grouped by problem, shuffled within a problem and across
   // batches by a seeded 64-bit LCG (Knuth's MMIX constants)

@@ -1,8 +1,8 @@
 // Tall-skinny block kernels of the MPCG step (Section 2.2, Algorithm 1):
 //   * the Gram blocks W_j = (A P_j)^T Z against the stored window,
-//   * the A-orthogonalisation P = Z - sum_j P_j beta_j with the same
-//     recurrence for A P, fused with the new Gram matrix sym(P^T A P) and
-//     the right-hand side P^T r,
+//   * the A-orthogonalisation P = Z - sum_j P_j beta_j,
+//   * the new Gram matrix sym(P^T A P) and the right-hand side P^T r, once
+//     the block SpMM has formed A P,
 //   * the update x += P alpha, r -= A P alpha with ||r||^2.
 //
 // These kernels stream the padded arrays (pads are zero, so they take part
@@ -20,264 +20,219 @@ namespace mpcg {
 
 namespace {
 
-// W_jj[a][b] = sum_i AP_slot(jj)[a][i] Z[b][i].  Block b works on window
-// block jj = b % m and on the contiguous point chunk b / m, so that the
-// blocks running together read the same chunk of Z (L2 reuse).
-// double-word Gram: two blocks per SM (128 registers) without the software
-// pipelining of the next point's loads (which needs 24 more registers)
-constexpr bool kGramDwPrefetch = false;
+// Window Gram W_jj[a][b] = sum_i AP_slot(jj)[a][i] Z[b][i].  The cnt * C rows
+// (jj, a) are dealt out in tasks of kGramRows<T, C> rows; a warp keeps the
+// task's rows x C partial sums in registers and walks the points in chunks of
+// 32 W, so a point's Z values are loaded once per task instead of once per
+// window block and the warps of a block, which hold different tasks of the
+// same chunk, share them in L1.  The row count is set by the register file:
+// with all C rows of a block per thread the C = 9 instance spilled 568 bytes
+// at 80 registers and ran at a third of the HBM rate (1025^2, m = 5: 102 us
+// for 227 MB, now 51 us); a task holds at most 45 FP32 or 24 FP64 sums
+// (5 FP64 rows instead of 4 at C = 5: 13.0 instead of 12.8 ms per 65^2 solve;
+// 4 double-word rows instead of 5 at C = 6: 235 instead of 213 us at 129^3).
+template <typename T, int C>
+constexpr int kGramRows = sizeof(T) == 4 ? (45 / C < 6 ? 45 / C : 6)
+                                         : (kIsDw<T> ? (30 / C < 8 ? 30 / C : 8) : (24 / C < 8 ? 24 / C : 8));
+// points per lane and step: one 16-byte vector in FP32 (8 bytes from C = 10 on,
+// registers), one value in FP64 and double-word (small grids then spread over
+// more warps, and their arithmetic, not their loads, is the bound)
+template <typename T, int C>
+constexpr int kGramW = sizeof(T) == 4 ? (C < 10 ? 4 : 2) : 1;
+// steps before the lane's partial sums leave it (at most 64 points)
+template <typename T, int C>
+constexpr int kGramSteps = sizeof(T) == 4 ? 64 / kGramW<T, C> : 32;
+
+// The walkers of a task: the warps of the launch shared out over the tasks
+// present (cnt blocks in the window), at most one per chunk or partial slot.
+__device__ __forceinline__ int gram_walkers(int cnt, int C, int rows, int nwarps, int slots) {
+  const int ntask = (cnt * C + rows - 1) / rows;
+  const int w = nwarps / ntask;
+  return w < slots ? w : slots;
+}
 
 template <typename T, int C>
-__global__ void __launch_bounds__(kBlock, kIsDw<T> ? 2 : 3) k_gram_window(GridDesc g, Window<T> win, const T* __restrict__ Z,
-                                                        double* part, int nchunks, const DevState* state) {
+__global__ void __launch_bounds__(kBlock, 2) k_gram_window(GridDesc g, Window<T> win, const T* __restrict__ Z,
+                                                           double* part, int nwarps, int slots,
+                                                           const DevState* state) {
   const int pb = blockIdx.y;
   state += pb;
   if (state->done) return;
-  const int m = state->m;
-  const int jj = blockIdx.x % m, chunk = blockIdx.x / m;
-  if (jj >= state->count) return;
-  const int slot = (state->newest - jj + m) % m;
+  const int cnt = state->count;
+  if (cnt == 0) return;
+  constexpr int RB = kGramRows<T, C>, W = kGramW<T, C>, NV = RB * C;
+  const int m = state->m, newest = state->newest;
+  const int lane = threadIdx.x & 31;
+  const int wid = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int nrows = cnt * C, ntask = (nrows + RB - 1) / RB;
+  const int walkers = gram_walkers(cnt, C, RB, nwarps, slots);
+  const int task = wid % ntask, walker = wid / ntask;
+  if (walker >= walkers) return;
   const long long bo = (long long)pb * g.len + g.G;
-  const T* AP = win.AP[slot] + bo;
+  const T* row[RB];
+#pragma unroll
+  for (int k = 0; k < RB; ++k) {
+    int r = task * RB + k;
+    if (r >= nrows) r = nrows - 1;   // the last task repeats its last row (not stored)
+    const int jj = r / C;
+    row[k] = win.AP[(newest - jj + m) % m] + bo + (long long)(r - jj * C) * g.cp;
+  }
   const T* Zb = Z + bo;
-  // double-word: one point per thread and step (register pressure); the
-  // group count per chunk follows the chunking of the vector width
-  constexpr int VW = Vec<T>::W;
-  constexpr int W = kIsDw<T> ? 1 : VW;
-  const long long ngroups = g.npts / VW;
-  const long long per = (ngroups + nchunks - 1) / nchunks;
-  const long long g0 = (long long)chunk * per * (VW / W);
-  const long long g1 = (g0 + per * (VW / W)) < ngroups * (VW / W) ? g0 + per * (VW / W) : ngroups * (VW / W);
-  // the chunk count keeps every thread at <= 16 vector groups (64 points in
-  // FP32) before its partial sums enter the reduction
-  typename Acc<T>::type acc[C * C];
+  const long long steps = (g.npts + 32 * W - 1) / (32 * W);
+  double hold[rs_count(NV, 5)];
 #pragma unroll
-  for (int e = 0; e < C * C; ++e) acc[e] = Acc<T>::of(T(0));
-  auto load_point = [&](long long q, T (&z)[C][W], T (&ap)[C][W]) {
-    const long long i = q * W;
+  for (int i = 0; i < rs_count(NV, 5); ++i) hold[i] = 0.0;
+  int base = 0, nvalid = NV;
+  for (long long q = walker; q < steps;) {
+    typename Acc<T>::type acc[NV];
 #pragma unroll
-    for (int b = 0; b < C; ++b) VecN<T, W>::load_keep(Zb + (long long)b * g.cp + i, z[b]);
+    for (int e = 0; e < NV; ++e) acc[e] = Acc<T>::of(T(0));
+    for (int n = 0; n < kGramSteps<T, C> && q < steps; ++n, q += walkers) {
+      const long long i = (q * 32 + lane) * W;
+      if (i >= g.npts) continue;
+      T z[C][W];
 #pragma unroll
-    for (int a = 0; a < C; ++a) VecN<T, W>::load(AP + (long long)a * g.cp + i, ap[a]);
-  };
-  auto accumulate = [&](const T (&z)[C][W], const T (&ap)[C][W]) {
+      for (int b = 0; b < C; ++b) VecN<T, W>::load_keep(Zb + (long long)b * g.cp + i, z[b]);
+      T ap[RB][W];
 #pragma unroll
-    for (int a = 0; a < C; ++a)
+      for (int k = 0; k < RB; ++k) VecN<T, W>::load(row[k] + i, ap[k]);
 #pragma unroll
-      for (int b = 0; b < C; ++b)
+      for (int k = 0; k < RB; ++k)
 #pragma unroll
-        for (int w = 0; w < W; ++w) mac(acc[a * C + b], ap[a][w], z[b][w]);
-  };
-  if constexpr (kIsDw<T> && kGramDwPrefetch) {
-    // the next point's loads are issued before the current point's products
-    // (software pipelining)
-    long long q = g0 + threadIdx.x;
-    T z[C][W], ap[C][W];
-    if (q < g1) load_point(q, z, ap);
-    while (q < g1) {
-      const long long qn = q + blockDim.x;
-      T zn[C][W], apn[C][W];
-      if (qn < g1) load_point(qn, zn, apn);
-      accumulate(z, ap);
+        for (int b = 0; b < C; ++b)
 #pragma unroll
-      for (int b = 0; b < C; ++b)
-#pragma unroll
-        for (int w = 0; w < W; ++w) {
-          z[b][w] = zn[b][w];
-          ap[b][w] = apn[b][w];
-        }
-      q = qn;
+          for (int w = 0; w < W; ++w) mac(acc[k * C + b], ap[k][w], z[b][w]);
     }
-  } else {
-    for (long long q = g0 + threadIdx.x; q < g1; q += blockDim.x) {
-      T z[C][W], ap[C][W];
-      load_point(q, z, ap);
-      accumulate(z, ap);
-    }
+    // the warp's sums in T, above the warp in FP64
+    T v[NV];
+#pragma unroll
+    for (int e = 0; e < NV; ++e) v[e] = Acc<T>::value(acc[e]);
+    warp_reduce_scatter<T, NV>(v, base, nvalid, lane);
+#pragma unroll
+    for (int i = 0; i < rs_count(NV, 5); ++i) hold[i] += (double)v[i];
   }
-  T fin[C * C];
+  double* pj = part + (long long)pb * m * C * C * slots;
 #pragma unroll
-  for (int e = 0; e < C * C; ++e) fin[e] = Acc<T>::value(acc[e]);
-  double* pj = part + ((long long)pb * m + jj) * C * C * nchunks;
-  block_sum_store<T, C * C>(fin, pj, nchunks, chunk);
-}
-
-// Gram partials of one point group: G = sym(P^T A P) (upper triangle,
-// p_a ap_b + p_b ap_a) and g = P^T r.
-template <typename T, int C, int W>
-__device__ __forceinline__ void gram_point(const T (&p)[C][W], const T (&ap)[C][W], const T* rp,
-                                           typename Acc<T>::type (&acc)[C * (C + 1) / 2 + C]) {
-  constexpr int NG = C * (C + 1) / 2;
-  T rv[W];
-  VecN<T, W>::load(rp, rv);
-  int k = 0;
-#pragma unroll
-  for (int a = 0; a < C; ++a) {
-#pragma unroll
-    for (int b = a; b < C; ++b) {
-#pragma unroll
-      for (int w = 0; w < W; ++w) {
-        mac(acc[k], p[a][w], ap[b][w]);
-        mac(acc[k], p[b][w], ap[a][w]);
-      }
-      ++k;
-    }
-#pragma unroll
-    for (int w = 0; w < W; ++w) mac(acc[NG + a], p[a][w], rv[w]);
+  for (int i = 0; i < rs_count(NV, 5); ++i) {
+    const int e = task * NV + base + i;   // = (jj C + a) C + b
+    if (i < nvalid && e < nrows * C) pj[(long long)e * slots + walker] = hold[i];
   }
 }
 
-// In double-word arithmetic the Gram partials of the new block go to a
-// second kernel (k_orth_gram_dw): without their 27 double-word accumulators
-// the orthogonalisation fits 128 registers and two blocks per SM.
+// P = Z - sum_j P_j beta_j into the next ring slot.  A P of the new block is
+// the block SpMM of P itself (not the recurrence A Z - sum_j A P_j beta_j):
+// this kernel then reads the window's P_j only and no A Z exists, (m + 2) C
+// words a point at a full window instead of (2 m + 4) C + 1 (129^3, FP32,
+// C = 6, four blocks in the window: 102 -> 43 us; 1025^2, C = 9, m = 5: 133 ->
+// 49 us).
+// Bound by HBM in FP32, by the FP64 and FP32 pipes in FP64 and double-word.
 template <typename T, int C>
-__global__ void __launch_bounds__(kBlock, 2) k_orth_update(GridDesc g, Window<T> win, const T* __restrict__ Z,
-                                                        const T* __restrict__ AZ, const T* __restrict__ r,
-                                                        double* part, const DevState* state) {
+__global__ void __launch_bounds__(kBlock) k_orth_update(GridDesc g, Window<T> win, const T* __restrict__ Z,
+                                                        const DevState* state) {
   const int pb = blockIdx.y;
   state += pb;
   if (state->done) return;
   const int cnt = state->count, m = state->m, newest = state->newest;
-  const int ns = (newest + 1) % m;
   const long long bo = (long long)pb * g.len + g.G;
-  __shared__ T beta[kMaxWindow][C][C];
+  constexpr int CP = sizeof(T) == 4 ? (C + 3) / 4 * 4 : (C + 1) / 2 * 2;   // rows start on 16 bytes
+  __shared__ __align__(16) T nbeta[kMaxWindow][C][CP];                      // -beta
   __shared__ const T* pp[kMaxWindow];
-  __shared__ const T* app[kMaxWindow];
   for (int e = threadIdx.x; e < cnt * C * C; e += blockDim.x) {
     const int jj = e / (C * C), a = (e / C) % C, b = e % C;
-    beta[jj][a][b] = (T)state->beta[jj][a][b];
+    nbeta[jj][a][b] = -(T)state->beta[jj][a][b];
   }
-  for (int jj = threadIdx.x; jj < cnt; jj += blockDim.x) {
-    const int slot = (newest - jj + m) % m;
-    pp[jj] = win.P[slot] + bo;
-    app[jj] = win.AP[slot] + bo;
-  }
+  for (int jj = threadIdx.x; jj < cnt; jj += blockDim.x) pp[jj] = win.P[(newest - jj + m) % m] + bo;
   __syncthreads();
-  T* Pn = win.P[ns] + bo;
-  T* APn = win.AP[ns] + bo;
+  T* Pn = win.P[(newest + 1) % m] + bo;
   const T* Zb = Z + bo;
-  const T* AZb = AZ + bo;
-  const T* rb = r + bo;
-  constexpr int W = kIsDw<T> ? 1 : Vec<T>::W;   // double-word: one point per thread (registers)
-  constexpr bool kParts = !kIsDw<T>;             // Gram partials here, or in k_orth_gram_dw
-  constexpr int NG = C * (C + 1) / 2;
+  constexpr int W = sizeof(T) == 4 ? (C < 10 ? 4 : 2) : 1;
   using A = typename Acc<T>::type;
-  A acc[kParts ? NG + C : 1];
-#pragma unroll
-  for (int i = 0; i < (kParts ? NG + C : 1); ++i) acc[i] = Acc<T>::of(T(0));
   const long long ngroups = g.npts / W;
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < ngroups;
        q += (long long)gridDim.x * blockDim.x) {
     const long long i = q * W;
-    A pacc[C][W], apacc[C][W];
+    A pacc[C][W];
 #pragma unroll
     for (int b = 0; b < C; ++b) {
-      T zv[W], azv[W];
+      T zv[W];
       VecN<T, W>::load(Zb + (long long)b * g.cp + i, zv);
-      VecN<T, W>::load(AZb + (long long)b * g.cp + i, azv);
 #pragma unroll
-      for (int w = 0; w < W; ++w) {
-        pacc[b][w] = Acc<T>::of(zv[w]);
-        apacc[b][w] = Acc<T>::of(azv[w]);
-      }
+      for (int w = 0; w < W; ++w) pacc[b][w] = Acc<T>::of(zv[w]);
     }
-    auto load_block = [&](int jj, T (&pa)[C][W], T (&apa)[C][W]) {
+    for (int jj = 0; jj < cnt; ++jj) {
+      const T* pj = pp[jj] + i;
+      T pa[C][W];
 #pragma unroll
-      for (int a = 0; a < C; ++a) {
-        VecN<T, W>::load(pp[jj] + (long long)a * g.cp + i, pa[a]);
-        VecN<T, W>::load(app[jj] + (long long)a * g.cp + i, apa[a]);
-      }
-    };
-    auto apply_block = [&](int jj, const T (&pa)[C][W], const T (&apa)[C][W]) {
+      for (int a = 0; a < C; ++a) VecN<T, W>::load(pj + (long long)a * g.cp, pa[a]);
 #pragma unroll
       for (int a = 0; a < C; ++a)
 #pragma unroll
         for (int b = 0; b < C; ++b) {
-          const T bt = beta[jj][a][b];
+          const T bt = nbeta[jj][a][b];
 #pragma unroll
-          for (int w = 0; w < W; ++w) {
-            mac(pacc[b][w], -pa[a][w], bt);
-            mac(apacc[b][w], -apa[a][w], bt);
-          }
+          for (int w = 0; w < W; ++w) mac(pacc[b][w], pa[a][w], bt);
         }
-    };
-    if constexpr (kIsDw<T>) {
-      // few warps per SM in double-word: block jj + 1 is loaded while
-      // block jj's products run (software pipelining)
-      T pa[C][W], apa[C][W];
-      if (cnt > 0) load_block(0, pa, apa);
-      for (int jj = 0; jj < cnt; ++jj) {
-        T pn[C][W], apn[C][W];
-        if (jj + 1 < cnt) load_block(jj + 1, pn, apn);
-        apply_block(jj, pa, apa);
-#pragma unroll
-        for (int a = 0; a < C; ++a)
-#pragma unroll
-          for (int w = 0; w < W; ++w) {
-            pa[a][w] = pn[a][w];
-            apa[a][w] = apn[a][w];
-          }
-      }
-    } else {
-      for (int jj = 0; jj < cnt; ++jj) {
-        T pa[C][W], apa[C][W];
-        load_block(jj, pa, apa);
-        apply_block(jj, pa, apa);
-      }
     }
-    T p[C][W], ap[C][W];
 #pragma unroll
-    for (int b = 0; b < C; ++b)
+    for (int b = 0; b < C; ++b) {
+      T p[W];
 #pragma unroll
-      for (int w = 0; w < W; ++w) {
-        p[b][w] = Acc<T>::value(pacc[b][w]);
-        ap[b][w] = Acc<T>::value(apacc[b][w]);
-      }
-#pragma unroll
-    for (int a = 0; a < C; ++a) {
-      VecN<T, W>::store(Pn + (long long)a * g.cp + i, p[a]);
-      VecN<T, W>::store(APn + (long long)a * g.cp + i, ap[a]);
+      for (int w = 0; w < W; ++w) p[w] = Acc<T>::value(pacc[b][w]);
+      VecN<T, W>::store(Pn + (long long)b * g.cp + i, p);
     }
-    if constexpr (kParts) gram_point<T, C, W>(p, ap, rb + i, acc);
-  }
-  if constexpr (kParts) {
-    T fin[NG + C];
-#pragma unroll
-    for (int i = 0; i < NG + C; ++i) fin[i] = Acc<T>::value(acc[i]);
-    block_sum_store<T, NG + C>(fin, part + (long long)pb * (NG + C) * gridDim.x, gridDim.x, blockIdx.x);
   }
 }
 
-// The Gram partials of the new block, double-word: the same points per
-// thread and the same order as the fused FP32 / FP64 kernels (same grid).
-template <int C>
-__global__ void __launch_bounds__(kBlock, 2) k_orth_gram_dw(GridDesc g, Window<dw> win, const dw* __restrict__ r,
-                                                             double* part, const DevState* state) {
+// Gram partials of the new block: the upper triangle of G = P^T A P and
+// g = P^T r.  A P is the product of A with the very P read here, so p_a^T A p_b
+// and p_b^T A p_a differ by the rounding of one product and one of them serves
+// for both (the recurrence A Z - sum_j A P_j beta_j drifts from A P and had to
+// be symmetrised): 27 instead of 48 multiply-adds a point at C = 6, which the
+// FP64 pipe pays for in full (97^3, FP64: 65.5 -> 38 us).
+template <typename T, int C>
+__global__ void __launch_bounds__(kBlock, (sizeof(T) == 4 || C <= 7) ? 2 : 1)
+    k_block_gram(GridDesc g, Window<T> win, const T* __restrict__ r, double* part, const DevState* state) {
   const int pb = blockIdx.y;
   state += pb;
   if (state->done) return;
   const int ns = (state->newest + 1) % state->m;
   const long long bo = (long long)pb * g.len + g.G;
-  const dw* Pn = win.P[ns] + bo;
-  const dw* APn = win.AP[ns] + bo;
+  const T* Pn = win.P[ns] + bo;
+  const T* APn = win.AP[ns] + bo;
+  const T* rb = r + bo;
+  constexpr int W = sizeof(T) == 4 ? (C <= 7 ? 4 : (C <= 9 ? 2 : 1)) : 1;
   constexpr int NG = C * (C + 1) / 2;
-  dwacc acc[NG + C];
+  typename Acc<T>::type acc[NG + C];
 #pragma unroll
-  for (int i = 0; i < NG + C; ++i) acc[i] = dwacc_of(dw(0));
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < g.npts;
+  for (int i = 0; i < NG + C; ++i) acc[i] = Acc<T>::of(T(0));
+  const long long ngroups = g.npts / W;
+  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < ngroups;
        q += (long long)gridDim.x * blockDim.x) {
-    dw p[C][1], ap[C][1];
+    const long long i = q * W;
+    T p[C][W], ap[C][W], rv[W];
+    VecN<T, W>::load_keep(rb + i, rv);
 #pragma unroll
     for (int a = 0; a < C; ++a) {
-      VecN<dw, 1>::load(Pn + (long long)a * g.cp + q, p[a]);
-      VecN<dw, 1>::load(APn + (long long)a * g.cp + q, ap[a]);
+      VecN<T, W>::load_keep(Pn + (long long)a * g.cp + i, p[a]);
+      VecN<T, W>::load_keep(APn + (long long)a * g.cp + i, ap[a]);
     }
-    gram_point<dw, C, 1>(p, ap, r + bo + q, acc);
-  }
-  dw fin[NG + C];
+    int k = 0;
 #pragma unroll
-  for (int i = 0; i < NG + C; ++i) fin[i] = dwacc_value(acc[i]);
-  block_sum_store<dw, NG + C>(fin, part + (long long)pb * (NG + C) * gridDim.x, gridDim.x, blockIdx.x);
+    for (int a = 0; a < C; ++a) {
+#pragma unroll
+      for (int b = a; b < C; ++b) {
+#pragma unroll
+        for (int w = 0; w < W; ++w) mac(acc[k], p[a][w], ap[b][w]);
+        ++k;
+      }
+#pragma unroll
+      for (int w = 0; w < W; ++w) mac(acc[NG + a], p[a][w], rv[w]);
+    }
+  }
+  T fin[NG + C];
+#pragma unroll
+  for (int i = 0; i < NG + C; ++i) fin[i] = Acc<T>::value(acc[i]);
+  block_sum_store<T, NG + C>(fin, part + (long long)pb * (NG + C) * gridDim.x, gridDim.x, blockIdx.x);
 }
 
 template <typename T, int C>
@@ -407,17 +362,31 @@ __global__ void __launch_bounds__(kBlock) k_axpy_mixed(GridDesc g, double* __res
     default: break;                                                                              \
   }
 
-int gram_chunks_default(const GridDesc& g) {
-  // 8 vector groups (32 points in FP32, 16 in FP64) per thread and chunk
-  const long long groups = g.npts / 4;
-  long long c = (groups + kBlock * 8 - 1) / (kBlock * 8);
-  if (c < 1) c = 1;
-  return (int)(c < kGramChunksMax ? c : kGramChunksMax);
+// Threads per block for `items` elementwise work items: 256, or as few as a
+// warp where 256 would leave SMs without a block.  The FP64 pipe takes a warp
+// instruction every 64 cycles, so a small FP64 grid has to be spread over all
+// SMs: at 65^2 points, C = 5, 8 blocks of 256 became 65 or more of 32, and the
+// window Gram went from 34.8 to 9.7 us, the orthogonalisation from 45 to 12 us,
+// the block SpMM from 14.3 to 8.1 us (serialised, event-timed launches).
+int spread_threads(long long items) {
+  const int sms = sm_count() > 0 ? sm_count() : 152;
+  int t = kBlock;
+  while (t > 32 && (items + t - 1) / t < sms) t /= 2;
+  return t;
 }
-// at most 16 vector groups (64 FP32 points) per thread and chunk
+
+// of the reducing kernels: the same for a problem alone and in a batch
+int stream_threads(const GridDesc& g) { return spread_threads(g.npts / 2); }
+
+// Slots of the window Gram's partial sums, the most warps that share a task's
+// points (gram_shape): one per 32 points, at most four per SM.
+int gram_chunks_default(const GridDesc& g) {
+  const long long c = (g.npts + 31) / 32;
+  return (int)(c < 2 * kStreamBlocks ? c : 2 * kStreamBlocks);
+}
 int gram_chunks_min(const GridDesc& g) { return (gram_chunks_default(g) + 1) / 2; }
 int gram_chunks_cap(const GridDesc& g) {
-  const long long c = 4LL * gram_chunks_default(g);
+  const long long c = 2LL * gram_chunks_default(g);
   return (int)(c < kGramChunksMax ? c : kGramChunksMax);
 }
 int gram_chunks(const GridDesc& g) {
@@ -427,15 +396,15 @@ int gram_chunks(const GridDesc& g) {
 }
 
 int stream_blocks_min(const GridDesc& g) {
-  const long long groups = g.npts / 2;
-  long long need = (groups + kBlock * 16 - 1) / (kBlock * 16);   // <= 64 points per thread
+  const long long groups = g.npts / 2, bd = stream_threads(g);
+  long long need = (groups + bd * 16 - 1) / (bd * 16);   // <= 64 points per thread
   if (need < 1) need = 1;
   return (int)(need < kStreamBlocksMax ? need : kStreamBlocksMax);
 }
 int stream_blocks_default(const GridDesc& g) {
-  const long long groups = g.npts / 2;
+  const long long groups = g.npts / 2, bd = stream_threads(g);
   long long need = stream_blocks_min(g);
-  long long fill = (groups + kBlock - 1) / kBlock;                // no idle threads
+  long long fill = (groups + bd - 1) / bd;                // no idle threads
   long long nb = kStreamBlocks < fill ? kStreamBlocks : fill;
   if (need > nb) nb = need;
   if (nb < 1) nb = 1;
@@ -444,8 +413,8 @@ int stream_blocks_default(const GridDesc& g) {
 // the most blocks the tuner may choose (and the reduction buffers reserve):
 // eight per SM, without idle threads
 int stream_blocks_cap(const GridDesc& g) {
-  const long long groups = g.npts / 2;
-  const long long fill = (groups + kBlock - 1) / kBlock;
+  const long long groups = g.npts / 2, bd = stream_threads(g);
+  const long long fill = (groups + bd - 1) / bd;
   long long c = 8LL * (sm_count() > 0 ? sm_count() : 152);
   if (c > fill) c = fill;
   const long long d = stream_blocks_default(g);
@@ -458,59 +427,113 @@ int stream_blocks(const GridDesc& g) {
   return v < lo ? lo : (v > hi ? hi : v);
 }
 
+// Partial slots per value, the most walkers of a task: a warp's set-up and
+// its final reduction cost about two steps, so walkers take two or four steps
+// each once the grid has enough of them (a batch of 12 problems of 257^2
+// points, C = 7: 70 us with one or two steps, 41 us with four); the slow FP64
+// and double-word steps are shared out more finely.  The shape depends on the
+// grid alone: a problem sums alike on its own and in a batch.
+template <typename T>
+int gram_slots(const GridDesc& g) {
+  const int w = sizeof(T) == 4 ? 4 : 1;
+  const long long steps = (g.npts + 32 * w - 1) / (32 * w);
+  const int per = sizeof(T) == 4 ? (steps >= 512 ? 4 : (steps >= 128 ? 2 : 1))
+                                 : (steps >= 2048 ? 4 : (steps >= 512 ? 2 : 1));
+  const long long n = (steps + per - 1) / per;
+  const int v = gram_chunks(g);
+  return (int)(n < v ? n : v);
+}
+template int gram_slots<float>(const GridDesc&);
+template int gram_slots<double>(const GridDesc&);
+template int gram_slots<dw>(const GridDesc&);
+
+template <typename T, int C>
+static GramShape gram_shape_c(const GridDesc& g, int m) {
+  constexpr int RB = kGramRows<T, C>;
+  GramShape s;
+  s.rows = RB;
+  s.slots = gram_slots<T>(g);
+  const int ntask = (m * C + RB - 1) / RB;
+  const long long full = (long long)ntask * s.slots;
+  const int cap = 16 * (sm_count() > 0 ? sm_count() : 152);   // two blocks of eight warps per SM
+  s.nwarps = (int)(full < cap ? full : (cap > ntask ? cap : ntask));
+  return s;
+}
+
+template <typename T>
+GramShape gram_shape(const GridDesc& g, int C, int m) {
+  GramShape s = {};
+  MPCG_C_SWITCH(C, (s = gram_shape_c<T, CC>(g, m)));
+  return s;
+}
+template GramShape gram_shape<float>(const GridDesc&, int, int);
+template GramShape gram_shape<double>(const GridDesc&, int, int);
+template GramShape gram_shape<dw>(const GridDesc&, int, int);
+
 template <typename T>
 void launch_gram_window(const GridDesc& g, Window<T> win, const T* Z, int C, int m, double* part,
                         const DevState* state, cudaStream_t s) {
-  const int nch = gram_chunks(g);
-  MPCG_C_SWITCH(C, (k_gram_window<T, CC><<<dim3(nch * m, g.nb), kBlock, 0, s>>>(g, win, Z, part, nch, state)));
+  const GramShape q = gram_shape<T>(g, C, m);
+  const int threads = spread_threads(32LL * q.nwarps);
+  const int blocks = (32 * q.nwarps + threads - 1) / threads;
+  MPCG_C_SWITCH(C, (k_gram_window<T, CC><<<dim3(blocks, g.nb), threads, 0, s>>>(g, win, Z, part, q.nwarps, q.slots,
+                                                                                state)));
 }
 
 template <typename T>
-void launch_orth_update(const GridDesc& g, Window<T> win, const T* Z, const T* AZ, const T* r, int C, double* part,
-                        const DevState* state, cudaStream_t s) {
-  const int nb = stream_blocks(g);
-  MPCG_C_SWITCH(C, (k_orth_update<T, CC><<<dim3(nb, g.nb), kBlock, 0, s>>>(g, win, Z, AZ, r, part, state)));
+void launch_orth_update(const GridDesc& g, Window<T> win, const T* Z, int C, const DevState* state,
+                        cudaStream_t s) {
+  const int w = sizeof(T) == 4 ? (C < 10 ? 4 : 2) : 1;
+  const long long groups = g.npts / w;
+  const int threads = spread_threads(groups * g.nb);   // elementwise: any shape gives the same values
+  const long long need = (groups + threads - 1) / threads;
+  const int nb = (int)(need < 2 * kStreamBlocks ? need : 2 * kStreamBlocks);
+  MPCG_C_SWITCH(C, (k_orth_update<T, CC><<<dim3(nb, g.nb), threads, 0, s>>>(g, win, Z, state)));
 }
 
-void launch_orth_gram_dw(const GridDesc& g, Window<dw> win, const dw* r, int C, double* part, const DevState* state,
-                         cudaStream_t s) {
+template <typename T>
+void launch_block_gram(const GridDesc& g, Window<T> win, const T* r, int C, double* part, const DevState* state,
+                       cudaStream_t s) {
   const int nb = stream_blocks(g);
-  MPCG_C_SWITCH(C, (k_orth_gram_dw<CC><<<dim3(nb, g.nb), kBlock, 0, s>>>(g, win, r, part, state)));
+  MPCG_C_SWITCH(C, (k_block_gram<T, CC><<<dim3(nb, g.nb), stream_threads(g), 0, s>>>(g, win, r, part, state)));
 }
 
 template <typename T>
 void launch_update_xr(const GridDesc& g, Window<T> win, T* x, T* r, int C, double* part, const DevState* state,
                       cudaStream_t s) {
   const int nb = stream_blocks(g);
-  MPCG_C_SWITCH(C, (k_update_xr<T, CC><<<dim3(nb, g.nb), kBlock, 0, s>>>(g, win, x, r, part, state)));
+  MPCG_C_SWITCH(C, (k_update_xr<T, CC><<<dim3(nb, g.nb), stream_threads(g), 0, s>>>(g, win, x, r, part, state)));
 }
 
 void launch_start_inner(const GridDesc& g, const double* r64, const double* nrm2, const int* active, float* b32,
                         float* r32, double* part, cudaStream_t s) {
-  k_start_inner<<<dim3(stream_blocks(g), g.nb), kBlock, 0, s>>>(g, r64, nrm2, active, b32, r32, part);
+  k_start_inner<<<dim3(stream_blocks(g), g.nb), stream_threads(g), 0, s>>>(g, r64, nrm2, active, b32, r32, part);
 }
 void launch_axpy_mixed(const GridDesc& g, double* x, const float* d, const double* scale, int* xnz,
                        cudaStream_t s) {
-  k_axpy_mixed<<<dim3(stream_blocks(g), g.nb), kBlock, 0, s>>>(g, x, d, scale, xnz);
+  k_axpy_mixed<<<dim3(stream_blocks(g), g.nb), stream_threads(g), 0, s>>>(g, x, d, scale, xnz);
 }
 
-template void launch_gram_window<double>(const GridDesc&, Window<double>, const double*, int, int, double*,
-                                         const DevState*, cudaStream_t);
-template void launch_gram_window<float>(const GridDesc&, Window<float>, const float*, int, int, double*,
-                                        const DevState*, cudaStream_t);
-template void launch_orth_update<double>(const GridDesc&, Window<double>, const double*, const double*,
-                                         const double*, int, double*, const DevState*, cudaStream_t);
-template void launch_orth_update<float>(const GridDesc&, Window<float>, const float*, const float*, const float*,
-                                        int, double*, const DevState*, cudaStream_t);
-template void launch_update_xr<double>(const GridDesc&, Window<double>, double*, double*, int, double*,
-                                       const DevState*, cudaStream_t);
-template void launch_update_xr<float>(const GridDesc&, Window<float>, float*, float*, int, double*,
-                                      const DevState*, cudaStream_t);
+template void launch_gram_window<double>(const GridDesc&, Window<double>, const double*, int, int, double*, const DevState*,
+                                         cudaStream_t);
+template void launch_orth_update<double>(const GridDesc&, Window<double>, const double*, int, const DevState*, cudaStream_t);
+template void launch_block_gram<double>(const GridDesc&, Window<double>, const double*, int, double*, const DevState*,
+                                        cudaStream_t);
+template void launch_update_xr<double>(const GridDesc&, Window<double>, double*, double*, int, double*, const DevState*,
+                                       cudaStream_t);
+template void launch_gram_window<float>(const GridDesc&, Window<float>, const float*, int, int, double*, const DevState*,
+                                         cudaStream_t);
+template void launch_orth_update<float>(const GridDesc&, Window<float>, const float*, int, const DevState*, cudaStream_t);
+template void launch_block_gram<float>(const GridDesc&, Window<float>, const float*, int, double*, const DevState*,
+                                        cudaStream_t);
+template void launch_update_xr<float>(const GridDesc&, Window<float>, float*, float*, int, double*, const DevState*,
+                                       cudaStream_t);
 template void launch_gram_window<dw>(const GridDesc&, Window<dw>, const dw*, int, int, double*, const DevState*,
-                                     cudaStream_t);
-template void launch_orth_update<dw>(const GridDesc&, Window<dw>, const dw*, const dw*, const dw*, int, double*,
-                                     const DevState*, cudaStream_t);
+                                         cudaStream_t);
+template void launch_orth_update<dw>(const GridDesc&, Window<dw>, const dw*, int, const DevState*, cudaStream_t);
+template void launch_block_gram<dw>(const GridDesc&, Window<dw>, const dw*, int, double*, const DevState*,
+                                        cudaStream_t);
 template void launch_update_xr<dw>(const GridDesc&, Window<dw>, dw*, dw*, int, double*, const DevState*,
-                                   cudaStream_t);
+                                       cudaStream_t);
 
 }  // namespace mpcg

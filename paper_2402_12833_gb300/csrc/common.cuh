@@ -213,6 +213,7 @@ struct DevState {
   double rnorm;
   double delta;
   double tau;
+  double zpz[kMaxCols];   // z_b^T A z_b less p_b^T A p_b of the new block: sum_j (W_j^T beta_j)_bb
   double alpha[kMaxCols];
   double beta[kMaxWindow][kMaxCols][kMaxCols];
   double gpinv[kMaxWindow][kMaxCols][kMaxCols];
@@ -223,5 +224,46 @@ struct Window {
   T* P[kMaxWindow];
   T* AP[kMaxWindow];
 };
+
+// Operands of a block SpMM Y = A X: two arrays, or the block being built in
+// the ring (X = P and Y = A P of the slot after the newest, per problem).
+template <typename T>
+struct SpmmIO {
+  const T* X;
+  T* Y;
+  Window<T> win;
+  bool ring;
+};
+template <typename T>
+inline SpmmIO<T> spmm_io(const T* X, T* Y) {
+  SpmmIO<T> io = {};
+  io.X = X;
+  io.Y = Y;
+  return io;
+}
+// offset: added to both ring arrays (the ELL kernels take pointers at G)
+template <typename T>
+inline SpmmIO<T> spmm_ring(const Window<T>& win, int m, long long offset = 0) {
+  SpmmIO<T> io = {};
+  io.win = win;
+  for (int j = 0; j < m; ++j) {
+    io.win.P[j] += offset;
+    io.win.AP[j] += offset;
+  }
+  io.ring = true;
+  return io;
+}
+#ifdef __CUDACC__
+template <typename T>
+__device__ __forceinline__ void spmm_operands(const SpmmIO<T>& io, const DevState* st, const T*& X, T*& Y) {
+  X = io.X;
+  Y = io.Y;
+  if (io.ring) {
+    const int ns = (st->newest + 1) % st->m;
+    X = io.win.P[ns];
+    Y = io.win.AP[ns];
+  }
+}
+#endif
 
 }  // namespace mpcg

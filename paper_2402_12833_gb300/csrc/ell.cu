@@ -1,6 +1,5 @@
 // Operators of an algebraic hierarchy (sliced ELLPACK, EllDev in
-// common.cuh): the block SpMM A Z of the Section 2.2 update with the
-// z_i^T A z_i partials, the residual, damped Jacobi on every grid (Eq. 2,
+// common.cuh): the block SpMM A P of the Section 2.2 update, the residual, damped Jacobi on every grid (Eq. 2,
 // c_0 = 0) and the transfers R_j = P_j^T (restriction) and P_j
 // (prolongation) of Section 2.1.  Vectors are flat padded arrays (unknown i
 // at G + i); every launcher takes pointers already offset by G.
@@ -30,16 +29,14 @@ __device__ __forceinline__ T group_sum(T v, int lg) {
 }
 
 // Y[:, c] = A X[:, c] (ADD: Y[:, c] += A X[:, c]) for C columns (column
-// pitches ldx, ldy); with ZAZ the per-block partials of X[:, c]^T Y[:, c]
-// (value-major, stride gridDim.x).
-template <typename T, int C, bool ZAZ, bool ADD = false>
-__global__ void __launch_bounds__(kBlock) k_ell_spmm(EllDev<T> A, const T* __restrict__ X, long long ldx,
-                                                     T* __restrict__ Y, long long ldy, double* zaz,
+// pitches ldx, ldy).
+template <typename T, int C, bool ADD = false>
+__global__ void __launch_bounds__(kBlock) k_ell_spmm(EllDev<T> A, SpmmIO<T> io, long long ldx, long long ldy,
                                                      const DevState* state) {
   if (state && state[0].done) return;
-  T zacc[ZAZ ? C : 1];
-#pragma unroll
-  for (int c = 0; c < (ZAZ ? C : 1); ++c) zacc[c] = 0;
+  const T* X;
+  T* Y;
+  spmm_operands(io, state, X, Y);
   const long long nt = (long long)A.nslices * 32;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < nt; t += (long long)gridDim.x * blockDim.x) {
     const int s = (int)(t >> 5), lane = (int)(t & 31);
@@ -64,11 +61,9 @@ __global__ void __launch_bounds__(kBlock) k_ell_spmm(EllDev<T> A, const T* __res
       for (int c = 0; c < C; ++c) {
         if (ADD) Y[c * ldy + r] += acc[c];
         else Y[c * ldy + r] = acc[c];
-        if (ZAZ) zacc[c] = fma(X[c * ldx + r], acc[c], zacc[c]);
       }
     }
   }
-  if (ZAZ) block_sum_store<T, ZAZ ? C : 1>(zacc, zaz, gridDim.x, blockIdx.x);
 }
 
 // r = b - A x with the partials of |r|^2 and |b|^2 (NORMS; without them it
@@ -147,13 +142,12 @@ int ell_threads_blocks(const EllDev<T>& A) {
 }  // namespace
 
 template <typename T>
-void launch_ell_spmm(const EllDev<T>& A, const T* X, long long ldx, T* Y, long long ldy, int C, double* zaz,
-                     int nblocks, const DevState* state, cudaStream_t s) {
-  const int grid = nblocks > 0 ? nblocks : ell_threads_blocks(A);
+void launch_ell_spmm(const EllDev<T>& A, const SpmmIO<T>& io, long long ldx, long long ldy, int C,
+                     const DevState* state, cudaStream_t s) {
+  const int grid = ell_threads_blocks(A);
 #define MPCG_ELL_CASE(CC)                                                                                \
   case CC:                                                                                               \
-    if (zaz) k_ell_spmm<T, CC, true><<<grid, kBlock, 0, s>>>(A, X, ldx, Y, ldy, zaz, state);             \
-    else k_ell_spmm<T, CC, false><<<grid, kBlock, 0, s>>>(A, X, ldx, Y, ldy, zaz, state);                \
+    k_ell_spmm<T, CC><<<grid, kBlock, 0, s>>>(A, io, ldx, ldy, state);                                   \
     break;
   switch (C) {
     MPCG_ELL_CASE(1) MPCG_ELL_CASE(2) MPCG_ELL_CASE(3) MPCG_ELL_CASE(4) MPCG_ELL_CASE(5) MPCG_ELL_CASE(6)
@@ -162,15 +156,17 @@ void launch_ell_spmm(const EllDev<T>& A, const T* X, long long ldx, T* Y, long l
   }
 #undef MPCG_ELL_CASE
 }
-template void launch_ell_spmm<double>(const EllDev<double>&, const double*, long long, double*, long long, int,
-                                      double*, int, const DevState*, cudaStream_t);
-template void launch_ell_spmm<float>(const EllDev<float>&, const float*, long long, float*, long long, int, double*,
-                                     int, const DevState*, cudaStream_t);
+template void launch_ell_spmm<double>(const EllDev<double>&, const SpmmIO<double>&, long long, long long, int,
+                                      const DevState*, cudaStream_t);
+template void launch_ell_spmm<float>(const EllDev<float>&, const SpmmIO<float>&, long long, long long, int,
+                                     const DevState*, cudaStream_t);
+template void launch_ell_spmm<dw>(const EllDev<dw>&, const SpmmIO<dw>&, long long, long long, int, const DevState*,
+                                  cudaStream_t);
 
 template <typename T>
-void launch_ell_residual(const EllDev<T>& A, const T* b, const T* x, T* r, double* part, int nblocks, cudaStream_t s,
-                         const int* xnz) {
-  k_ell_residual<T><<<nblocks, kBlock, 0, s>>>(A, b, x, r, part, xnz);
+void launch_ell_residual(const EllDev<T>& A, const T* b, const T* x, T* r, double* part, int nblocks, int threads,
+                         cudaStream_t s, const int* xnz) {
+  k_ell_residual<T><<<nblocks, threads, 0, s>>>(A, b, x, r, part, xnz);
 }
 
 template <typename T>
@@ -185,14 +181,14 @@ template void launch_ell_defect<float>(const EllDev<float>&, const float*, const
 
 template <typename T>
 void launch_ell_spmv_add(const EllDev<T>& A, const T* X, T* Y, const DevState* state, cudaStream_t s) {
-  k_ell_spmm<T, 1, false, true><<<ell_threads_blocks(A), kBlock, 0, s>>>(A, X, 0, Y, 0, nullptr, state);
+  k_ell_spmm<T, 1, true><<<ell_threads_blocks(A), kBlock, 0, s>>>(A, spmm_io(X, Y), 0, 0, state);
 }
 template void launch_ell_spmv_add<double>(const EllDev<double>&, const double*, double*, const DevState*,
                                           cudaStream_t);
 template void launch_ell_spmv_add<float>(const EllDev<float>&, const float*, float*, const DevState*, cudaStream_t);
-template void launch_ell_residual<double>(const EllDev<double>&, const double*, const double*, double*, double*, int,
+template void launch_ell_residual<double>(const EllDev<double>&, const double*, const double*, double*, double*, int, int,
                                           cudaStream_t, const int*);
-template void launch_ell_residual<float>(const EllDev<float>&, const float*, const float*, float*, double*, int,
+template void launch_ell_residual<float>(const EllDev<float>&, const float*, const float*, float*, double*, int, int,
                                          cudaStream_t, const int*);
 
 template <typename T>
@@ -206,11 +202,9 @@ template void launch_ell_jacobi<float>(const EllDev<float>&, const float*, const
                                        const DevState*, cudaStream_t);
 
 // double-word instances (MPCG_FP64_DW)
-template void launch_ell_spmm<dw>(const EllDev<dw>&, const dw*, long long, dw*, long long, int, double*, int,
-                                  const DevState*, cudaStream_t);
 template void launch_ell_defect<dw>(const EllDev<dw>&, const dw*, const dw*, dw*, const DevState*, cudaStream_t);
 template void launch_ell_spmv_add<dw>(const EllDev<dw>&, const dw*, dw*, const DevState*, cudaStream_t);
-template void launch_ell_residual<dw>(const EllDev<dw>&, const dw*, const dw*, dw*, double*, int, cudaStream_t,
+template void launch_ell_residual<dw>(const EllDev<dw>&, const dw*, const dw*, dw*, double*, int, int, cudaStream_t,
                                       const int*);
 template void launch_ell_jacobi<dw>(const EllDev<dw>&, const dw*, const dw*, const dw*, dw*, int, const DevState*,
                                     cudaStream_t);

@@ -29,6 +29,15 @@ int stream_blocks_min(const GridDesc& g);
 int stream_blocks_cap(const GridDesc& g);
 int gram_chunks_min(const GridDesc& g);
 int gram_chunks_cap(const GridDesc& g);
+// threads per block: 256, fewer where 256 would leave SMs without a block
+int spread_threads(long long items);
+int stream_threads(const GridDesc& g);   // of the kernels launched with stream_blocks / spmm_blocks
+// launch of the window Gram: rows per task, warps, partial slots per value
+struct GramShape {
+  int rows, nwarps, slots;
+};
+template <typename T>
+GramShape gram_shape(const GridDesc& g, int C, int m);
 // number of SMs (set at hierarchy setup; 0 before)
 int sm_count();
 template <typename T>
@@ -53,15 +62,14 @@ inline int grid_for(long long work, int cap) {
 }
 
 // ---- ell.cu (algebraic hierarchies; vectors offset by G) -----------------
-// Y[:, c] = A X[:, c], c < C <= 12 (column pitches ldx, ldy); zaz (may be
-// null) receives per-block partials of X_c^T Y_c, value-major with stride
-// nblocks.  nblocks <= 0: one thread per row.
+// Y[:, c] = A X[:, c], c < C <= 12 (column pitches ldx, ldy; a ring's
+// pointers offset by G), one thread group per row
 template <typename T>
-void launch_ell_spmm(const EllDev<T>& A, const T* X, long long ldx, T* Y, long long ldy, int C, double* zaz,
-                     int nblocks, const DevState* state, cudaStream_t s);
+void launch_ell_spmm(const EllDev<T>& A, const SpmmIO<T>& io, long long ldx, long long ldy, int C,
+                     const DevState* state, cudaStream_t s);
 // r = b - A x, partials [|r|^2, |b|^2] over nblocks blocks; xnz as launch_residual
 template <typename T>
-void launch_ell_residual(const EllDev<T>& A, const T* b, const T* x, T* r, double* part, int nblocks,
+void launch_ell_residual(const EllDev<T>& A, const T* b, const T* x, T* r, double* part, int nblocks, int threads,
                          cudaStream_t s, const int* xnz = nullptr);
 // d = b - A x without norms (V-cycle defect)
 template <typename T>
@@ -83,17 +91,15 @@ template <typename TO>
 void launch_pack_flag(const GridDesc& g, const double* src, TO* dst, int* nz, cudaStream_t s);
 // SM count used to size one-wave launches (set at hierarchy setup)
 void set_sm_count(int n);
-// blocks (and zaz partial slots) of launch_spmm on grid g with C columns
+// blocks of launch_spmm on grid g with C columns
 template <typename T>
 int spmm_blocks(const GridDesc& g, int C);
 template <typename TI, typename TO>
 void launch_unpack(const GridDesc& g, const TI* src, TO* dst, long long ld, int ncols, cudaStream_t s);
 
-// Y = A X over C columns; if zaz != nullptr also partials of X_b^T Y_b
-// (value-major, stride kRedBlocks).  `state` (may be null) gates on done.
+// Y = A X over C columns.  `state` (may be null without a ring) gates on done.
 template <typename T>
-void launch_spmm(const GridDesc& g, const T* st, const T* X, T* Y, int C, double* zaz,
-                 const DevState* state, cudaStream_t s);
+void launch_spmm(const GridDesc& g, const T* st, const SpmmIO<T>& io, int C, const DevState* state, cudaStream_t s);
 // r = b - A x; partials [||r||^2, ||b||^2].  xnz (may be null): per problem,
 // 0 when x is known to be zero (then r = b without reading the stencil)
 template <typename T>
@@ -116,8 +122,8 @@ int sym_planes(int dim);
 // couplings with a pad row or column stored as zero
 void launch_sym_half(const GridDesc& g, const double* st, float* half, cudaStream_t s);
 // launch_spmm<float> and launch_jacobi<float> (scalar grids) reading the half
-void launch_spmm_sym(const GridDesc& g, const float* half, const float* X, float* Y, int C, double* zaz,
-                     const DevState* state, cudaStream_t s);
+void launch_spmm_sym(const GridDesc& g, const float* half, const SpmmIO<float>& io, int C, const DevState* state,
+                     cudaStream_t s);
 void launch_jacobi_sym(const GridDesc& g, const float* half, const float* dinv, const float* r, const float* sin,
                        float* out, int mode, const DevState* state, cudaStream_t s);
 // Vector operators (3 unknowns per node): t = r - A x (one sweep's residual)
@@ -171,20 +177,18 @@ void launch_convert_f32(const double* src, float* dst, long long count, cudaStre
 void launch_convert_dw(const double* src, dw* dst, long long count, cudaStream_t s);
 
 // ---- block.cu --------------------------------------------------------------
-// W partials: rows jj*C+a (window block jj, newest first), cols b:
-//   sum_i AP_slot(jj)[a][i] * Z[b][i]
+// W partials: value (jj C + a) C + b (window block jj, newest first) is
+//   sum_i AP_slot(jj)[a][i] * Z[b][i], in gram_shape's slots
 template <typename T>
 void launch_gram_window(const GridDesc& g, Window<T> win, const T* Z, int C, int m, double* part,
                         const DevState* state, cudaStream_t s);
-// P_new = Z - sum P_j beta_j, AP_new = AZ - sum AP_j beta_j into the next
-// ring slot; partials of sym(P^T AP) (upper triangle) and P^T r.
+// P_new = Z - sum P_j beta_j into the next ring slot
 template <typename T>
-void launch_orth_update(const GridDesc& g, Window<T> win, const T* Z, const T* AZ, const T* r,
-                        int C, double* part, const DevState* state, cudaStream_t s);
-// double-word: the Gram partials of the new block (launch_orth_update<dw>
-// leaves them to this kernel), same partial layout as the fused kernels
-void launch_orth_gram_dw(const GridDesc& g, Window<dw> win, const dw* r, int C, double* part,
-                         const DevState* state, cudaStream_t s);
+void launch_orth_update(const GridDesc& g, Window<T> win, const T* Z, int C, const DevState* state, cudaStream_t s);
+// partials of P^T AP (upper triangle) and P^T r of the next ring slot
+template <typename T>
+void launch_block_gram(const GridDesc& g, Window<T> win, const T* r, int C, double* part, const DevState* state,
+                       cudaStream_t s);
 // x += P alpha, r -= AP alpha (newest block); partial of ||r||^2
 template <typename T>
 void launch_update_xr(const GridDesc& g, Window<T> win, T* x, T* r, int C, double* part,
@@ -199,10 +203,9 @@ void launch_update_xr(const GridDesc& g, Window<T> win, T* x, T* r, int C, doubl
 mpcg_status place_kappa(const GridDesc& g, const double* kappa, int ne, double h, float* k32, double* k64,
                         unsigned long long* check, const double* st64, double* maxdiff, double* maxabs,
                         cudaStream_t s);
-// Y = A X (C <= 12 columns, zaz partials as launch_spmm with nblocks blocks;
-// false for other C) and the fused two-sweep Jacobi, A rebuilt from k32
-// (2D / 3D scalar, FP32).
-bool launch_spmm_mf(const GridDesc& g, const float* k32, const float* X, float* Y, int C, int nblocks, double* zaz,
+// Y = A X (C <= 12 columns, nblocks blocks; false for other C) and the fused
+// two-sweep Jacobi, A rebuilt from k32 (2D / 3D scalar, FP32).
+bool launch_spmm_mf(const GridDesc& g, const float* k32, const SpmmIO<float>& io, int C, int nblocks,
                     const DevState* state, cudaStream_t s);
 void launch_jacobi_mf(const GridDesc& g, const float* k32, const float* dinv, const float* r, float* out,
                       const DevState* state, cudaStream_t s);
@@ -216,11 +219,10 @@ void launch_init(DevState* st, int nb, const double* part_res, int nblk, double*
 constexpr int kSmallGrid = 96;
 constexpr int kSmallScratchAlpha = kMaxWindow * kMaxCols * kMaxCols;   // offset of small_alpha's values
 constexpr int kSmallScratch = kSmallScratchAlpha + kMaxCols * kMaxCols + 3 * kMaxCols;   // per problem
-void launch_small_beta(DevState* st, int nb, const double* part_W, int nchunks, int C, double* scratch,
+void launch_small_beta(DevState* st, int nb, const double* part_W, GramShape shape, int C, double* scratch,
                        unsigned* counter, cudaStream_t s);
-void launch_small_alpha(DevState* st, int nb, const double* part_G, int nblk_G, const double* part_zaz, int nblk_zaz,
-                        int zaz_stride, int C, double* alpha_hist, long long ahist_stride, double* scratch,
-                        unsigned* counter, cudaStream_t s);
+void launch_small_alpha(DevState* st, int nb, const double* part_G, int nblk_G, int C, double* alpha_hist,
+                        long long ahist_stride, double* scratch, unsigned* counter, cudaStream_t s);
 void launch_check(DevState* st, int nb, const double* part_r, int nblk, double* res_hist, long long hist_stride,
                   cudaGraphConditionalHandle cond, int use_cond, cudaStream_t s);
 void launch_set_params(DevState* st, int nb, double rtol, int maxit, int m, int C, double delta, double tau,

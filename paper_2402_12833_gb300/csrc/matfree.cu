@@ -189,16 +189,15 @@ __device__ __forceinline__ void mf_group(const float (&kq)[4][5], const float* _
   apply_row<1, 1, C>(kq, X, pitch, idx, px, pxy, acc);
 }
 
-// Y = A X over C columns (+ partials of z_c^T A z_c), A from k.
+// Y = A X over C columns, A from k.
 template <int C>
 __global__ void __launch_bounds__(kBlock, 3) k_spmm_mf(GridDesc g, const float* __restrict__ k32,
-                                                    const float* __restrict__ X, float* __restrict__ Y, double* zaz,
-                                                    const DevState* state) {
+                                                    SpmmIO<float> io, const DevState* state) {
   const int pb = blockIdx.y;
   if (state && state[pb].done) return;
-  float zacc[C];
-#pragma unroll
-  for (int c = 0; c < C; ++c) zacc[c] = 0.f;
+  const float* X;
+  float* Y;
+  spmm_operands(io, state + pb, X, Y);
   const long long ngroups = g.npts / 4;
   const long long bo = (long long)pb * g.len + g.G;
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < ngroups;
@@ -221,15 +220,8 @@ __global__ void __launch_bounds__(kBlock, 3) k_spmm_mf(GridDesc g, const float* 
       for (int w = 0; w < 4; ++w)
         if (!row_in || x0 + w >= g.nx) acc[c][w] = 0.f;   // pad points: zero rows
       Vec<float>::store(Y + (long long)c * g.cp + idx, acc[c]);
-      if (zaz) {
-        float xc[4];
-        Vec<float>::load_keep(X + (long long)c * g.cp + idx, xc);
-#pragma unroll
-        for (int w = 0; w < 4; ++w) zacc[c] = fmaf(xc[w], acc[c][w], zacc[c]);
-      }
     }
   }
-  if (zaz) block_sum_store<float, C>(zacc, zaz + (long long)pb * C * gridDim.x, gridDim.x, blockIdx.x);
 }
 
 // Two damped-Jacobi sweeps from zero on the fine grid, fused (as k_jacobi
@@ -312,13 +304,12 @@ __device__ __forceinline__ void row_coefs2(const float (&kq)[2][5], float (&cf)[
 
 template <int C>
 __global__ void __launch_bounds__(kBlock, 3) k_spmm_mf2d(GridDesc g, const float* __restrict__ k32,
-                                                      const float* __restrict__ X, float* __restrict__ Y, double* zaz,
-                                                      const DevState* state) {
+                                                      SpmmIO<float> io, const DevState* state) {
   const int pb = blockIdx.y;
   if (state && state[pb].done) return;
-  float zacc[C];
-#pragma unroll
-  for (int c = 0; c < C; ++c) zacc[c] = 0.f;
+  const float* X;
+  float* Y;
+  spmm_operands(io, state + pb, X, Y);
   const long long ngroups = g.npts / 4;
   const long long bo = (long long)pb * g.len + g.G;
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < ngroups;
@@ -350,15 +341,8 @@ __global__ void __launch_bounds__(kBlock, 3) k_spmm_mf2d(GridDesc g, const float
       for (int w = 0; w < 4; ++w)
         if (y >= g.ny || x0 + w >= g.nx) acc[w] = 0.f;   // pad points: zero rows
       Vec<float>::store(Y + (long long)c * g.cp + idx, acc);
-      if (zaz) {
-        float xc[4];
-        Vec<float>::load_keep(X + (long long)c * g.cp + idx, xc);
-#pragma unroll
-        for (int w = 0; w < 4; ++w) zacc[c] = fmaf(xc[w], acc[w], zacc[c]);
-      }
     }
   }
-  if (zaz) block_sum_store<float, C>(zacc, zaz + (long long)pb * C * gridDim.x, gridDim.x, blockIdx.x);
 }
 
 __global__ void __launch_bounds__(kBlock, 4) k_jacobi_mf2d(GridDesc g, const float* __restrict__ k32,
@@ -418,30 +402,31 @@ mpcg_status place_kappa(const GridDesc& g, const double* kappa, int ne, double h
 }
 
 #define MPCG_MF_CASES(K, ...)                                                                      \
-  case 1: K<1><<<__VA_ARGS__>>>(g, k32, X, Y, zaz, state); break;                                   \
-  case 2: K<2><<<__VA_ARGS__>>>(g, k32, X, Y, zaz, state); break;                                   \
-  case 3: K<3><<<__VA_ARGS__>>>(g, k32, X, Y, zaz, state); break;                                   \
-  case 4: K<4><<<__VA_ARGS__>>>(g, k32, X, Y, zaz, state); break;                                   \
-  case 5: K<5><<<__VA_ARGS__>>>(g, k32, X, Y, zaz, state); break;                                   \
-  case 6: K<6><<<__VA_ARGS__>>>(g, k32, X, Y, zaz, state); break;                                   \
-  case 7: K<7><<<__VA_ARGS__>>>(g, k32, X, Y, zaz, state); break;                                   \
-  case 8: K<8><<<__VA_ARGS__>>>(g, k32, X, Y, zaz, state); break;                                   \
-  case 9: K<9><<<__VA_ARGS__>>>(g, k32, X, Y, zaz, state); break;                                   \
-  case 10: K<10><<<__VA_ARGS__>>>(g, k32, X, Y, zaz, state); break;                                 \
-  case 11: K<11><<<__VA_ARGS__>>>(g, k32, X, Y, zaz, state); break;                                 \
-  case 12: K<12><<<__VA_ARGS__>>>(g, k32, X, Y, zaz, state); break;
+  case 1: K<1><<<__VA_ARGS__>>>(g, k32, io, state); break;                                   \
+  case 2: K<2><<<__VA_ARGS__>>>(g, k32, io, state); break;                                   \
+  case 3: K<3><<<__VA_ARGS__>>>(g, k32, io, state); break;                                   \
+  case 4: K<4><<<__VA_ARGS__>>>(g, k32, io, state); break;                                   \
+  case 5: K<5><<<__VA_ARGS__>>>(g, k32, io, state); break;                                   \
+  case 6: K<6><<<__VA_ARGS__>>>(g, k32, io, state); break;                                   \
+  case 7: K<7><<<__VA_ARGS__>>>(g, k32, io, state); break;                                   \
+  case 8: K<8><<<__VA_ARGS__>>>(g, k32, io, state); break;                                   \
+  case 9: K<9><<<__VA_ARGS__>>>(g, k32, io, state); break;                                   \
+  case 10: K<10><<<__VA_ARGS__>>>(g, k32, io, state); break;                                 \
+  case 11: K<11><<<__VA_ARGS__>>>(g, k32, io, state); break;                                 \
+  case 12: K<12><<<__VA_ARGS__>>>(g, k32, io, state); break;
 
-bool launch_spmm_mf(const GridDesc& g, const float* k32, const float* X, float* Y, int C, int nblocks, double* zaz,
+bool launch_spmm_mf(const GridDesc& g, const float* k32, const SpmmIO<float>& io, int C, int nblocks,
                     const DevState* state, cudaStream_t s) {
   const dim3 grid(nblocks, g.nb);
+  const int threads = stream_threads(g);
   if (g.dim == 3) {
     switch (C) {
-      MPCG_MF_CASES(k_spmm_mf, grid, kBlock, 0, s)
+      MPCG_MF_CASES(k_spmm_mf, grid, threads, 0, s)
       default: return false;
     }
   } else {
     switch (C) {
-      MPCG_MF_CASES(k_spmm_mf2d, grid, kBlock, 0, s)
+      MPCG_MF_CASES(k_spmm_mf2d, grid, threads, 0, s)
       default: return false;
     }
   }

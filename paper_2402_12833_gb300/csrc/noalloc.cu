@@ -148,7 +148,7 @@ extern "C" mpcg_status mg_stencil_apply_noalloc(int dim, int nodes, const double
   }
   launch_pack<double, double>(g, values_dev, g.n, st_pad, S, s);
   launch_pack<double, double>(g, X_dev, g.n, x_pad, ncols, s);
-  launch_spmm<double>(g, st_pad, x_pad, y_pad, ncols, nullptr, nullptr, s);
+  launch_spmm<double>(g, st_pad, spmm_io<double>(x_pad, y_pad), ncols, nullptr, s);
   launch_unpack<double, double>(g, y_pad, Y_dev, g.n, ncols, s);
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) {

@@ -64,29 +64,46 @@ __device__ void reduce_values(const double* __restrict__ part, int nv, int nblk,
 // summed by block v % gridDim.x over its nblk partials in a fixed order and
 // written to red[v].  Exactly one block -- the last to finish -- gets true,
 // after which every red[v] is visible to it (read them with __ldcg).  The
-// counter is zero between launches.  Values below nv_a come from part_a
-// (stride stride_a, nblk_a partials), the rest from part_b.
-__device__ bool reduce_values_grid(const double* __restrict__ part_a, int nv_a, int nblk_a, int stride_a,
-                                   const double* __restrict__ part_b, int nv_b, int nblk_b, int stride_b,
-                                   double* red, unsigned* counter) {
+// counter is zero between launches.
+__device__ bool reduce_values_grid(const double* __restrict__ part, int nv, int nblk, int stride, double* red,
+                                   unsigned* counter) {
   __shared__ double wsum[32];
   __shared__ bool last;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  for (int v = blockIdx.x; v < nv_a + nv_b; v += gridDim.x) {
-    const double* p = v < nv_a ? part_a + (long long)v * stride_a : part_b + (long long)(v - nv_a) * stride_b;
-    const int nb = v < nv_a ? nblk_a : nblk_b;
-    double a = 0.0;
-    for (int b = threadIdx.x; b < nb; b += blockDim.x) a += p[b];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if (nv > 2 * (int)gridDim.x) {
+    // many values: one warp each (the FP64 pipe takes a warp instruction per
+    // 64 cycles, so the serial part per value is what costs)
+    for (int v = blockIdx.x + gridDim.x * warp; v < nv; v += gridDim.x * nw) {
+      const double* p = part + (long long)v * stride;
+      double a0 = 0.0, a1 = 0.0;
+      int b = lane;
+      for (; b + 32 < nblk; b += 64) {
+        a0 += p[b];
+        a1 += p[b + 32];
+      }
+      if (b < nblk) a0 += p[b];
+      double a = a0 + a1;
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    if (lane == 0) wsum[warp] = a;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += wsum[w];
-      red[v] = t;
+      for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+      if (lane == 0) red[v] = a;
     }
-    __syncthreads();
+  } else {
+    for (int v = blockIdx.x; v < nv; v += gridDim.x) {
+      const double* p = part + (long long)v * stride;
+      double a = 0.0;
+      for (int b = threadIdx.x; b < nblk; b += blockDim.x) a += p[b];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+      if (lane == 0) wsum[warp] = a;
+      __syncthreads();
+      if (warp == 0) {
+        double t = lane < nw ? wsum[lane] : 0.0;
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) red[v] = t;
+      }
+      __syncthreads();
+    }
   }
   __threadfence();
   __syncthreads();
@@ -223,28 +240,46 @@ __global__ void k_init(DevState* st, const double* part_res, int nblk, double* r
 }
 
 // beta_j = G_j^+ W_j for the window blocks: the W partial sums are reduced by
-// all blocks of the grid, the last block forms beta.
-__global__ void k_small_beta(DevState* st, const double* part_W, int nchunks, int C, double* scratch,
+// all blocks of the grid, the last block forms beta, and the energy
+// zpz_b = sum_j (W_j^T beta_j)_bb that the orthogonalisation removes from
+// column b: p = z - sum_j P_j beta_j with p and the P_j A-orthogonal gives
+// z^T A z = p^T A p + sum_j beta_j^T G_j beta_j and G_j beta_j = W_j up to the
+// cut of the pseudo-inverse, so the drop rule needs no product A Z.
+__global__ void k_small_beta(DevState* st, const double* part_W, GramShape shape, int C, double* scratch,
                              unsigned* counter) {
   const int pb = blockIdx.y;
   st += pb;
   scratch += (long long)pb * kSmallScratch;
   counter += 2 * pb;
-  part_W += (long long)pb * st->m * C * C * nchunks;
+  part_W += (long long)pb * st->m * C * C * shape.slots;
   if (st->done) return;
   const int cnt = st->count;
-  if (cnt == 0) return;
+  if (cnt == 0) {
+    if (blockIdx.x == 0 && threadIdx.x < C) st->zpz[threadIdx.x] = 0.0;
+    return;
+  }
   const int m = st->m, newest = st->newest;
-  if (!reduce_values_grid(part_W, cnt * C * C, nchunks, nchunks, nullptr, 0, 0, 0, scratch, counter)) return;
+  const int ntask = (cnt * C + shape.rows - 1) / shape.rows;
+  const int walkers = shape.nwarps / ntask < shape.slots ? shape.nwarps / ntask : shape.slots;   // gram_walkers
+  if (!reduce_values_grid(part_W, cnt * C * C, walkers, shape.slots, scratch, counter)) return;
   __shared__ double W[kMaxWindow * kMaxCols * kMaxCols];
   for (int e = threadIdx.x; e < cnt * C * C; e += blockDim.x) W[e] = __ldcg(scratch + e);
   __syncthreads();
-  for (int e = threadIdx.x; e < cnt * C * C; e += blockDim.x) {
-    const int jj = e / (C * C), a = (e / C) % C, b = e % C;
-    const int slot = (newest - jj + m) % m;
-    double s = 0.0;
-    for (int c = 0; c < C; ++c) s += st->gpinv[slot][a][c] * W[(jj * C + c) * C + b];
-    st->beta[jj][a][b] = s;
+  // one warp per column b, lanes over the rows (jj, a)
+  const int lane = threadIdx.x & 31;
+  for (int b = threadIdx.x >> 5; b < C; b += blockDim.x >> 5) {
+    double e = 0.0;
+    for (int r = lane; r < cnt * C; r += 32) {
+      const int jj = r / C, a = r - jj * C;
+      const double* gp = st->gpinv[(newest - jj + m) % m][a];
+      double s = 0.0;
+      for (int c = 0; c < C; ++c) s = fma(gp[c], W[(jj * C + c) * C + b], s);
+      st->beta[jj][a][b] = s;
+      e = fma(W[r * C + b], s, e);
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) e += __shfl_xor_sync(0xffffffffu, e, o);
+    if (lane == 0) st->zpz[b] = e;
   }
 }
 
@@ -252,8 +287,8 @@ __global__ void k_small_beta(DevState* st, const double* part_W, int nchunks, in
 // reduced Gram values ((0,0), (0,1), ..., (0,C-1), (1,1), ...).
 __device__ __forceinline__ int tri_index(int a, int b, int C) { return a * C - a * (a - 1) / 2 + (b - a); }
 
-// alpha = G^+ g after the grid reduction of G = sym(P^T A P), g = P^T r and
-// the z^T A z of the new block; G^+ also goes to the window ring.  One warp,
+// alpha = G^+ g after the grid reduction of G = P^T A P and g = P^T r of
+// the new block; G^+ also goes to the window ring.  One warp,
 // C columns known at compile time.  GB300 issues one FP64 warp instruction
 // per 64 cycles per SM sub-partition whatever the active lanes, so the
 // factorisation keeps one row per lane in registers and every step is a
@@ -264,7 +299,6 @@ __device__ __forceinline__ int tri_index(int a, int b, int C) { return a * C - a
 // row i of (D G D)^{-1} = L^{-T} (L^{-1} e_i) by backward substitution.
 template <int C>
 __global__ void __launch_bounds__(kBlock) k_small_alpha(DevState* st, const double* part_G, int nblk_G,
-                                                        const double* part_zaz, int nblk_zaz, int zaz_stride,
                                                         double* alpha_hist, long long ahist_stride, double* scratch,
                                                         unsigned* counter) {
   constexpr int NG = C * (C + 1) / 2;
@@ -272,12 +306,11 @@ __global__ void __launch_bounds__(kBlock) k_small_alpha(DevState* st, const doub
   const int pb = blockIdx.y;
   st += pb;
   part_G += (long long)pb * (NG + C) * nblk_G;
-  part_zaz += (long long)pb * C * zaz_stride;
   if (alpha_hist) alpha_hist += pb * ahist_stride;
   scratch += (long long)pb * kSmallScratch + kSmallScratchAlpha;
   counter += 2 * pb + 1;
   if (st->done) return;
-  __shared__ double red[NG + 2 * C];
+  __shared__ double red[NG + C];
   __shared__ double Lsm[C][C];
   __shared__ double dsm[C];
   __shared__ int map[C];
@@ -285,18 +318,17 @@ __global__ void __launch_bounds__(kBlock) k_small_alpha(DevState* st, const doub
   __shared__ double A[kPad * kPad], V[kPad * kPad], Ah[kPad * kPad];
   __shared__ double rc[kPad], rs[kPad], lam[kPad];
   __shared__ int rp[kPad], rq[kPad];
-  if (!reduce_values_grid(part_G, NG + C, nblk_G, nblk_G, part_zaz, C, nblk_zaz, zaz_stride, scratch, counter))
-    return;
-  for (int e = threadIdx.x; e < NG + 2 * C; e += blockDim.x) red[e] = __ldcg(scratch + e);
+  if (!reduce_values_grid(part_G, NG + C, nblk_G, nblk_G, scratch, counter)) return;
+  for (int e = threadIdx.x; e < NG + C; e += blockDim.x) red[e] = __ldcg(scratch + e);
   __syncthreads();
   if (threadIdx.x >= 32) return;
   const int lane = threadIdx.x;
-  // column-drop rule on the diagonal (the partials hold p_a ap_b + p_b ap_a)
+  // column-drop rule on the diagonal
   double pap = 0.0, gv = 0.0;
   bool act = false, bad = false;
   if (lane < C) {
-    pap = 0.5 * red[tri_index(lane, lane, C)];
-    const double zaz = red[NG + C + lane];
+    pap = red[tri_index(lane, lane, C)];
+    const double zaz = pap + st->zpz[lane];   // z^T A z (k_small_beta)
     gv = red[NG + lane];
     bad = !isfinite(pap) || !isfinite(zaz);
     act = pap > st->delta * zaz && pap > 0.0;
@@ -320,15 +352,14 @@ __global__ void __launch_bounds__(kBlock) k_small_alpha(DevState* st, const doub
 #pragma unroll
   for (int j = 0; j < C; ++j) Z[j] = 0.0;
   if (na > 0) {
-    // row `lane` of D G D (G = 0.5 red; scaling by 0.5 is exact)
+    // row `lane` of D G D
     double Ar[C];
-    const double hdi = 0.5 * di;
 #pragma unroll
     for (int j = 0; j < C; ++j) {
       const int cj = map[j < na ? j : 0];
       const double dj = __shfl_sync(kFull, dsc, cj);
       const int lo = ci < cj ? ci : cj, hi = ci < cj ? cj : ci;
-      Ar[j] = (lane < na && j < na) ? hdi * red[tri_index(lo, hi, C)] * dj : 0.0;
+      Ar[j] = (lane < na && j < na) ? di * red[tri_index(lo, hi, C)] * dj : 0.0;
     }
     // Cholesky D G D = L L^T; dinv[k] = 1 / L_kk
     double dinv[C];
@@ -397,7 +428,7 @@ __global__ void __launch_bounds__(kBlock) k_small_alpha(DevState* st, const doub
         double v = 0.0;
         if (i < na && j < na) {
           const int a = map[i], b = map[j];
-          v = (0.5 * dsm[a]) * red[tri_index(a < b ? a : b, a < b ? b : a, C)] * dsm[b];
+          v = dsm[a] * red[tri_index(a < b ? a : b, a < b ? b : a, C)] * dsm[b];
         }
         A[e] = v;
       }
@@ -686,16 +717,14 @@ void launch_init(DevState* st, int nb, const double* part_res, int nblk, double*
                  cudaGraphConditionalHandle cond, int use_cond, cudaStream_t s) {
   k_init<<<nb, kBlock, 0, s>>>(st, part_res, nblk, res_hist, hist_stride, cond, use_cond);
 }
-void launch_small_beta(DevState* st, int nb, const double* part_W, int nchunks, int C, double* scratch,
+void launch_small_beta(DevState* st, int nb, const double* part_W, GramShape shape, int C, double* scratch,
                        unsigned* counter, cudaStream_t s) {
-  k_small_beta<<<dim3(kSmallGrid, nb), kBlock, 0, s>>>(st, part_W, nchunks, C, scratch, counter);
+  k_small_beta<<<dim3(kSmallGrid, nb), kBlock, 0, s>>>(st, part_W, shape, C, scratch, counter);
 }
-void launch_small_alpha(DevState* st, int nb, const double* part_G, int nblk_G, const double* part_zaz, int nblk_zaz,
-                        int zaz_stride, int C, double* alpha_hist, long long ahist_stride, double* scratch,
-                        unsigned* counter, cudaStream_t s) {
+void launch_small_alpha(DevState* st, int nb, const double* part_G, int nblk_G, int C, double* alpha_hist,
+                        long long ahist_stride, double* scratch, unsigned* counter, cudaStream_t s) {
   MPCG_SMALL_C_SWITCH(C, (k_small_alpha<CC><<<dim3(kSmallGrid, nb), kBlock, 0, s>>>(
-                             st, part_G, nblk_G, part_zaz, nblk_zaz, zaz_stride, alpha_hist, ahist_stride, scratch,
-                             counter)));
+                             st, part_G, nblk_G, alpha_hist, ahist_stride, scratch, counter)));
 }
 void launch_check(DevState* st, int nb, const double* part_r, int nblk, double* res_hist, long long hist_stride,
                   cudaGraphConditionalHandle cond, int use_cond, cudaStream_t s) {

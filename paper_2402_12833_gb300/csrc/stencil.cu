@@ -206,16 +206,16 @@ __device__ __forceinline__ void stencil_group(const T* __restrict__ st, long lon
 // The FP32 3D instances with up to 6 columns run three blocks per SM (at most
 // 85 registers) in one wave of resident blocks (spmm_blocks): measured faster
 // than two blocks per SM over two waves, whose loads wait longer.
-template <typename T, int DIM, int C, bool ZAZ, bool SYM = false>
-__global__ void __launch_bounds__(kBlock, (sizeof(T) == 4 && DIM == 3 && C <= 6) ? 3 : (kIsDw<T> ? 2 : 1)) k_spmm(GridDesc g, const T* __restrict__ st, const T* __restrict__ X,
-                                                 T* __restrict__ Y, double* zaz, const DevState* state) {
+template <typename T, int DIM, int C, bool SYM = false>
+__global__ void __launch_bounds__(kBlock, (sizeof(T) == 4 && DIM == 3 && C <= 6) ? 3 : (kIsDw<T> ? 2 : 1))
+    k_spmm(GridDesc g, const T* __restrict__ st, SpmmIO<T> io, const DevState* state) {
   const int pb = blockIdx.y;
   if (state && state[pb].done) return;
+  const T* X;
+  T* Y;
+  spmm_operands(io, state + pb, X, Y);
   constexpr int W = Vec<T>::W;
   const long long bo = (long long)pb * g.len;
-  T zacc[ZAZ ? C : 1];
-#pragma unroll
-  for (int c = 0; c < (ZAZ ? C : 1); ++c) zacc[c] = 0;
   const long long ngroups = g.npts / W;
   for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < ngroups;
        q += (long long)gridDim.x * blockDim.x) {
@@ -227,17 +227,8 @@ __global__ void __launch_bounds__(kBlock, (sizeof(T) == 4 && DIM == 3 && C <= 6)
       for (int w = 0; w < W; ++w) acc[c][w] = 0;
     stencil_group<T, DIM, C, SYM>(st, g.cp, X, idx, g.px, g.pxy, acc);
 #pragma unroll
-    for (int c = 0; c < C; ++c) {
-      Vec<T>::store(Y + (long long)c * g.cp + idx, acc[c]);
-      if (ZAZ) {
-        T xc[W];
-        Vec<T>::load_keep(X + (long long)c * g.cp + idx, xc);
-#pragma unroll
-        for (int w = 0; w < W; ++w) zacc[c] = fma(xc[w], acc[c][w], zacc[c]);
-      }
-    }
+    for (int c = 0; c < C; ++c) Vec<T>::store(Y + (long long)c * g.cp + idx, acc[c]);
   }
-  if (ZAZ) block_sum_store<T, ZAZ ? C : 1>(zacc, zaz + (long long)pb * C * gridDim.x, gridDim.x, blockIdx.x);
 }
 
 // r = b - A x with the partials of |r|^2 and |b|^2.  xnz (may be null) flags
@@ -793,17 +784,17 @@ __global__ void k_sym_half(GridDesc g, const double* __restrict__ st, float* __r
 // of W x-points), so that only the C columns' accumulators are live (all
 // three components per thread would cap occupancy at one block per SM for
 // C = 5).  Consecutive threads take consecutive groups of the same component.
-template <typename T, int C, bool ZAZ>
-__global__ void __launch_bounds__(kBlock) k_vspmm(GridDesc g, const T* __restrict__ st, const T* __restrict__ X,
-                                                  T* __restrict__ Y, double* zaz, const DevState* state) {
+template <typename T, int C>
+__global__ void __launch_bounds__(kBlock) k_vspmm(GridDesc g, const T* __restrict__ st, SpmmIO<T> io,
+                                                  const DevState* state) {
   const int pb = blockIdx.y;
   if (state && state[pb].done) return;
+  const T* X;
+  T* Y;
+  spmm_operands(io, state + pb, X, Y);
   constexpr int W = Vec<T>::W;
   const long long bo = (long long)pb * g.len;
   const long long cs = g.cstride;
-  T zacc[ZAZ ? C : 1];
-#pragma unroll
-  for (int c = 0; c < (ZAZ ? C : 1); ++c) zacc[c] = 0;
   const long long ngroups = cs / W;
   for (long long item = blockIdx.x * (long long)blockDim.x + threadIdx.x; item < 3 * ngroups;
        item += (long long)gridDim.x * blockDim.x) {
@@ -838,18 +829,8 @@ __global__ void __launch_bounds__(kBlock) k_vspmm(GridDesc g, const T* __restric
       }
     }
 #pragma unroll
-    for (int c = 0; c < C; ++c) {
-      const long long o = (long long)c * g.cp + idx0 + a * cs;
-      Vec<T>::store(Y + o, acc[c]);
-      if (ZAZ) {
-        T xc[W];
-        Vec<T>::load_keep(X + o, xc);
-#pragma unroll
-        for (int w = 0; w < W; ++w) zacc[c] = fma(xc[w], acc[c][w], zacc[c]);
-      }
-    }
+    for (int c = 0; c < C; ++c) Vec<T>::store(Y + (long long)c * g.cp + idx0 + a * cs, acc[c]);
   }
-  if (ZAZ) block_sum_store<T, ZAZ ? C : 1>(zacc, zaz + (long long)pb * C * gridDim.x, gridDim.x, blockIdx.x);
 }
 
 // r = b - A x for a vector operator, one thread per (component, group), the
@@ -1041,13 +1022,12 @@ int spmm_blocks(const GridDesc& g, int C) {
   int dflt = nb;
   if (sizeof(T) == 4 && g.dim == 3 && g.ncomp == 1 && C <= 6 && g_sm_count > 0) {
     const long long groups = g.npts / 2;
-    const long long need = (groups + kBlock * 16 - 1) / (kBlock * 16);
+    const long long bd = stream_threads(g), need = (groups + bd * 16 - 1) / (bd * 16);
     long long w = 3LL * g_sm_count;   // one wave at three blocks per SM
     if (w < need) w = need;
     dflt = (int)(w < nb ? w : nb);
   }
-  // tuned: between the 64-points-per-thread minimum and the partial-sum
-  // slots the solver reserves (stream_blocks_cap)
+  // tuned: within the range of the streaming kernels
   const int v = tune::lookup(tune::kSpmm, kind_of<T>(), g.npts, g.nb, C, dflt);
   const int lo = stream_blocks_min(g), hi = stream_blocks_cap(g);
   return v < lo ? lo : (v > hi ? hi : v);
@@ -1071,13 +1051,17 @@ template void launch_unpack<float, float>(const GridDesc&, const float*, float*,
 #endif
 
 template <typename T, int DIM, bool SYM = false>
-static void spmm_dim(const GridDesc& g, const T* st, const T* X, T* Y, int C, double* zaz, const DevState* state,
+static void spmm_dim(const GridDesc& g, const T* st, const SpmmIO<T>& io, int C, const DevState* state,
                      cudaStream_t s) {
-  const dim3 grid(spmm_blocks<T>(g, C), g.nb);
+  int threads = stream_threads(g), blocks = spmm_blocks<T>(g, C);
+  if (g.nb > 1 && threads < kBlock) {   // the batch fills the SMs: whole blocks
+    blocks = (int)(((long long)blocks * threads + kBlock - 1) / kBlock);
+    threads = kBlock;
+  }
+  const dim3 grid(blocks, g.nb);
 #define MPCG_SPMM_CASE(CC)                                                                      \
   case CC:                                                                                      \
-    if (zaz) k_spmm<T, DIM, CC, true, SYM><<<grid, kBlock, 0, s>>>(g, st, X, Y, zaz, state);    \
-    else k_spmm<T, DIM, CC, false, SYM><<<grid, kBlock, 0, s>>>(g, st, X, Y, zaz, state);      \
+    k_spmm<T, DIM, CC, SYM><<<grid, threads, 0, s>>>(g, st, io, state);                         \
     break;
   switch (C) {
     MPCG_SPMM_CASE(1) MPCG_SPMM_CASE(2) MPCG_SPMM_CASE(3) MPCG_SPMM_CASE(4) MPCG_SPMM_CASE(5)
@@ -1089,13 +1073,13 @@ static void spmm_dim(const GridDesc& g, const T* st, const T* X, T* Y, int C, do
 }
 
 template <typename T>
-static void vspmm(const GridDesc& g, const T* st, const T* X, T* Y, int C, double* zaz, const DevState* state,
+static void vspmm(const GridDesc& g, const T* st, const SpmmIO<T>& io, int C, const DevState* state,
                   cudaStream_t s) {
   const dim3 grid(stream_blocks(g), g.nb);
+  const int threads = stream_threads(g);
 #define MPCG_VSPMM_CASE(CC)                                                                     \
   case CC:                                                                                      \
-    if (zaz) k_vspmm<T, CC, true><<<grid, kBlock, 0, s>>>(g, st, X, Y, zaz, state);             \
-    else k_vspmm<T, CC, false><<<grid, kBlock, 0, s>>>(g, st, X, Y, zaz, state);               \
+    k_vspmm<T, CC><<<grid, threads, 0, s>>>(g, st, io, state);                                  \
     break;
   switch (C) {
     MPCG_VSPMM_CASE(1) MPCG_VSPMM_CASE(2) MPCG_VSPMM_CASE(3) MPCG_VSPMM_CASE(4) MPCG_VSPMM_CASE(5)
@@ -1106,26 +1090,25 @@ static void vspmm(const GridDesc& g, const T* st, const T* X, T* Y, int C, doubl
 }
 
 template <typename T>
-void launch_spmm(const GridDesc& g, const T* st, const T* X, T* Y, int C, double* zaz, const DevState* state,
-                 cudaStream_t s) {
-  if (g.ncomp == 3) vspmm<T>(g, st, X, Y, C, zaz, state, s);
-  else if (g.dim == 3) spmm_dim<T, 3>(g, st, X, Y, C, zaz, state, s);
-  else spmm_dim<T, 2>(g, st, X, Y, C, zaz, state, s);
+void launch_spmm(const GridDesc& g, const T* st, const SpmmIO<T>& io, int C, const DevState* state, cudaStream_t s) {
+  if (g.ncomp == 3) vspmm<T>(g, st, io, C, state, s);
+  else if (g.dim == 3) spmm_dim<T, 3>(g, st, io, C, state, s);
+  else spmm_dim<T, 2>(g, st, io, C, state, s);
 }
 #if MPCG_STENCIL_PLAIN
-template void launch_spmm<double>(const GridDesc&, const double*, const double*, double*, int, double*,
-                                  const DevState*, cudaStream_t);
-template void launch_spmm<float>(const GridDesc&, const float*, const float*, float*, int, double*,
-                                 const DevState*, cudaStream_t);
+template void launch_spmm<double>(const GridDesc&, const double*, const SpmmIO<double>&, int, const DevState*,
+                                  cudaStream_t);
+template void launch_spmm<float>(const GridDesc&, const float*, const SpmmIO<float>&, int, const DevState*,
+                                 cudaStream_t);
 #endif
 
 template <typename T>
 void launch_residual(const GridDesc& g, const T* st, const T* b, const T* x, T* r, double* part, cudaStream_t s,
                      const int* xnz) {
   const dim3 grid(stream_blocks(g), g.nb);
-  if (g.ncomp == 3) k_vres<T, true><<<grid, kBlock, 0, s>>>(g, st, b, x, r, part, nullptr, xnz);
-  else if (g.dim == 3) k_residual<T, 3><<<grid, kBlock, 0, s>>>(g, st, b, x, r, part, xnz);
-  else k_residual<T, 2><<<grid, kBlock, 0, s>>>(g, st, b, x, r, part, xnz);
+  if (g.ncomp == 3) k_vres<T, true><<<grid, stream_threads(g), 0, s>>>(g, st, b, x, r, part, nullptr, xnz);
+  else if (g.dim == 3) k_residual<T, 3><<<grid, stream_threads(g), 0, s>>>(g, st, b, x, r, part, xnz);
+  else k_residual<T, 2><<<grid, stream_threads(g), 0, s>>>(g, st, b, x, r, part, xnz);
 }
 #if MPCG_STENCIL_PLAIN
 template void launch_residual<double>(const GridDesc&, const double*, const double*, const double*, double*,
@@ -1239,7 +1222,7 @@ __global__ void k_sum_columns(GridDesc g, const T* __restrict__ Zc, int ncols, T
 
 template <typename T>
 void launch_sum_columns(const GridDesc& g, const T* Zc, int ncols, T* out, const DevState* state, cudaStream_t s) {
-  k_sum_columns<T><<<dim3(stream_blocks(g), g.nb), kBlock, 0, s>>>(g, Zc, ncols, out, state);
+  k_sum_columns<T><<<dim3(stream_blocks(g), g.nb), stream_threads(g), 0, s>>>(g, Zc, ncols, out, state);
 }
 #if MPCG_STENCIL_PLAIN
 template void launch_sum_columns<double>(const GridDesc&, const double*, int, double*, const DevState*, cudaStream_t);
@@ -1387,8 +1370,7 @@ template void launch_pack<double, dw>(const GridDesc&, const double*, long long,
 template void launch_unpack<dw, double>(const GridDesc&, const dw*, double*, long long, int, cudaStream_t);
 template void launch_pack_flag<dw>(const GridDesc&, const double*, dw*, int*, cudaStream_t);
 template int spmm_blocks<dw>(const GridDesc&, int);
-template void launch_spmm<dw>(const GridDesc&, const dw*, const dw*, dw*, int, double*, const DevState*,
-                              cudaStream_t);
+template void launch_spmm<dw>(const GridDesc&, const dw*, const SpmmIO<dw>&, int, const DevState*, cudaStream_t);
 template void launch_residual<dw>(const GridDesc&, const dw*, const dw*, const dw*, dw*, double*, cudaStream_t,
                                   const int*);
 template void launch_restrict<dw>(const GridDesc&, const GridDesc&, const dw*, dw*, const DevState*, cudaStream_t);
@@ -1436,11 +1418,11 @@ void launch_sym_half(const GridDesc& g, const double* st, float* half, cudaStrea
   else k_sym_half<2><<<grid_for(g.cp, 4096), kBlock, 0, s>>>(g, st, half);
 }
 
-void launch_spmm_sym(const GridDesc& g, const float* half, const float* X, float* Y, int C, double* zaz,
-                     const DevState* state, cudaStream_t s) {
+void launch_spmm_sym(const GridDesc& g, const float* half, const SpmmIO<float>& io, int C, const DevState* state,
+                     cudaStream_t s) {
   if (g.ncomp != 1) return;
-  if (g.dim == 3) spmm_dim<float, 3, true>(g, half, X, Y, C, zaz, state, s);
-  else spmm_dim<float, 2, true>(g, half, X, Y, C, zaz, state, s);
+  if (g.dim == 3) spmm_dim<float, 3, true>(g, half, io, C, state, s);
+  else spmm_dim<float, 2, true>(g, half, io, C, state, s);
 }
 
 void launch_jacobi_sym(const GridDesc& g, const float* half, const float* dinv, const float* r, const float* sin,

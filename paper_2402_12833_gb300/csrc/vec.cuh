@@ -73,6 +73,20 @@ struct VecN<T, 1> {
   __device__ static __forceinline__ void store(T* p, const T (&v)[1]) { *p = v[0]; }
 };
 template <>
+struct VecN<float, 2> {
+  __device__ static __forceinline__ void load(const float* p, float (&v)[2]) {
+    const float2 q = __ldcs(reinterpret_cast<const float2*>(p));
+    v[0] = q.x; v[1] = q.y;
+  }
+  __device__ static __forceinline__ void load_keep(const float* p, float (&v)[2]) {
+    const float2 q = *reinterpret_cast<const float2*>(p);
+    v[0] = q.x; v[1] = q.y;
+  }
+  __device__ static __forceinline__ void store(float* p, const float (&v)[2]) {
+    *reinterpret_cast<float2*>(p) = make_float2(v[0], v[1]);
+  }
+};
+template <>
 struct VecN<float, 4> : Vec<float> {};
 template <>
 struct VecN<double, 2> : Vec<double> {};
@@ -110,6 +124,19 @@ __device__ __forceinline__ void rs_step(T (&a)[NV], int& base, int& nvalid, int 
   }
 }
 
+// Warp sum of NV per-lane values: afterwards lane holds, in a[0 .. rs_count(NV,
+// 5)), the sums of the values base + i, i < nvalid.
+template <typename T, int NV>
+__device__ __forceinline__ void warp_reduce_scatter(T (&a)[NV], int& base, int& nvalid, int lane) {
+  base = 0;
+  nvalid = NV;
+  rs_step<T, NV, rs_count(NV, 0), 16>(a, base, nvalid, lane);
+  rs_step<T, NV, rs_count(NV, 1), 8>(a, base, nvalid, lane);
+  rs_step<T, NV, rs_count(NV, 2), 4>(a, base, nvalid, lane);
+  rs_step<T, NV, rs_count(NV, 3), 2>(a, base, nvalid, lane);
+  rs_step<T, NV, rs_count(NV, 4), 1>(a, base, nvalid, lane);
+}
+
 // Block sum of NV per-thread values, written to part[i * stride + slot].
 // The warp stage sums in T (FP32 in the FP32 path) by a butterfly
 // reduce-scatter (lane pairs 16, 8, 4, 2, 1 apart exchange half of their
@@ -123,12 +150,8 @@ __device__ __forceinline__ void block_sum_store(const T (&v)[NV], double* part, 
   T a[NV];
 #pragma unroll
   for (int i = 0; i < NV; ++i) a[i] = v[i];
-  int base = 0, nvalid = NV;
-  rs_step<T, NV, rs_count(NV, 0), 16>(a, base, nvalid, lane);
-  rs_step<T, NV, rs_count(NV, 1), 8>(a, base, nvalid, lane);
-  rs_step<T, NV, rs_count(NV, 2), 4>(a, base, nvalid, lane);
-  rs_step<T, NV, rs_count(NV, 3), 2>(a, base, nvalid, lane);
-  rs_step<T, NV, rs_count(NV, 4), 1>(a, base, nvalid, lane);
+  int base, nvalid;
+  warp_reduce_scatter<T, NV>(a, base, nvalid, lane);
   constexpr int K5 = rs_count(NV, 5);
 #pragma unroll
   for (int i = 0; i < K5; ++i)

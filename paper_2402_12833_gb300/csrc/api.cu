@@ -129,7 +129,7 @@ struct Solver {
   DevState* state = nullptr;
   double *part_res = nullptr, *part_W = nullptr, *part_G = nullptr, *part_r = nullptr;
   double* small_scratch = nullptr;   // reduced values of the small solves
-  unsigned* counters = nullptr;      // last-block counters of small_beta / small_alpha
+  unsigned* counters = nullptr;      // last-block counters of small_beta / small_alpha, and the loop condition's
   int* flag = nullptr;               // "some problem still running" (batched loop condition)
   int* kdone = nullptr;              // gathered (iterations, done) per problem
   double *res_hist = nullptr, *alpha_hist = nullptr;
@@ -245,7 +245,7 @@ struct mg_hierarchy {
   cudaStream_t stream = 0;
   cudaStream_t cap_stream = nullptr;
   cudaStream_t side[kMaxLevels] = {};   // branches of the MG chain: fine smoothing, one per coarse grid
-  cudaEvent_t ev_fork = nullptr, ev_fine = nullptr;
+  cudaEvent_t ev_fork = nullptr, ev_fine = nullptr, ev_inv = nullptr;
   cudaEvent_t ev_r[kMaxLevels] = {}, ev_sm[kMaxLevels] = {};
   double* A0inv = nullptr;
   Level lev[kMaxLevels];
@@ -386,7 +386,7 @@ mpcg_status build_solver(mg_hierarchy* h, Solver<T>& S) {
   CKS(S.mem.get(&S.part_G, nb * (C * (C + 1) / 2 + C) * sbc, s));
   CKS(S.mem.get(&S.part_r, nb * sbc, s));
   CKS(S.mem.get(&S.small_scratch, nb * kSmallScratch, s));
-  CKS(S.mem.get(&S.counters, 2 * nb, s));
+  CKS(S.mem.get(&S.counters, 2 * nb + 1, s));
   CKS(S.mem.get(&S.flag, 1, s));
   CKS(S.mem.get(&S.kdone, 2 * nb, s));
   S.built = true;
@@ -549,51 +549,50 @@ void enqueue_mg(mg_hierarchy* h, Solver<T>& S, const T* r, T* Z, const DevState*
   cudaStreamWaitEvent(s2, h->ev_fork, 0);
   enqueue_smooth<T>(h, S, J, r, Z + (size_t)J * h->lev[J].g.cp, state, s2);
   cudaEventRecord(h->ev_fine, s2);
+  GridDesc gs[kMaxLevels];
+  for (int j = 0; j <= J; ++j) gs[j] = h->lev[j].g;
   // grids of at most kTailPoints padded points (scalar unknowns, two sweeps)
   // go through one single-block launch: their restrictions, smoothings and
   // the coarse solve are latency-bound as separate launches
   int jt = -1;
   if (h->lev[0].g.ncomp == 1 && h->opt.nu == 2 && h->opt.smoother == MPCG_SMOOTHER_JACOBI)
-    for (int j = 0; j < J; ++j)
-      if (h->lev[j].g.npts <= kTailPoints) jt = j;
+    jt = tail_finest(gs, J);
   const T* rj = r;
-  for (int j = J; j >= (jt >= 0 ? jt + 2 : 1); --j) {
-    LAUNCH(h, K_RESTRICT, s, launch_restrict<T>(h->lev[j].g, h->lev[j - 1].g, rj, S.rlev[j - 1], state, s));
-    rj = S.rlev[j - 1];
-    if (j - 1 >= 1) {   // smoothing of grid j-1 can start now, on its own branch
-      cudaStream_t s3 = h->prof.on ? s : h->side[j - 1];
-      cudaEventRecord(h->ev_r[j - 1], s);
-      cudaStreamWaitEvent(s3, h->ev_r[j - 1], 0);
-      enqueue_smooth<T>(h, S, j - 1, S.rlev[j - 1], S.zc[j - 1] + (size_t)(j - 1) * h->lev[j - 1].g.cp, state, s3);
-      cudaEventRecord(h->ev_sm[j - 1], s3);
+  const int last = jt >= 0 ? jt + 1 : 0;   // coarsest grid of the restriction chain before the tail
+  for (int j = J; j > last;) {
+    const int K = restrict_group(h->dim, j - last);
+    LAUNCH(h, K_RESTRICT, s, launch_restrict_chain<T>(gs, j, K, rj, S.rlev, state, s));
+    for (int k = j - 1; k >= j - K && k >= 1; --k) {   // smoothing of grid k can start now, on its own branch
+      cudaStream_t s3 = h->prof.on ? s : h->side[k];
+      cudaEventRecord(h->ev_r[k], s);
+      cudaStreamWaitEvent(s3, h->ev_r[k], 0);
+      enqueue_smooth<T>(h, S, k, S.rlev[k], S.zc[k] + (size_t)k * h->lev[k].g.cp, state, s3);
+      cudaEventRecord(h->ev_sm[k], s3);
     }
+    j -= K;
+    rj = S.rlev[j];
   }
   if (jt >= 0) {
-    GridDesc tg[kMaxLevels];
     const T* tst[kMaxLevels];
     const T* tdi[kMaxLevels];
-    T* tr[kMaxLevels];
     T* tz[kMaxLevels];
     for (int j = 0; j <= jt + 1; ++j) {
-      tg[j] = h->lev[j].g;
       tst[j] = st_of<T>(h->lev[j]);
       tdi[j] = dinv_of<T>(h->lev[j]);
-      tr[j] = j <= jt ? S.rlev[j] : nullptr;
       tz[j] = j <= jt ? S.zc[j] + (size_t)j * h->lev[j].g.cp : nullptr;
     }
-    LAUNCH(h, K_COARSE, s, launch_coarse_tail<T>(jt, tg, tst, tdi, tr, tz, rj, h->A0inv, state, s));
-  } else {
+    LAUNCH(h, K_COARSE, s, launch_coarse_tail<T>(jt, gs, tst, tdi, tz, S.rlev[0], rj, h->A0inv, state, s));
+  }
+  if (jt < 0 || gs[0].n > kTailCoarse) {
     LAUNCH(h, K_COARSE, s, launch_coarse_solve<T>(h->lev[0].g, h->A0inv, S.rlev[0], S.zc[0], state, s));
   }
   // every grid's correction straight to the fine grid in one launch
   const T* src[kMaxLevels];
-  GridDesc gcs[kMaxLevels];
   for (int j = 0; j < J; ++j) {
     if (j >= 1 && j > jt) cudaStreamWaitEvent(s, h->ev_sm[j], 0);
     src[j] = S.zc[j] + (size_t)j * h->lev[j].g.cp;
-    gcs[j] = h->lev[j].g;
   }
-  LAUNCH(h, K_PROLONG, s, launch_prolong_all<T>(h->lev[J].g, src, gcs, J, Z, state, s));
+  LAUNCH(h, K_PROLONG, s, launch_prolong_all<T>(h->lev[J].g, src, gs, J, Z, state, s));
   cudaStreamWaitEvent(s, h->ev_fine, 0);
 }
 
@@ -743,7 +742,9 @@ void enqueue_vcycle(mg_hierarchy* h, Solver<T>& S, const T* r, T* out, const Dev
 }
 
 template <typename T>
-void enqueue_any(mg_hierarchy* h, Solver<T>& S, cudaGraphConditionalHandle cond, int use_cond, cudaStream_t s);
+LoopCond loop_cond(const mg_hierarchy* h, const Solver<T>& S, cudaGraphConditionalHandle cond, int use_cond) {
+  return LoopCond{cond, use_cond, S.flag, S.counters + 2 * (size_t)h->nb};
+}
 
 template <typename T>
 void enqueue_prologue(mg_hierarchy* h, Solver<T>& S, cudaGraphConditionalHandle cond, int use_cond,
@@ -753,18 +754,8 @@ void enqueue_prologue(mg_hierarchy* h, Solver<T>& S, cudaGraphConditionalHandle 
   // the FP64 iterate was packed with its nonzero flag (a zero x0 skips the stencil)
   const int* xnz = std::is_same<T, float>::value ? nullptr : h->xnz;
   if (!S.zero_start) LAUNCH(h, K_RESIDUAL, s, launch_fine_residual<T>(h, S.b, S.x, S.r, S.part_res, s, xnz));
-  // a batch decides its loop condition from all problems (enqueue_any)
-  LAUNCH(h, K_INIT, s, launch_init(S.state, h->nb, S.part_res, stream_blocks(L.g), S.res_hist, S.hist_cap, cond,
-                                   use_cond && h->nb == 1, s));
-  enqueue_any<T>(h, S, cond, use_cond, s);
-}
-
-// Batched graphs: the loop runs while any problem of the batch runs.
-template <typename T>
-void enqueue_any(mg_hierarchy* h, Solver<T>& S, cudaGraphConditionalHandle cond, int use_cond, cudaStream_t s) {
-  if (h->nb == 1) return;
-  LAUNCH(h, K_CHECK, s, launch_any_running(S.state, h->nb, S.flag, s));
-  if (use_cond) LAUNCH(h, K_CHECK, s, launch_set_cond(S.flag, cond, s));
+  LAUNCH(h, K_INIT, s, launch_init(S.state, h->nb, S.part_res, stream_blocks(L.g), S.res_hist, S.hist_cap,
+                                   loop_cond(h, S, cond, use_cond), s));
 }
 
 // A P of the block being built (the ring slot after the newest).
@@ -821,10 +812,16 @@ void enqueue_body(mg_hierarchy* h, Solver<T>& S, cudaGraphConditionalHandle cond
   LAUNCH(h, K_OGRAM, s, launch_block_gram<T>(L.g, S.win, S.r, C, S.part_G, S.state, s));
   LAUNCH(h, K_ALPHA, s, launch_small_alpha(S.state, h->nb, S.part_G, stream_blocks(L.g), C, S.alpha_hist,
                                           (long long)S.hist_cap * C, S.small_scratch, S.counters, s));
+  // the new block's inverse Gram, which the next beta reads, beside the update
+  cudaStream_t si = h->prof.on ? s : h->side[0];
+  cudaEventRecord(h->ev_fork, s);
+  cudaStreamWaitEvent(si, h->ev_fork, 0);
+  LAUNCH(h, K_ALPHA, si, launch_small_inverse(S.state, h->nb, C, si));
+  cudaEventRecord(h->ev_inv, si);
   LAUNCH(h, K_UPDATE, s, launch_update_xr<T>(L.g, S.win, S.x, S.r, C, S.part_r, S.state, s));
-  LAUNCH(h, K_CHECK, s, launch_check(S.state, h->nb, S.part_r, stream_blocks(L.g), S.res_hist, S.hist_cap, cond,
-                                     use_cond && h->nb == 1, s));
-  enqueue_any<T>(h, S, cond, use_cond, s);
+  LAUNCH(h, K_CHECK, s, launch_check(S.state, h->nb, S.part_r, stream_blocks(L.g), S.res_hist, S.hist_cap,
+                                     loop_cond(h, S, cond, use_cond), s));
+  cudaStreamWaitEvent(s, h->ev_inv, 0);
 }
 
 // Capture prologue + while(cond){body} as one graph.  On any failure the
@@ -1058,6 +1055,7 @@ mpcg_status check_options(const mpcg_options& opt) {
 mpcg_status create_streams(mg_hierarchy* h) {
   bool ev_ok = cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming) == cudaSuccess &&
                cudaEventCreateWithFlags(&h->ev_fine, cudaEventDisableTiming) == cudaSuccess &&
+               cudaEventCreateWithFlags(&h->ev_inv, cudaEventDisableTiming) == cudaSuccess &&
                cudaStreamCreateWithFlags(&h->side[0], cudaStreamNonBlocking) == cudaSuccess;
   for (int j = 1; j < h->levels && ev_ok; ++j)
     ev_ok = cudaStreamCreateWithFlags(&h->side[j], cudaStreamNonBlocking) == cudaSuccess;
@@ -1154,6 +1152,7 @@ void mg_hierarchy_destroy(mg_hierarchy* h) {
     if (sd) cudaStreamDestroy(sd);
   if (h->ev_fork) cudaEventDestroy(h->ev_fork);
   if (h->ev_fine) cudaEventDestroy(h->ev_fine);
+  if (h->ev_inv) cudaEventDestroy(h->ev_inv);
   for (int j = 0; j < kMaxLevels; ++j) {
     if (h->ev_r[j]) cudaEventDestroy(h->ev_r[j]);
     if (h->ev_sm[j]) cudaEventDestroy(h->ev_sm[j]);

@@ -215,6 +215,11 @@ struct DevState {
   double tau;
   double zpz[kMaxCols];   // z_b^T A z_b less p_b^T A p_b of the new block: sum_j (W_j^T beta_j)_bb
   double alpha[kMaxCols];
+  // Cholesky factor of the scaled Gram of the newest block, left by the step
+  // length for the launch that forms its inverse (gpend = 1): the factor L,
+  // 1 / L_kk, the scaling and the column of every active position
+  int gpend, gna, gmap[kMaxCols];
+  double gL[kMaxCols][kMaxCols], gdinv[kMaxCols], gscale[kMaxCols];
   double beta[kMaxWindow][kMaxCols][kMaxCols];
   double gpinv[kMaxWindow][kMaxCols][kMaxCols];
 };

@@ -11,6 +11,8 @@ namespace mpcg {
 // partial-sum buffers are sized for it.
 constexpr int kRedBlocks = 1216;         // 152 SMs x 8 (stencil kernels with partial sums)
 constexpr int kTailPoints = 512;      // grids this small go through the single-block MG tail
+constexpr int kTailThreads = 768;     // ... as far as one thread per padded point allows
+constexpr int kTailCoarse = 32;       // the tail solves a coarsest grid of at most this many unknowns itself
 constexpr int kStreamBlocks = 608;       // 152 SMs x 4 (streaming block kernels)
 constexpr int kStreamBlocksMax = 8192;
 constexpr int kGramChunksMax = 4096;
@@ -109,6 +111,12 @@ void launch_residual(const GridDesc& g, const T* st, const T* b, const T* x, T* 
 template <typename T>
 void launch_restrict(const GridDesc& gf, const GridDesc& gc, const T* rf, T* rc,
                      const DevState* state, cudaStream_t s);
+// rlev[j - 1] .. rlev[j - K] from rf on grid j in one launch, K restrictions as
+// restrict_group gives it for the number still to do
+int restrict_group(int dim, int left);
+template <typename T>
+void launch_restrict_chain(const GridDesc* gs, int j, int K, const T* rf, T* const* rlev, const DevState* state,
+                           cudaStream_t s);
 // damped Jacobi: mode 0: out = dinv r; mode 1: two sweeps from zero;
 // mode 2: out = sin + dinv (r - A sin)
 template <typename T>
@@ -142,11 +150,14 @@ void launch_vblock(const GridDesc& g, const T* dinv, const T* t, const T* sin, T
 template <typename T>
 void launch_sum_columns(const GridDesc& g, const T* Zc, int ncols, T* out, const DevState* state, cudaStream_t s);
 // The small-grid tail of the MG chain in one block (scalar unknowns, nu = 2):
-// restrictions from grid jt + 1 (residual rin) down to 0 into r[j], Jacobi
-// smoothing of grids 1 .. jt into z[j], coarse solve into z[0].
+// restrictions from grid jt + 1 (residual rin) down to 0, Jacobi smoothing of
+// grids 1 .. jt into z[j], coarse solve into z[0] (left to launch_coarse_solve,
+// from r0, when grid 0 has more than kTailCoarse unknowns).  tail_finest: the
+// finest grid jt of the tail among grids 0 .. J - 1, or -1.
+int tail_finest(const GridDesc* g, int J);
 template <typename T>
-void launch_coarse_tail(int jt, const GridDesc* g, const T* const* st, const T* const* dinv, T* const* r,
-                        T* const* z, const T* rin, const double* a0inv, const DevState* state, cudaStream_t s);
+void launch_coarse_tail(int jt, const GridDesc* g, const T* const* st, const T* const* dinv, T* const* z, T* r0,
+                        const T* rin, const double* a0inv, const DevState* state, cudaStream_t s);
 // Z columns 0 .. J-1 on the fine grid gf from grid j's correction coarse[j]
 // (grid descriptor gcs[j]) by the composite multilinear interpolation.
 template <typename T>
@@ -211,8 +222,18 @@ void launch_jacobi_mf(const GridDesc& g, const float* k32, const float* dinv, co
                       const DevState* state, cudaStream_t s);
 
 // ---- small.cu ------------------------------------------------------------
+// The loop condition that k_init and k_check set: the graph's conditional
+// handle (use = 1; otherwise the host decides), and for batches the flag "some
+// problem still runs" and the ticket of the last block (both zero between
+// launches).
+struct LoopCond {
+  cudaGraphConditionalHandle cond;
+  int use;
+  int* flag;
+  unsigned* ticket;
+};
 void launch_init(DevState* st, int nb, const double* part_res, int nblk, double* res_hist, long long hist_stride,
-                 cudaGraphConditionalHandle cond, int use_cond, cudaStream_t s);
+                 LoopCond lc, cudaStream_t s);
 // The small solves reduce their partial sums with kSmallGrid blocks; the last
 // block to finish (atomic counter, zero between launches) does the solve.
 // scratch holds the reduced values (>= m C^2 + C^2 + 3C doubles).
@@ -223,13 +244,12 @@ void launch_small_beta(DevState* st, int nb, const double* part_W, GramShape sha
                        unsigned* counter, cudaStream_t s);
 void launch_small_alpha(DevState* st, int nb, const double* part_G, int nblk_G, int C, double* alpha_hist,
                         long long ahist_stride, double* scratch, unsigned* counter, cudaStream_t s);
+// the inverse Gram of the newest block from the factor small_alpha left
+void launch_small_inverse(DevState* st, int nb, int C, cudaStream_t s);
 void launch_check(DevState* st, int nb, const double* part_r, int nblk, double* res_hist, long long hist_stride,
-                  cudaGraphConditionalHandle cond, int use_cond, cudaStream_t s);
+                  LoopCond lc, cudaStream_t s);
 void launch_set_params(DevState* st, int nb, double rtol, int maxit, int m, int C, double delta, double tau,
                        cudaStream_t s);
-// batched graphs: flag |= any problem running; then cond = flag, flag = 0
-void launch_any_running(const DevState* st, int nb, int* flag, cudaStream_t s);
-void launch_set_cond(int* flag, cudaGraphConditionalHandle cond, cudaStream_t s);
 void launch_gather_kd(const DevState* st, int nb, int* out, cudaStream_t s);
 // Cholesky of the dense coarsest matrix (in place, lower); info[0] = 0 or the
 // failing pivot + 1

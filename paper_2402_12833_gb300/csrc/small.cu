@@ -210,35 +210,6 @@ __global__ void k_set_params(DevState* st, double rtol, int maxit, int m, int C,
   st->tau = tau;
 }
 
-__global__ void k_init(DevState* st, const double* part_res, int nblk, double* res_hist, long long hist_stride,
-                       cudaGraphConditionalHandle cond, int use_cond) {
-  __shared__ double v[2];
-  const int pb = blockIdx.x;
-  st += pb;
-  part_res += (long long)pb * 2 * nblk;
-  if (res_hist) res_hist += pb * hist_stride;
-  reduce_values(part_res, 2, nblk, nblk, v);
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    st->k = 0;
-    st->count = 0;
-    st->newest = st->m - 1;
-    st->dropped_total = 0;
-    st->pinv_fallbacks = 0;
-    st->rnorm = sqrt(v[0]);
-    st->bnorm = sqrt(v[1]);
-    int done = 0;
-    // a non-finite b or x_0 is a breakdown, tested first: with b infinite,
-    // ||r|| <= rtol ||b|| reads inf <= inf and would pass as converged
-    if (!isfinite(st->rnorm) || !isfinite(st->bnorm)) done = 3;
-    else if (st->bnorm == 0.0 || st->rnorm <= st->rtol * st->bnorm) done = 1;
-    else if (st->maxit <= 0) done = 2;
-    st->done = done;
-    if (res_hist) res_hist[0] = st->bnorm > 0.0 ? st->rnorm / st->bnorm : 0.0;
-    if (use_cond) cudaGraphSetConditional(cond, done == 0 ? 1u : 0u);
-  }
-}
-
 // beta_j = G_j^+ W_j for the window blocks: the W partial sums are reduced by
 // all blocks of the grid, the last block forms beta, and the energy
 // zpz_b = sum_j (W_j^T beta_j)_bb that the orthogonalisation removes from
@@ -287,16 +258,20 @@ __global__ void k_small_beta(DevState* st, const double* part_W, GramShape shape
 // reduced Gram values ((0,0), (0,1), ..., (0,C-1), (1,1), ...).
 __device__ __forceinline__ int tri_index(int a, int b, int C) { return a * C - a * (a - 1) / 2 + (b - a); }
 
-// alpha = G^+ g after the grid reduction of G = P^T A P and g = P^T r of
-// the new block; G^+ also goes to the window ring.  One warp,
-// C columns known at compile time.  GB300 issues one FP64 warp instruction
-// per 64 cycles per SM sub-partition whatever the active lanes, so the
-// factorisation keeps one row per lane in registers and every step is a
-// handful of warp-wide instructions: the drop rule and the scaling are one
-// pass over the lanes; the Cholesky factor of D G D (right-looking, lane i
-// holds row i); the columns of L^{-1} by forward substitution (lane j holds
-// column j), whose squares give trace((D G D)^{-1}) for the cut test; and
-// row i of (D G D)^{-1} = L^{-T} (L^{-1} e_i) by backward substitution.
+// alpha = G^+ g after the grid reduction of G = P^T A P and g = P^T r of the
+// new block.  One warp, C columns known at compile time.  GB300 issues one
+// FP64 warp instruction per 64 cycles per SM sub-partition whatever the active
+// lanes, so the instruction count on the way to alpha is what costs: the
+// Cholesky factor of D G D (right-looking, lane i holds row i) with D g as one
+// more row, which makes L^{-1} D g along the way, and a back substitution, 2
+// instructions a column.  The inverse (P^T A P)^+, which only the next block's
+// beta reads, is left to k_small_inverse beside the update of x and r.
+// det(D G D) = prod L_kk^2 certifies the cut: the trace is n, so lambda_min >=
+// det ((n - 1) / n)^(n - 1) > det / e and lambda_max <= n, and det > 3 tau n
+// keeps every eigenvalue.  Where that fails, the inverse is formed here: its
+// trace gives the sharper certificate, and the eigenvalue method follows.
+// (Event-timed launch with its reduction: C = 9 22.5 -> 16.4 us, C = 6 16.4 ->
+// 12.3 us; the inverse beside the update takes 12.3 and 8.2 us.)
 template <int C>
 __global__ void __launch_bounds__(kBlock) k_small_alpha(DevState* st, const double* part_G, int nblk_G,
                                                         double* alpha_hist, long long ahist_stride, double* scratch,
@@ -352,14 +327,15 @@ __global__ void __launch_bounds__(kBlock) k_small_alpha(DevState* st, const doub
 #pragma unroll
   for (int j = 0; j < C; ++j) Z[j] = 0.0;
   if (na > 0) {
-    // row `lane` of D G D
+    // row `lane` of D G D; lane na holds (D g)^T
     double Ar[C];
 #pragma unroll
     for (int j = 0; j < C; ++j) {
       const int cj = map[j < na ? j : 0];
       const double dj = __shfl_sync(kFull, dsc, cj);
       const int lo = ci < cj ? ci : cj, hi = ci < cj ? cj : ci;
-      Ar[j] = (lane < na && j < na) ? di * red[tri_index(lo, hi, C)] * dj : 0.0;
+      Ar[j] = 0.0;
+      if (j < na && lane <= na) Ar[j] = (lane < na ? di * red[tri_index(lo, hi, C)] : red[NG + cj]) * dj;
     }
     // Cholesky D G D = L L^T; dinv[k] = 1 / L_kk
     double dinv[C];
@@ -374,11 +350,59 @@ __global__ void __launch_bounds__(kBlock) k_small_alpha(DevState* st, const doub
         } else {
           const double li = rsqrt(piv);
           dinv[k] = li;
-          Ar[k] *= li;   // L_ik; lane k: L_kk = piv / sqrt(piv)
+          Ar[k] *= li;   // L_ik; lane k: L_kk = piv / sqrt(piv); lane na: (L^{-1} D g)_k
 #pragma unroll
           for (int j = k + 1; j < C; ++j)
             if (j < na) Ar[j] = fma(-Ar[k], __shfl_sync(kFull, Ar[k], j), Ar[j]);
         }
+      }
+    }
+    if (ok) {
+      double lkk = 1.0, yv = 0.0;
+#pragma unroll
+      for (int k = 0; k < C; ++k) {
+        if (lane == k && k < na) lkk = Ar[k];
+        const double yk = __shfl_sync(kFull, Ar[k], na);
+        if (lane == k && k < na) yv = yk;
+      }
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) lkk *= __shfl_xor_sync(kFull, lkk, o);   // the same value on every lane
+      if (lkk * lkk > 3.0 * st->tau * na) {   // every eigenvalue passes the cut
+        if (lane < na) {
+#pragma unroll
+          for (int j = 0; j < C; ++j) Lsm[lane][j] = Ar[j];
+        }
+        __syncwarp();
+#pragma unroll
+        for (int k = C - 1; k >= 0; --k) {
+          if (k < na) {
+            const double ak = __shfl_sync(kFull, yv * dinv[k], k);
+            if (lane < k) yv = fma(-Lsm[k][lane], ak, yv);
+            if (lane == k) yv = ak;
+          }
+        }
+        if (lane < C && !act) {
+          st->alpha[lane] = 0.0;
+          if (alpha_hist) alpha_hist[(long long)st->k * C + lane] = 0.0;
+        }
+        if (lane < na) {
+          const double al = di * yv;
+          st->alpha[ci] = al;
+          if (alpha_hist) alpha_hist[(long long)st->k * C + ci] = al;
+          st->gmap[lane] = ci;
+          st->gscale[lane] = di;
+#pragma unroll
+          for (int j = 0; j < C; ++j) st->gL[lane][j] = Ar[j];
+        }
+        if (lane == 0) {
+#pragma unroll
+          for (int k = 0; k < C; ++k) st->gdinv[k] = dinv[k];
+          st->gna = na;
+          st->gpend = 1;
+          st->newest = (st->newest + 1) % st->m;
+          if (st->count < st->m) st->count += 1;
+        }
+        return;
       }
     }
     if (ok) {
@@ -466,47 +490,146 @@ __global__ void __launch_bounds__(kBlock) k_small_alpha(DevState* st, const doub
   }
   __syncwarp();
   if (lane == 0) {
+    st->gpend = 0;
     st->newest = ns;
     if (st->count < st->m) st->count += 1;
   }
 }
 
+// G^+ = D L^{-T} L^{-1} D of the newest block on its active columns (zero rows
+// and columns for dropped ones) into the window ring, from the factor that
+// k_small_alpha left.  One warp per problem, on a side branch: only the next
+// block's beta waits for it.  Lane j holds column j of L^{-1}, then row j of
+// the inverse.
+template <int C>
+__global__ void __launch_bounds__(32) k_small_inverse(DevState* st) {
+  st += blockIdx.x;
+  if (!st->gpend) return;
+  __shared__ double L[C][C];
+  const int lane = threadIdx.x, na = st->gna;
+  for (int e = lane; e < C * C; e += 32) L[e / C][e % C] = st->gL[e / C][e % C];
+  const double di = lane < na ? st->gscale[lane] : 0.0;
+  const int ci = lane < na ? st->gmap[lane] : 0;
+  double dinv[C], X[C], Z[C];
+#pragma unroll
+  for (int k = 0; k < C; ++k) dinv[k] = k < na ? st->gdinv[k] : 0.0;
+  __syncwarp();
+#pragma unroll
+  for (int k = 0; k < C; ++k) {
+    X[k] = 0.0;
+    if (k < na) {
+      double s = k == lane ? 1.0 : 0.0;
+#pragma unroll
+      for (int m = 0; m < k; ++m) s = fma(-L[k][m], X[m], s);
+      X[k] = s * dinv[k];
+    }
+  }
+#pragma unroll
+  for (int k = C - 1; k >= 0; --k) {
+    Z[k] = 0.0;
+    if (k < na) {
+      double s = X[k];
+#pragma unroll
+      for (int m = k + 1; m < C; ++m)
+        if (m < na) s = fma(-L[m][k], Z[m], s);
+      Z[k] = s * dinv[k];
+    }
+  }
+  double(*gp)[kMaxCols] = st->gpinv[st->newest];
+  for (int e = lane; e < C * C; e += 32) gp[e / C][e % C] = 0.0;
+  __syncwarp();
+#pragma unroll
+  for (int j = 0; j < C; ++j) {
+    const double dj = __shfl_sync(0xffffffffu, di, j);
+    const int cj = __shfl_sync(0xffffffffu, ci, j);
+    if (lane < na && j < na) gp[ci][cj] = di * Z[j] * dj;
+  }
+}
+
+// The loop condition after every problem of the launch has decided its own
+// state (one block each): the single problem sets it; in a batch the last
+// block to finish sets it to "some problem still runs" (without a graph the
+// flag stays for the host).  flag and ticket are zero between launches.
+__device__ __forceinline__ void decide_loop(int done, const LoopCond& lc) {
+  if (gridDim.x == 1) {
+    if (lc.use) cudaGraphSetConditional(lc.cond, done == 0 ? 1u : 0u);
+    return;
+  }
+  if (done == 0) atomicOr(lc.flag, 1);
+  if (!lc.use) return;
+  __threadfence();
+  if (atomicAdd(lc.ticket, 1u) == gridDim.x - 1) {
+    *lc.ticket = 0u;
+    __threadfence();
+    cudaGraphSetConditional(lc.cond, atomicExch(lc.flag, 0) ? 1u : 0u);
+  }
+}
+
+__global__ void k_init(DevState* st, const double* part_res, int nblk, double* res_hist, long long hist_stride,
+                       LoopCond lc) {
+  __shared__ double v[2];
+  const int pb = blockIdx.x;
+  st += pb;
+  part_res += (long long)pb * 2 * nblk;
+  if (res_hist) res_hist += pb * hist_stride;
+  reduce_values(part_res, 2, nblk, nblk, v);
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    st->k = 0;
+    st->count = 0;
+    st->newest = st->m - 1;
+    st->dropped_total = 0;
+    st->pinv_fallbacks = 0;
+    st->gpend = 0;
+    st->rnorm = sqrt(v[0]);
+    st->bnorm = sqrt(v[1]);
+    int done = 0;
+    // a non-finite b or x_0 is a breakdown, tested first: with b infinite,
+    // ||r|| <= rtol ||b|| reads inf <= inf and would pass as converged
+    if (!isfinite(st->rnorm) || !isfinite(st->bnorm)) done = 3;
+    else if (st->bnorm == 0.0 || st->rnorm <= st->rtol * st->bnorm) done = 1;
+    else if (st->maxit <= 0) done = 2;
+    st->done = done;
+    if (res_hist) res_hist[0] = st->bnorm > 0.0 ? st->rnorm / st->bnorm : 0.0;
+    decide_loop(done, lc);
+  }
+}
+
+// Convergence test after the update (one block per problem; latency-bound:
+// the state is read beside the partial sums, not after them).
 __global__ void k_check(DevState* st, const double* part_r, int nblk, double* res_hist, long long hist_stride,
-                        cudaGraphConditionalHandle cond, int use_cond) {
-  __shared__ double v[1];
+                        LoopCond lc) {
   __shared__ double w[kBlock / 32];
   const int pb = blockIdx.x;
   st += pb;
   part_r += (long long)pb * nblk;
   if (res_hist) res_hist += pb * hist_stride;
-  const int was_done = st->done;
-  if (!was_done) {
-    // one value: every thread takes a strided share, then a fixed tree
-    double a = 0.0;
-    for (int b = threadIdx.x; b < nblk; b += blockDim.x) a += part_r[b];
+  const int was_done = st->done, k = st->k + 1, maxit = st->maxit;
+  const double bnorm = st->bnorm, bound = st->rtol * bnorm;
+  // one value: every thread takes a strided share, then a fixed tree
+  double a = 0.0;
+  for (int b = threadIdx.x; b < nblk; b += blockDim.x) a += part_r[b];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = a;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t += w[i];
-      v[0] = t;
-    }
-  }
+  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  if ((threadIdx.x & 31) == 0) w[threadIdx.x >> 5] = a;
   __syncthreads();
+  if (threadIdx.x >= 32) return;
+  double t = threadIdx.x < kBlock / 32 ? w[threadIdx.x] : 0.0;
+#pragma unroll
+  for (int o = kBlock / 64; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
   if (threadIdx.x == 0) {
     int done = was_done;
     if (!was_done) {
-      st->k += 1;
-      st->rnorm = sqrt(v[0]);
-      if (res_hist) res_hist[st->k] = st->rnorm / st->bnorm;
-      if (!isfinite(st->rnorm)) done = 3;
-      else if (st->rnorm <= st->rtol * st->bnorm) done = 1;
-      else if (st->k >= st->maxit) done = 2;
+      const double rnorm = sqrt(t);
+      if (!isfinite(rnorm)) done = 3;
+      else if (rnorm <= bound) done = 1;
+      else if (k >= maxit) done = 2;
+      st->k = k;
+      st->rnorm = rnorm;
       st->done = done;
+      if (res_hist) res_hist[k] = rnorm / bnorm;
     }
-    if (use_cond) cudaGraphSetConditional(cond, done == 0 ? 1u : 0u);
+    decide_loop(done, lc);
   }
 }
 
@@ -622,7 +745,6 @@ __global__ void k_sum_partials(const double* part, int nv, int nblk, double* out
   reduce_values(part + (long long)pb * nv * nblk, nv, nblk, nblk, out + (long long)pb * nv);
 }
 
-// flag |= some problem of the batch is still running.
 // Device side of the mixed-precision refinement loop (one graph per solve):
 // mix[p] = {inner iterations so far, status (0 running, 1 converged, 2 out
 // of iterations or steps, 3 breakdown), active}.
@@ -688,23 +810,12 @@ __global__ void k_outer_accumulate(int* mix, int nb, const DevState* st) {
   }
 }
 
-__global__ void k_any_running(const DevState* st, int nb, int* flag) {
-  for (int b = threadIdx.x; b < nb; b += blockDim.x)
-    if (st[b].done == 0) atomicOr(flag, 1);
-}
-
 // out[2b] = iterations, out[2b+1] = done of problem b.
 __global__ void k_gather_kd(const DevState* st, int nb, int* out) {
   for (int b = threadIdx.x + blockIdx.x * blockDim.x; b < nb; b += blockDim.x * gridDim.x) {
     out[2 * b] = st[b].k;
     out[2 * b + 1] = st[b].done;
   }
-}
-
-// The loop condition of a batched graph: continue while any problem runs.
-__global__ void k_set_cond(int* flag, cudaGraphConditionalHandle cond) {
-  cudaGraphSetConditional(cond, *flag ? 1u : 0u);
-  *flag = 0;
 }
 
 }  // namespace
@@ -714,8 +825,8 @@ void launch_set_params(DevState* st, int nb, double rtol, int maxit, int m, int 
   k_set_params<<<nb, 1, 0, s>>>(st, rtol, maxit, m, C, delta, tau);
 }
 void launch_init(DevState* st, int nb, const double* part_res, int nblk, double* res_hist, long long hist_stride,
-                 cudaGraphConditionalHandle cond, int use_cond, cudaStream_t s) {
-  k_init<<<nb, kBlock, 0, s>>>(st, part_res, nblk, res_hist, hist_stride, cond, use_cond);
+                 LoopCond lc, cudaStream_t s) {
+  k_init<<<nb, kBlock, 0, s>>>(st, part_res, nblk, res_hist, hist_stride, lc);
 }
 void launch_small_beta(DevState* st, int nb, const double* part_W, GramShape shape, int C, double* scratch,
                        unsigned* counter, cudaStream_t s) {
@@ -726,9 +837,12 @@ void launch_small_alpha(DevState* st, int nb, const double* part_G, int nblk_G, 
   MPCG_SMALL_C_SWITCH(C, (k_small_alpha<CC><<<dim3(kSmallGrid, nb), kBlock, 0, s>>>(
                              st, part_G, nblk_G, alpha_hist, ahist_stride, scratch, counter)));
 }
+void launch_small_inverse(DevState* st, int nb, int C, cudaStream_t s) {
+  MPCG_SMALL_C_SWITCH(C, (k_small_inverse<CC><<<nb, 32, 0, s>>>(st)));
+}
 void launch_check(DevState* st, int nb, const double* part_r, int nblk, double* res_hist, long long hist_stride,
-                  cudaGraphConditionalHandle cond, int use_cond, cudaStream_t s) {
-  k_check<<<nb, kBlock, 0, s>>>(st, part_r, nblk, res_hist, hist_stride, cond, use_cond);
+                  LoopCond lc, cudaStream_t s) {
+  k_check<<<nb, kBlock, 0, s>>>(st, part_r, nblk, res_hist, hist_stride, lc);
 }
 void launch_dense_from_stencil(const GridDesc& g, const double* st, double* dense, cudaStream_t s) {
   k_dense_from_stencil<<<(int)((g.n + 127) / 128), 128, 0, s>>>(g, st, dense);
@@ -764,12 +878,6 @@ void launch_outer_accumulate(int* mix, int nb, const DevState* st, cudaStream_t 
 }
 void launch_sum_partials(const double* part, int nb, int nv, int nblk, double* out, cudaStream_t s) {
   k_sum_partials<<<nb, kBlock, 0, s>>>(part, nv, nblk, out);
-}
-void launch_any_running(const DevState* st, int nb, int* flag, cudaStream_t s) {
-  k_any_running<<<1, kBlock, 0, s>>>(st, nb, flag);
-}
-void launch_set_cond(int* flag, cudaGraphConditionalHandle cond, cudaStream_t s) {
-  k_set_cond<<<1, 1, 0, s>>>(flag, cond);
 }
 void launch_gather_kd(const DevState* st, int nb, int* out, cudaStream_t s) {
   k_gather_kd<<<(nb + kBlock - 1) / kBlock, kBlock, 0, s>>>(st, nb, out);

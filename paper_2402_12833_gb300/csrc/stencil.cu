@@ -302,6 +302,89 @@ __global__ void __launch_bounds__(kBlock) k_restrict(GridDesc gf, GridDesc gc, c
   rc[idc] = acc;
 }
 
+// K restrictions of a 2D grid in one launch, g[0] -> g[1] -> ... -> g[K]: a
+// block owns a tile of TC x TC points of g[K] and forms it from its own cone
+// of finer points (2 n + 1 points per axis of the next finer grid for n), held
+// in shared memory; points of the grids in between that two cones share are
+// computed twice and stored by the block whose tile they lie over.  The chain
+// is bound by the latency of its launches (6-7 us each on grids below 10^6
+// points), so the cones' repeated reads cost less than the launches they save:
+// 1025^2 -> 33^2 in two launches of 10 + 9 us instead of five of 33 us, 257^2 ->
+// 33^2 in one of 10 us instead of three of 20 us (serialised, event-timed).  In
+// 3D two levels share 2.6 times the source and gained nothing (129^3: 12.2
+// against 12.3 us; 65^3 x 3 lost, 25.6 against 13.6 us).  The sums are those of
+// k_restrict, bit for bit.
+template <typename T, int K>
+struct RestrictArgs {
+  GridDesc g[K + 1];
+  const T* rf;
+  T* rc[K];        // residuals of g[1] .. g[K]
+};
+
+// points per axis of the cone `up` grids above tc points, and the first
+// element of the region of g[k] among the K regions held in shared memory
+constexpr int cone(int tc, int up) { return up == 0 ? tc : 2 * cone(tc, up - 1) + 1; }
+template <int K, int TC>
+constexpr int cone_offset(int k) {
+  return k == 0 ? 0 : cone_offset<K, TC>(k - 1) + cone(TC, K - k + 1) * cone(TC, K - k + 1);
+}
+
+template <typename T, int K, int TC, int KK>
+__device__ __forceinline__ void restrict_step(const RestrictArgs<T, K>& a, T* buf, int tx, int ty, bool lastx,
+                                              bool lasty, int pb) {
+  constexpr int n = cone(TC, K - KK), nf = 2 * n + 1, up = K - KK;
+  const GridDesc& g = a.g[KK];
+  const T* src = buf + cone_offset<K, TC>(KK - 1);
+  T* dst = buf + (KK < K ? cone_offset<K, TC>(KK) : 0);
+  T* out = a.rc[KK - 1] + (long long)pb * g.len + g.G;
+  // the tile's points of g[KK]; the region starts (1 - lo) (2^up - 1) before them
+  const int ox = tx * TC << up, oy = ty * TC << up;
+  for (int e = threadIdx.x; e < n * n; e += blockDim.x) {
+    const int lx = e % n, ly = e / n;
+    const int x = ox - (1 - g.lox) * ((1 << up) - 1) + lx, y = oy - (1 - g.loy) * ((1 << up) - 1) + ly;
+    T acc = 0;
+    if (x >= 0 && x < g.nx && y >= 0 && y < g.ny) {
+      const T* p = src + (2 * lx + 1) + nf * (2 * ly + 1);
+#pragma unroll
+      for (int ey = -1; ey <= 1; ++ey)
+#pragma unroll
+        for (int ex = -1; ex <= 1; ++ex) {
+          const T w = (T)((ex ? 0.5f : 1.f) * (ey ? 0.5f : 1.f));
+          acc = fma(w, p[ex + nf * ey], acc);
+        }
+      if (x >= ox && (lastx || x < ox + (TC << up)) && y >= oy && (lasty || y < oy + (TC << up)))
+        out[x + (long long)g.px * y] = acc;
+    }
+    if (KK < K) dst[e] = acc;
+  }
+  __syncthreads();
+  if constexpr (KK < K) restrict_step<T, K, TC, KK + 1>(a, buf, tx, ty, lastx, lasty, pb);
+}
+
+template <typename T, int K, int TC>
+__global__ void __launch_bounds__(kBlock) k_restrict_multi(RestrictArgs<T, K> a, int ntx, int nty,
+                                                           const DevState* state) {
+  const int pb = blockIdx.y;
+  if (state && state[pb].done) return;
+  __shared__ T buf[cone_offset<K, TC>(K)];
+  constexpr int n = cone(TC, K);
+  const int tx = blockIdx.x % ntx, ty = blockIdx.x / ntx;
+  const GridDesc& g = a.g[0];
+  const T* rf = a.rf + (long long)pb * g.len + g.G;
+  const int x0 = (tx * TC << K) - (1 - g.lox) * ((1 << K) - 1), y0 = (ty * TC << K) - (1 - g.loy) * ((1 << K) - 1);
+  const int lane = threadIdx.x & 31;
+  for (int row = threadIdx.x >> 5; row < n; row += kBlock / 32) {   // a warp per row of the region
+    const int y = y0 + row;
+    const T* p = rf + (long long)g.px * y;
+    for (int l = lane; l < n; l += 32) {
+      const int x = x0 + l;
+      buf[row * n + l] = y >= 0 && y < g.ny && x >= 0 && x < g.nx ? p[x] : T(0);
+    }
+  }
+  __syncthreads();
+  restrict_step<T, K, TC, 1>(a, buf, tx, ty, tx == ntx - 1, ty == nty - 1, pb);
+}
+
 // Damped Jacobi (Eq. 2 with M = D / omega, dinv = omega / diag), c_0 = 0:
 //   mode 0: out = dinv r                          (one sweep)
 //   mode 1: out = s1 + dinv (r - A s1), s1 = dinv r  (two sweeps, s1 formed
@@ -553,83 +636,115 @@ __global__ void __launch_bounds__(kBlock) k_prolong_all(GridDesc gf, CoarseSrc<T
 // The small-grid tail of the MG chain in one block (scalar unknowns, two
 // Jacobi sweeps): the restrictions from grid jt + 1 down to grid 0, the
 // damped-Jacobi smoothing of grids 1 .. jt and the exact coarsest solve.
-// Grids this small are latency-bound as separate launches; one block of
-// 1024 threads takes them in turn with block barriers in between.
+// Bound by latency.  Every thread owns one entry (grid, point) of the padded
+// boxes of grids jt, jt - 1, ..., 0: it loads its stencil row and diagonal at
+// the start (they do not wait for the residual), computes its restricted
+// residual from the next finer grid, and all grids smooth at once at the end,
+// beside the coarse solve; between the restrictions the residuals stay in
+// shared memory.  (The form that walked the grids one after another through
+// global memory: 14.4 us at 1025^2 against 8.8 now, 14.5 against 11.5 at 129^3,
+// 23.4 against 16 there in double-word, event-timed launches.)
+// With more than kTailCoarse unknowns on grid 0 its residual goes to r0 and
+// the coarse solve is a launch of its own over many SMs: the dense FP64
+// product takes n^2 / 2 cycles of one SM's FP64 pipe (343 unknowns: 59 us; now
+// 8 + 11 us in two launches).
 template <typename T>
 struct TailArgs {
   int jt;                          // finest grid of the tail
   GridDesc g[kMaxLevels];
   const T* st[kMaxLevels];         // stencil planes of grid j
   const T* dinv[kMaxLevels];       // damped inverse diagonal of grid j
-  T* r[kMaxLevels];                // restricted residual of grid j (j <= jt)
   T* z[kMaxLevels];                // correction of grid j (grid 0: the coarse solve)
+  int off[kMaxLevels];             // start of grid j's arrays in shared memory
+  int total;                       // elements of all grids' arrays
+  T* r0;                           // restricted residual of grid 0, or null: solve here
   const T* rin;                    // residual of grid jt + 1
   const double* a0inv;             // explicit inverse of the coarsest operator
 };
 
 template <typename T, int DIM>
-__global__ void __launch_bounds__(1024) k_coarse_tail(TailArgs<T> a, const DevState* state) {
-  const int pb = blockIdx.y;
-  if (state && state[pb].done) return;
-  constexpr int S = DIM == 3 ? 27 : 9;
-  // restrictions jt + 1 -> jt -> ... -> 0
-  for (int j = a.jt; j >= 0; --j) {
-    const GridDesc& gf = a.g[j + 1];
-    const GridDesc& gc = a.g[j];
-    const T* rf = (j == a.jt ? a.rin : a.r[j + 1]) + (long long)pb * gf.len;
-    T* rc = a.r[j] + (long long)pb * gc.len;
-    for (long long t = threadIdx.x; t < gc.npts; t += blockDim.x) {
-      int X, Y, Z, c;
-      decode(gc, t, X, Y, Z, c);
-      T acc = 0;
-      if (interior(gc, X, Y, Z)) {
-        const long long pf = gf.px, pp = gf.pxy;
-        const long long idf = gf.G + (2 * X + gf.lox) + pf * (2 * Y + gf.loy) + (DIM == 3 ? pp * (2 * Z + gf.loz) : 0);
-        for (int ez = (DIM == 3 ? -1 : 0); ez <= (DIM == 3 ? 1 : 0); ++ez)
-          for (int ey = -1; ey <= 1; ++ey)
-            for (int ex = -1; ex <= 1; ++ex) {
-              const T w = (T)((ex ? 0.5f : 1.f) * (ey ? 0.5f : 1.f) * (ez ? 0.5f : 1.f));
-              acc = fma(w, rf[idf + ex + pf * ey + pp * ez], acc);
-            }
+__device__ __forceinline__ T restrict_point(const GridDesc& gf, const GridDesc& gc, const T* rf, int X, int Y, int Z) {
+  const int pf = gf.px, pp = (int)gf.pxy;
+  const T* p = rf + gf.G + (2 * X + gf.lox) + pf * (2 * Y + gf.loy) + (DIM == 3 ? pp * (2 * Z + gf.loz) : 0);
+  T acc = 0;
+#pragma unroll
+  for (int ez = (DIM == 3 ? -1 : 0); ez <= (DIM == 3 ? 1 : 0); ++ez)
+#pragma unroll
+    for (int ey = -1; ey <= 1; ++ey)
+#pragma unroll
+      for (int ex = -1; ex <= 1; ++ex) {
+        const T w = (T)((ex ? 0.5f : 1.f) * (ey ? 0.5f : 1.f) * (ez ? 0.5f : 1.f));
+        acc = fma(w, p[ex + pf * ey + pp * ez], acc);
       }
-      rc[gc.G + t] = acc;
+  return acc;
+}
+
+template <typename T, int DIM>
+__global__ void __launch_bounds__(kTailThreads) k_coarse_tail(TailArgs<T> a, const DevState* state) {
+  const int pb = blockIdx.y;
+  constexpr int S = DIM == 3 ? 27 : 9;
+  extern __shared__ __align__(16) unsigned char tail_smem[];
+  T* sr = reinterpret_cast<T*>(tail_smem);   // residuals, padded boxes with zero guards
+  T* ss = sr + a.total;                      // s1 = dinv r
+  __shared__ double y0[kTailCoarse];
+  // the entry this thread owns
+  int j = a.jt, t = threadIdx.x;
+  while (j >= 0 && t >= (int)a.g[j].npts) t -= (int)a.g[j--].npts;
+  int X = 0, Y = 0, Z = 0, comp;
+  bool in = false;
+  T c[S], di = 0;
+#pragma unroll
+  for (int s = 0; s < S; ++s) c[s] = 0;
+  if (j >= 0) {
+    decode(a.g[j], t, X, Y, Z, comp);
+    in = interior(a.g[j], X, Y, Z);
+    if (j >= 1 && in) {
+      const long long o = (long long)pb * a.g[j].len + a.g[j].G + t;
+      di = a.dinv[j][o];
+#pragma unroll
+      for (int s = 0; s < S; ++s) c[s] = a.st[j][(long long)s * a.g[j].cp + o];
+    }
+  }
+  if (state && state[pb].done) return;
+  for (int e = threadIdx.x; e < 2 * a.total; e += blockDim.x) sr[e] = 0;
+  __syncthreads();
+  // restrictions jt + 1 -> jt -> ... -> 0
+  for (int k = a.jt; k >= 0; --k) {
+    if (j == k && in) {
+      const T v = k == a.jt ? restrict_point<T, DIM>(a.g[k + 1], a.g[k], a.rin + (long long)pb * a.g[k + 1].len, X, Y, Z)
+                            : restrict_point<T, DIM>(a.g[k + 1], a.g[k], sr + a.off[k + 1], X, Y, Z);
+      const int o = a.off[k] + (int)a.g[k].G + t;
+      sr[o] = v;
+      ss[o] = di * v;
+      if (k == 0) {
+        const int i = X + a.g[0].nx * (Y + (DIM == 3 ? a.g[0].ny * Z : 0));
+        if (a.r0) a.r0[(long long)pb * a.g[0].len + a.g[0].G + t] = v;
+        else y0[i] = (double)v;
+      }
     }
     __syncthreads();
   }
   // two damped-Jacobi sweeps from zero on grids 1 .. jt (Eq. 2, c_0 = 0):
-  // out = s1 + dinv (r - A s1) with s1 = dinv r formed at the neighbours
-  for (int j = 1; j <= a.jt; ++j) {
+  // out = s1 + dinv (r - A s1)
+  if (j >= 1) {
     const GridDesc& g = a.g[j];
-    const long long bo = (long long)pb * g.len + g.G;
-    const T* st = a.st[j] + bo;
-    const T* di = a.dinv[j] + bo;
-    const T* rr = a.r[j] + bo;
-    T* out = a.z[j] + bo;
-    for (long long t = threadIdx.x; t < g.npts; t += blockDim.x) {
-      T acc = 0;
-      for (int s = 0; s < S; ++s) {
-        const long long off = (s % 3 - 1) + g.px * ((s / 3) % 3 - 1) + (DIM == 3 ? g.pxy * (s / 9 - 1) : 0);
-        acc = fma(st[(long long)s * g.cp + t], di[t + off] * rr[t + off], acc);
-      }
-      const T s1 = di[t] * rr[t];
-      out[t] = s1 + di[t] * (rr[t] - acc);
+    const int o = a.off[j] + (int)g.G + t;
+    T acc = 0;
+#pragma unroll
+    for (int s = 0; s < S; ++s) {
+      const int off = (s % 3 - 1) + g.px * ((s / 3) % 3 - 1) + (DIM == 3 ? (int)g.pxy * (s / 9 - 1) : 0);
+      acc = fma(c[s], ss[o + off], acc);
     }
+    a.z[j][(long long)pb * g.len + g.G + t] = ss[o] + di * (sr[o] - acc);
   }
   // exact coarsest solve: warp per row of the explicit inverse
-  {
-    extern __shared__ double yv[];
+  if (!a.r0) {
     const GridDesc& g = a.g[0];
-    const int n = (int)g.n;
+    const int n = (int)g.n, lane = threadIdx.x & 31;
     const double* inv = a.a0inv + (long long)pb * n * n;
-    const T* r0 = a.r[0] + (long long)pb * g.len;
     T* out = a.z[0] + (long long)pb * g.len;
-    for (int i = threadIdx.x; i < n; i += blockDim.x) yv[i] = (double)r0[padded_index(g, i)];
-    __syncthreads();
-    const int lane = threadIdx.x & 31;
     for (int i = threadIdx.x >> 5; i < n; i += blockDim.x >> 5) {
-      const double* row = inv + (long long)i * n;
-      double s = 0.0;
-      for (int k = lane; k < n; k += 32) s = fma(row[k], yv[k], s);
+      double s = lane < n ? inv[(long long)i * n + lane] * y0[lane] : 0.0;
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
       if (lane == 0) out[padded_index(g, i)] = (T)s;
@@ -1131,6 +1246,42 @@ template void launch_restrict<float>(const GridDesc&, const GridDesc&, const flo
                                      cudaStream_t);
 #endif
 
+template <typename T, int K, int TC>
+static void restrict_multi(const GridDesc* gs, int j, const T* rf, T* const* rlev, const DevState* state,
+                           cudaStream_t s) {
+  RestrictArgs<T, K> a = {};
+  a.rf = rf;
+  for (int k = 0; k <= K; ++k) a.g[k] = gs[j - k];
+  for (int k = 1; k <= K; ++k) a.rc[k - 1] = rlev[j - k];
+  const GridDesc& gc = gs[j - K];
+  const int tx = (gc.nx + TC - 1) / TC, ty = (gc.ny + TC - 1) / TC;
+  k_restrict_multi<T, K, TC><<<dim3(tx * ty, gc.nb), kBlock, 0, s>>>(a, tx, ty, state);
+}
+
+// Restrictions of the next launch when `left` are still to do: one in 3D; in
+// 2D at most three (their cones read 1.5 times the source, tile 4; two read 1.2
+// times, tile 8), the larger groups last, on the smaller grids.
+#if MPCG_STENCIL_PLAIN
+int restrict_group(int dim, int left) {
+  if (dim == 3) return 1;
+  return left <= 3 ? left : (left % 3 ? 2 : 3);
+}
+#endif
+
+template <typename T>
+void launch_restrict_chain(const GridDesc* gs, int j, int K, const T* rf, T* const* rlev, const DevState* state,
+                           cudaStream_t s) {
+  if (K == 1) launch_restrict<T>(gs[j], gs[j - 1], rf, rlev[j - 1], state, s);
+  else if (K == 2) restrict_multi<T, 2, 8>(gs, j, rf, rlev, state, s);
+  else restrict_multi<T, 3, 4>(gs, j, rf, rlev, state, s);
+}
+#if MPCG_STENCIL_PLAIN
+template void launch_restrict_chain<double>(const GridDesc*, int, int, const double*, double* const*,
+                                            const DevState*, cudaStream_t);
+template void launch_restrict_chain<float>(const GridDesc*, int, int, const float*, float* const*, const DevState*,
+                                           cudaStream_t);
+#endif
+
 template <typename T, bool SYM = false>
 static void jacobi_impl(const GridDesc& g, const T* st, const T* dinv, const T* r, const T* sin, T* out, int mode,
                         const DevState* state, cudaStream_t s) {
@@ -1229,31 +1380,51 @@ template void launch_sum_columns<double>(const GridDesc&, const double*, int, do
 template void launch_sum_columns<float>(const GridDesc&, const float*, int, float*, const DevState*, cudaStream_t);
 #endif
 
+#if MPCG_STENCIL_PLAIN
+int tail_finest(const GridDesc* g, int J) {
+  int jt = -1;
+  long long threads = 0;
+  for (int j = 0; j < J && g[j].npts <= kTailPoints; ++j) {
+    threads += g[j].npts;
+    if (threads > kTailThreads) break;
+    jt = j;
+  }
+  return jt;
+}
+#endif
+
 template <typename T>
-void launch_coarse_tail(int jt, const GridDesc* g, const T* const* st, const T* const* dinv, T* const* r,
-                        T* const* z, const T* rin, const double* a0inv, const DevState* state, cudaStream_t s) {
+void launch_coarse_tail(int jt, const GridDesc* g, const T* const* st, const T* const* dinv, T* const* z, T* r0,
+                        const T* rin, const double* a0inv, const DevState* state, cudaStream_t s) {
   TailArgs<T> a = {};
   a.jt = jt;
+  int threads = 0;
   for (int j = 0; j <= jt + 1; ++j) {
     a.g[j] = g[j];
     a.st[j] = st[j];
     a.dinv[j] = dinv[j];
-    a.r[j] = r[j];
     a.z[j] = z[j];
+    if (j <= jt) {
+      a.off[j] = a.total;
+      a.total += (int)g[j].len;
+      threads += (int)g[j].npts;
+    }
   }
+  a.r0 = g[0].n > kTailCoarse ? r0 : nullptr;
   a.rin = rin;
   a.a0inv = a0inv;
   const dim3 grid(1, g[0].nb);
-  const size_t smem = (size_t)g[0].n * sizeof(double);
-  if (g[0].dim == 3) k_coarse_tail<T, 3><<<grid, 1024, smem, s>>>(a, state);
-  else k_coarse_tail<T, 2><<<grid, 1024, smem, s>>>(a, state);
+  threads = (threads + 31) / 32 * 32;
+  const size_t smem = 2 * (size_t)a.total * sizeof(T);
+  if (g[0].dim == 3) k_coarse_tail<T, 3><<<grid, threads, smem, s>>>(a, state);
+  else k_coarse_tail<T, 2><<<grid, threads, smem, s>>>(a, state);
 }
 #if MPCG_STENCIL_PLAIN
 template void launch_coarse_tail<double>(int, const GridDesc*, const double* const*, const double* const*,
-                                         double* const*, double* const*, const double*, const double*,
-                                         const DevState*, cudaStream_t);
+                                         double* const*, double*, const double*, const double*, const DevState*,
+                                         cudaStream_t);
 template void launch_coarse_tail<float>(int, const GridDesc*, const float* const*, const float* const*,
-                                        float* const*, float* const*, const float*, const double*, const DevState*,
+                                        float* const*, float*, const float*, const double*, const DevState*,
                                         cudaStream_t);
 #endif
 
@@ -1374,6 +1545,8 @@ template void launch_spmm<dw>(const GridDesc&, const dw*, const SpmmIO<dw>&, int
 template void launch_residual<dw>(const GridDesc&, const dw*, const dw*, const dw*, dw*, double*, cudaStream_t,
                                   const int*);
 template void launch_restrict<dw>(const GridDesc&, const GridDesc&, const dw*, dw*, const DevState*, cudaStream_t);
+template void launch_restrict_chain<dw>(const GridDesc*, int, int, const dw*, dw* const*, const DevState*,
+                                        cudaStream_t);
 template void launch_jacobi<dw>(const GridDesc&, const dw*, const dw*, const dw*, const dw*, dw*, int,
                                 const DevState*, cudaStream_t);
 template void launch_vres<dw>(const GridDesc&, const dw*, const dw*, const dw*, dw*, const DevState*, cudaStream_t);
@@ -1382,8 +1555,8 @@ template void launch_vblock<dw>(const GridDesc&, const dw*, const dw*, const dw*
 template void launch_vres_block<dw>(const GridDesc&, const dw*, const dw*, const dw*, const dw*, dw*,
                                     const DevState*, cudaStream_t);
 template void launch_sum_columns<dw>(const GridDesc&, const dw*, int, dw*, const DevState*, cudaStream_t);
-template void launch_coarse_tail<dw>(int, const GridDesc*, const dw* const*, const dw* const*, dw* const*,
-                                     dw* const*, const dw*, const double*, const DevState*, cudaStream_t);
+template void launch_coarse_tail<dw>(int, const GridDesc*, const dw* const*, const dw* const*, dw* const*, dw*,
+                                     const dw*, const double*, const DevState*, cudaStream_t);
 template void launch_gs_colour<dw>(const GridDesc&, const dw*, const dw*, dw*, int, double, const DevState*,
                                    cudaStream_t);
 template void launch_defect<dw>(const GridDesc&, const dw*, const dw*, const dw*, dw*, const DevState*,

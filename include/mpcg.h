@@ -588,7 +588,7 @@ mpcg_status mg_stencil_apply_noalloc(int dim, int nodes, const double* values_de
  * problems in the batch, columns):
  *   MG_TUNE_STREAM_BLOCKS  blocks of the streaming block kernels (A-
  *                          orthogonalisation, update, residual) on a grid;
- *   MG_TUNE_SPMM_BLOCKS    blocks of the block SpMM;
+ *   MG_TUNE_SPMM_BLOCKS    blocks of the block SpMM on the full stored stencil;
  *   MG_TUNE_GRAM_CHUNKS    point chunks per window block of the window Gram;
  *   MG_TUNE_JACOBI_NARROW  1: one point per thread in the Jacobi sweep of a
  *                          grid, 0: a 16-byte vector per thread.

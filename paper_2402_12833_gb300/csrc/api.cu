@@ -771,7 +771,7 @@ void enqueue_block_spmm(mg_hierarchy* h, Solver<T>& S, cudaStream_t s) {
   const SpmmIO<T> io = spmm_ring(S.win, S.m);
   if constexpr (std::is_same<T, float>::value) {
     if (L.kq32) {   // fine operator rebuilt from the element coefficients
-      LAUNCH(h, K_SPMM, s, launch_spmm_mf(L.g, L.kq32, io, C, spmm_blocks<T>(L.g, C), S.state, s));
+      LAUNCH(h, K_SPMM, s, launch_spmm_mf(L.g, L.kq32, io, C, S.state, s));
       return;
     }
     if (L.sth32) {   // the symmetric half of the stored stencil

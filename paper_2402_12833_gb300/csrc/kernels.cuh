@@ -214,10 +214,9 @@ void launch_update_xr(const GridDesc& g, Window<T> win, T* x, T* r, int C, doubl
 mpcg_status place_kappa(const GridDesc& g, const double* kappa, int ne, double h, float* k32, double* k64,
                         unsigned long long* check, const double* st64, double* maxdiff, double* maxabs,
                         cudaStream_t s);
-// Y = A X (C <= 12 columns, nblocks blocks; false for other C) and the fused
-// two-sweep Jacobi, A rebuilt from k32 (2D / 3D scalar, FP32).
-bool launch_spmm_mf(const GridDesc& g, const float* k32, const SpmmIO<float>& io, int C, int nblocks,
-                    const DevState* state, cudaStream_t s);
+// Y = A X (C <= 12 columns; false for other C) and the fused two-sweep Jacobi, A rebuilt from k32 (2D / 3D scalar, FP32).
+bool launch_spmm_mf(const GridDesc& g, const float* k32, const SpmmIO<float>& io, int C, const DevState* state,
+                    cudaStream_t s);
 void launch_jacobi_mf(const GridDesc& g, const float* k32, const float* dinv, const float* r, float* out,
                       const DevState* state, cudaStream_t s);
 

@@ -25,6 +25,7 @@
 #include <string.h>
 
 #include "kernels.cuh"
+#include "rows.cuh"
 #include "vec.cuh"
 
 namespace mpcg {
@@ -92,294 +93,184 @@ __global__ void k_check_kappa(GridDesc g, const double* __restrict__ st, const d
   atomicMax(out + 1, (unsigned long long)__double_as_longlong(amax));
 }
 
-// Row segment v[-1 .. 4] around a group of four points: e[k] = v[k - 1].
-__device__ __forceinline__ void row6(const float* __restrict__ p, float (&e)[6]) {
-  float m[4];
-  Vec<float>::load_keep(p, m);
-  e[0] = p[-1];
-#pragma unroll
-  for (int w = 0; w < 4; ++w) e[w + 1] = m[w];
-  e[5] = p[4];
-}
-
-// k_e of the 8 elements around the points x0 .. x0+3 of a group:
-// kq[2b + c][k] for the element whose lowest node is (x0 - 1 + k, y - 1 + b,
+// k_e of the elements around the points x0 .. x0+3 of a group: kq[2b + c][k]
+// (2D: kq[b][k]) for the element whose lowest node is (x0 - 1 + k, y - 1 + b,
 // z - 1 + c).
+template <int DIM>
 __device__ __forceinline__ void load_kappa(const float* __restrict__ k32, long long idx, long long px, long long pxy,
-                                           float (&kq)[4][5]) {
+                                           float (&kq)[DIM == 3 ? 4 : 2][5]) {
 #pragma unroll
-  for (int b = 0; b < 2; ++b)
+  for (int e = 0; e < (DIM == 3 ? 4 : 2); ++e) {
+    const int b = DIM == 3 ? e >> 1 : e, c = DIM == 3 ? e & 1 : 1;
+    const float* p = k32 + idx + (long long)(b - 1) * px + (long long)(c - 1) * pxy;
+    float m[4];
+    Vec<float>::load_keep(p, m);
+    kq[e][0] = p[-1];
 #pragma unroll
-    for (int c = 0; c < 2; ++c) {
-      const float* p = k32 + idx + (long long)(b - 1) * px + (long long)(c - 1) * pxy;
-      float m[4];
-      Vec<float>::load_keep(p, m);
-      kq[2 * b + c][0] = p[-1];
-#pragma unroll
-      for (int w = 0; w < 4; ++w) kq[2 * b + c][w + 1] = m[w];
-    }
+    for (int w = 0; w < 4; ++w) kq[e][w + 1] = m[w];
+  }
 }
 
-// Coefficients of stencil row (DY, DZ) for the four points: cf[dx + 1][w].
-template <int DY, int DZ>
-__device__ __forceinline__ void row_coefs(const float (&kq)[4][5], float (&cf)[3][4]) {
-  constexpr int b = DY > 0, c = DZ > 0;
+// Coefficients of stencil row k (dy = k % 3 - 1, dz = k / 3 - 1; 2D: dy = k - 1)
+// for the group's points as sources (rows.cuh): the coupling of a point to its
+// left neighbour's column and to its right one's both come from the element
+// between them, e[w] and e[w + 1].
+template <int DIM>
+__device__ __forceinline__ void mf_row_coeffs(const float (&kq)[DIM == 3 ? 4 : 2][5], int k, float (&cl)[4],
+                                              float (&cc)[4], float (&cr)[4]) {
+  const int dy = k % 3 - 1, dz = DIM == 3 ? k / 3 - 1 : 0;
+  float e[5];
+#pragma unroll
+  for (int i = 0; i < 5; ++i) {
+    if constexpr (DIM == 3) {
+      const int b = dy > 0, c = dz > 0;
+      if (dy == 0 && dz == 0) e[i] = kq[0][i] + kq[1][i] + kq[2][i] + kq[3][i];
+      else if (dz == 0) e[i] = kq[2 * b][i] + kq[2 * b + 1][i];   // edges (+-1, dy, 0), face (0, dy, 0)
+      else if (dy == 0) e[i] = kq[c][i] + kq[2 + c][i];           // edges (+-1, 0, dz), face (0, 0, dz)
+      else e[i] = kq[2 * b + c][i];                               // corners (+-1, dy, dz), edge (0, dy, dz)
+    } else {
+      e[i] = dy == 0 ? kq[0][i] + kq[1][i] : kq[dy > 0][i];
+    }
+  }
 #pragma unroll
   for (int w = 0; w < 4; ++w) {
-    if (DY == 0 && DZ == 0) {
-      float s = 0.f;
-#pragma unroll
-      for (int q = 0; q < 4; ++q) s += kq[q][w] + kq[q][w + 1];
-      cf[0][w] = 0.f;
-      cf[1][w] = -4.f * s;
-      cf[2][w] = 0.f;
-    } else if (DZ == 0) {   // edges (+-1, DY, 0); face (0, DY, 0)
-      cf[0][w] = kq[2 * b][w] + kq[2 * b + 1][w];
-      cf[1][w] = 0.f;
-      cf[2][w] = kq[2 * b][w + 1] + kq[2 * b + 1][w + 1];
-    } else if (DY == 0) {   // edges (+-1, 0, DZ); face (0, 0, DZ)
-      cf[0][w] = kq[c][w] + kq[2 + c][w];
-      cf[1][w] = 0.f;
-      cf[2][w] = kq[c][w + 1] + kq[2 + c][w + 1];
-    } else {                // corners (+-1, DY, DZ); edge (0, DY, DZ)
-      cf[0][w] = kq[2 * b + c][w];
-      cf[1][w] = kq[2 * b + c][w] + kq[2 * b + c][w + 1];
-      cf[2][w] = kq[2 * b + c][w + 1];
-    }
-  }
-}
-
-template <int DY, int DZ, int C>
-__device__ __forceinline__ void apply_row(const float (&kq)[4][5], const float* __restrict__ X, long long pitch,
-                                          long long idx, long long px, long long pxy, float (&acc)[C][4]) {
-  float cf[3][4];
-  row_coefs<DY, DZ>(kq, cf);
-  const long long ro = (long long)DY * px + (long long)DZ * pxy;
-#pragma unroll
-  for (int c = 0; c < C; ++c) {
-    if (DY == 0 && DZ == 0) {   // the centre only
-      float m[4];
-      Vec<float>::load_keep(X + (long long)c * pitch + idx, m);
-#pragma unroll
-      for (int w = 0; w < 4; ++w) acc[c][w] = fmaf(cf[1][w], m[w], acc[c][w]);
+    const float s = e[w] + e[w + 1];
+    if constexpr (DIM == 3) {
+      cl[w] = e[w];
+      cr[w] = e[w + 1];
+      cc[w] = dy == 0 && dz == 0 ? -4.f * s : s;
     } else {
-      float e[6];
-      row6(X + (long long)c * pitch + idx + ro, e);
-#pragma unroll
-      for (int w = 0; w < 4; ++w) {
-        acc[c][w] = fmaf(cf[0][w], e[w], acc[c][w]);
-        if (DY != 0 && DZ != 0) acc[c][w] = fmaf(cf[1][w], e[w + 1], acc[c][w]);
-        acc[c][w] = fmaf(cf[2][w], e[w + 2], acc[c][w]);
-      }
+      cl[w] = dy == 0 ? e[w] : 2.f * e[w];
+      cr[w] = dy == 0 ? e[w + 1] : 2.f * e[w + 1];
+      cc[w] = dy == 0 ? -4.f * s : s;
     }
   }
 }
 
-template <int C>
-__device__ __forceinline__ void mf_group(const float (&kq)[4][5], const float* __restrict__ X, long long pitch,
-                                         long long idx, long long px, long long pxy, float (&acc)[C][4]) {
-  apply_row<-1, -1, C>(kq, X, pitch, idx, px, pxy, acc);
-  apply_row<0, -1, C>(kq, X, pitch, idx, px, pxy, acc);
-  apply_row<1, -1, C>(kq, X, pitch, idx, px, pxy, acc);
-  apply_row<-1, 0, C>(kq, X, pitch, idx, px, pxy, acc);
-  apply_row<0, 0, C>(kq, X, pitch, idx, px, pxy, acc);
-  apply_row<1, 0, C>(kq, X, pitch, idx, px, pxy, acc);
-  apply_row<-1, 1, C>(kq, X, pitch, idx, px, pxy, acc);
-  apply_row<0, 1, C>(kq, X, pitch, idx, px, pxy, acc);
-  apply_row<1, 1, C>(kq, X, pitch, idx, px, pxy, acc);
+// the products of row k: in 3D the face couplings are zero, and the row through
+// the point has no others
+template <int DIM>
+__device__ __forceinline__ void mf_row_products(int k, const float (&cl)[4], const float (&cc)[4],
+                                                const float (&cr)[4], const float (&x)[4], float (&acc)[6]) {
+  const bool centre_row = DIM == 3 && k == 4, edges = DIM == 3 && k != 4 && (k & 1);
+  if (centre_row) {
+#pragma unroll
+    for (int w = 0; w < 4; ++w) acc[w + 1] = fmaf(cc[w], x[w], acc[w + 1]);
+  } else if (edges) {
+#pragma unroll
+    for (int w = 0; w < 4; ++w) {
+      acc[w] = fmaf(cl[w], x[w], acc[w]);
+      acc[w + 2] = fmaf(cr[w], x[w], acc[w + 2]);
+    }
+  } else {
+    row_products(cl, cc, cr, x, acc);
+  }
 }
 
-// Y = A X over C columns, A from k.
-template <int C>
-__global__ void __launch_bounds__(kBlock, 3) k_spmm_mf(GridDesc g, const float* __restrict__ k32,
-                                                    SpmmIO<float> io, const DevState* state) {
+// Y = A X over C columns, A from k, rows read in aligned vectors only
+// (rows.cuh; the next row's loads are issued before the present one's
+// products): 113^3, C = 5, 36.8 -> 28.6 us, the fused Jacobi 21 -> 15 us against
+// gathering the neighbours (event-timed).
+template <int DIM, int C>
+__global__ void __launch_bounds__(kBlock, C <= 4 ? 3 : 2) k_spmm_mf(GridDesc g, RowMap map,
+                                                                    const float* __restrict__ k32, SpmmIO<float> io,
+                                                                    const DevState* state) {
   const int pb = blockIdx.y;
   if (state && state[pb].done) return;
   const float* X;
   float* Y;
   spmm_operands(io, state + pb, X, Y);
-  const long long ngroups = g.npts / 4;
-  const long long bo = (long long)pb * g.len + g.G;
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < ngroups;
-       q += (long long)gridDim.x * blockDim.x) {
-    int x0, y, z, a;
-    decode(g, q * 4, x0, y, z, a);
-    const long long idx = bo + q * 4;
-    const bool row_in = y < g.ny && z < g.nz;
-    float kq[4][5];
-    load_kappa(k32, idx, g.px, g.pxy, kq);
-    float acc[C][4];
+  constexpr int R = DIM == 3 ? 9 : 3;
+  const int lane = threadIdx.x & 31;
+  const long long wid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (wid >= map.nwarps) return;
+  long long q;
+  bool active, store;
+  row_group(map, wid, lane, g.npts / 4, q, active, store);
+  const long long idx = (long long)pb * g.len + g.G + q * 4;
+  float acc[C][6];
 #pragma unroll
-    for (int c = 0; c < C; ++c)
+  for (int c = 0; c < C; ++c)
 #pragma unroll
-      for (int w = 0; w < 4; ++w) acc[c][w] = 0.f;
-    mf_group<C>(kq, X, g.cp, idx, g.px, g.pxy, acc);
+    for (int i = 0; i < 6; ++i) acc[c][i] = 0.f;
+  if (active) {
+    float x[2][C][4], kq[DIM == 3 ? 4 : 2][5];
+    auto load = [&](int k) {
+      const long long ro = (k % 3 - 1) * (long long)g.px + (DIM == 3 ? (k / 3 - 1) * g.pxy : 0);
 #pragma unroll
-    for (int c = 0; c < C; ++c) {
+      for (int c = 0; c < C; ++c) Vec<float>::load_keep(X + (long long)c * g.cp + idx + ro, x[k & 1][c]);
+    };
+    load_kappa<DIM>(k32, idx, g.px, g.pxy, kq);
+    load(0);
 #pragma unroll
-      for (int w = 0; w < 4; ++w)
-        if (!row_in || x0 + w >= g.nx) acc[c][w] = 0.f;   // pad points: zero rows
-      Vec<float>::store(Y + (long long)c * g.cp + idx, acc[c]);
+    for (int k = 0; k < R; ++k) {
+      if (k + 1 < R) load(k + 1);
+      float cl[4], cc[4], cr[4];
+      mf_row_coeffs<DIM>(kq, k, cl, cc, cr);
+#pragma unroll
+      for (int c = 0; c < C; ++c) mf_row_products<DIM>(k, cl, cc, cr, x[k & 1][c], acc[c]);
     }
+  }
+  int x0 = 0, y = 0, z = 0, a;
+  if (store) decode(g, q * 4, x0, y, z, a);
+  const bool row_in = y < g.ny && (DIM == 2 || z < g.nz);
+#pragma unroll
+  for (int c = 0; c < C; ++c) {
+    edge_shift(acc[c], lane);
+    float o[4];
+#pragma unroll
+    for (int w = 0; w < 4; ++w) o[w] = row_in && x0 + w < g.nx ? acc[c][w + 1] : 0.f;   // pad points: zero rows
+    if (store) Vec<float>::store(Y + (long long)c * g.cp + idx, o);
   }
 }
 
 // Two damped-Jacobi sweeps from zero on the fine grid, fused (as k_jacobi
-// mode 1): s1 = dinv r, s = s1 + dinv (r - A s1), A from k; dinv (stored)
-// is omega / diagonal, zero at pads.
-__global__ void __launch_bounds__(kBlock, 4) k_jacobi_mf(GridDesc g, const float* __restrict__ k32,
-                                                      const float* __restrict__ dinv, const float* __restrict__ r,
-                                                      float* __restrict__ out, const DevState* state) {
+// mode 1): s1 = dinv r, s = s1 + dinv (r - A s1), A from k; dinv (stored) is
+// omega / diagonal, zero at pads.
+template <int DIM>
+__global__ void __launch_bounds__(kBlock, 4) k_jacobi_mf(GridDesc g, RowMap map, const float* __restrict__ k32,
+                                                         const float* __restrict__ dinv, const float* __restrict__ r,
+                                                         float* __restrict__ out, const DevState* state) {
   const int pb = blockIdx.y;
   if (state && state[pb].done) return;
-  const long long ngroups = g.npts / 4;
-  const long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (q >= ngroups) return;
+  constexpr int R = DIM == 3 ? 9 : 3;
+  const int lane = threadIdx.x & 31;
+  const long long wid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (wid >= map.nwarps) return;
+  long long q;
+  bool active, store;
+  row_group(map, wid, lane, g.npts / 4, q, active, store);
   const long long idx = (long long)pb * g.len + g.G + q * 4;
-  float kq[4][5];
-  load_kappa(k32, idx, g.px, g.pxy, kq);
-  // s1 = dinv r on the 3 x 3 row neighbourhood, then A s1 through the rows
-  float acc[1][4] = {{0.f, 0.f, 0.f, 0.f}};
-  float di[4], ri[4];
-  Vec<float>::load_keep(dinv + idx, di);
-  Vec<float>::load_keep(r + idx, ri);
-#define MPCG_JMF_ROW(DY, DZ)                                                                        \
-  {                                                                                                 \
-    float cf[3][4];                                                                                 \
-    row_coefs<DY, DZ>(kq, cf);                                                                      \
-    const long long ro = (long long)(DY) * g.px + (long long)(DZ) * g.pxy;                           \
-    float ed[6], er[6];                                                                             \
-    row6(dinv + idx + ro, ed);                                                           \
-    row6(r + idx + ro, er);                                                              \
-    _Pragma("unroll") for (int w = 0; w < 4; ++w) {                                                \
-      acc[0][w] = fmaf(cf[0][w], ed[w] * er[w], acc[0][w]);                                         \
-      acc[0][w] = fmaf(cf[1][w], ed[w + 1] * er[w + 1], acc[0][w]);                                 \
-      acc[0][w] = fmaf(cf[2][w], ed[w + 2] * er[w + 2], acc[0][w]);                                 \
-    }                                                                                               \
-  }
-  MPCG_JMF_ROW(-1, -1) MPCG_JMF_ROW(0, -1) MPCG_JMF_ROW(1, -1)
-  MPCG_JMF_ROW(-1, 0) MPCG_JMF_ROW(0, 0) MPCG_JMF_ROW(1, 0)
-  MPCG_JMF_ROW(-1, 1) MPCG_JMF_ROW(0, 1) MPCG_JMF_ROW(1, 1)
-#undef MPCG_JMF_ROW
-  float o[4];
+  float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, di[4] = {}, ri[4] = {};
+  if (active) {
+    float kq[DIM == 3 ? 4 : 2][5];
+    load_kappa<DIM>(k32, idx, g.px, g.pxy, kq);
 #pragma unroll
-  for (int w = 0; w < 4; ++w) {
-    const float s1 = di[w] * ri[w];
-    o[w] = s1 + di[w] * (ri[w] - acc[0][w]);
-  }
-  Vec<float>::store(out + idx, o);
-}
-
-// ---- 2D: kq[b][k] for the element whose lowest node is (x0 - 1 + k, y - 1 + b)
-__device__ __forceinline__ void load_kappa2(const float* __restrict__ k32, long long idx, long long px,
-                                            float (&kq)[2][5]) {
+    for (int k = 0; k < R; ++k) {
+      const long long ro = (k % 3 - 1) * (long long)g.px + (DIM == 3 ? (k / 3 - 1) * g.pxy : 0);
+      float dv[4], x[4], cl[4], cc[4], cr[4];
+      Vec<float>::load_keep(dinv + idx + ro, dv);
+      Vec<float>::load_keep(r + idx + ro, x);
+      if (k == R / 2) {
 #pragma unroll
-  for (int b = 0; b < 2; ++b) {
-    const float* p = k32 + idx + (long long)(b - 1) * px;
-    float m[4];
-    Vec<float>::load_keep(p, m);
-    kq[b][0] = p[-1];
-#pragma unroll
-    for (int w = 0; w < 4; ++w) kq[b][w + 1] = m[w];
-  }
-}
-
-// Coefficients of stencil row DY for the four points: cf[dx + 1][w].
-template <int DY>
-__device__ __forceinline__ void row_coefs2(const float (&kq)[2][5], float (&cf)[3][4]) {
-  constexpr int b = DY > 0;
-#pragma unroll
-  for (int w = 0; w < 4; ++w) {
-    if (DY == 0) {   // edges (+-1, 0), centre
-      cf[0][w] = kq[0][w] + kq[1][w];
-      cf[1][w] = -4.f * (kq[0][w] + kq[0][w + 1] + kq[1][w] + kq[1][w + 1]);
-      cf[2][w] = kq[0][w + 1] + kq[1][w + 1];
-    } else {         // corners (+-1, DY), edge (0, DY)
-      cf[0][w] = 2.f * kq[b][w];
-      cf[1][w] = kq[b][w] + kq[b][w + 1];
-      cf[2][w] = 2.f * kq[b][w + 1];
-    }
-  }
-}
-
-template <int C>
-__global__ void __launch_bounds__(kBlock, 3) k_spmm_mf2d(GridDesc g, const float* __restrict__ k32,
-                                                      SpmmIO<float> io, const DevState* state) {
-  const int pb = blockIdx.y;
-  if (state && state[pb].done) return;
-  const float* X;
-  float* Y;
-  spmm_operands(io, state + pb, X, Y);
-  const long long ngroups = g.npts / 4;
-  const long long bo = (long long)pb * g.len + g.G;
-  for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < ngroups;
-       q += (long long)gridDim.x * blockDim.x) {
-    int x0, y, z, a;
-    decode(g, q * 4, x0, y, z, a);
-    const long long idx = bo + q * 4;
-    float kq[2][5];
-    load_kappa2(k32, idx, g.px, kq);
-    float cf[3][3][4];
-    row_coefs2<-1>(kq, cf[0]);
-    row_coefs2<0>(kq, cf[1]);
-    row_coefs2<1>(kq, cf[2]);
-#pragma unroll
-    for (int c = 0; c < C; ++c) {
-      float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        float e[6];
-        row6(X + (long long)c * g.cp + idx + (long long)(k - 1) * g.px, e);
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-          acc[w] = fmaf(cf[k][0][w], e[w], acc[w]);
-          acc[w] = fmaf(cf[k][1][w], e[w + 1], acc[w]);
-          acc[w] = fmaf(cf[k][2][w], e[w + 2], acc[w]);
+        for (int i = 0; i < 4; ++i) {
+          di[i] = dv[i];
+          ri[i] = x[i];
         }
       }
 #pragma unroll
-      for (int w = 0; w < 4; ++w)
-        if (y >= g.ny || x0 + w >= g.nx) acc[w] = 0.f;   // pad points: zero rows
-      Vec<float>::store(Y + (long long)c * g.cp + idx, acc);
+      for (int i = 0; i < 4; ++i) x[i] *= dv[i];
+      mf_row_coeffs<DIM>(kq, k, cl, cc, cr);
+      mf_row_products<DIM>(k, cl, cc, cr, x, acc);
     }
   }
-}
-
-__global__ void __launch_bounds__(kBlock, 4) k_jacobi_mf2d(GridDesc g, const float* __restrict__ k32,
-                                                        const float* __restrict__ dinv, const float* __restrict__ r,
-                                                        float* __restrict__ out, const DevState* state) {
-  const int pb = blockIdx.y;
-  if (state && state[pb].done) return;
-  const long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (q >= g.npts / 4) return;
-  const long long idx = (long long)pb * g.len + g.G + q * 4;
-  float kq[2][5];
-  load_kappa2(k32, idx, g.px, kq);
-  float di[4], ri[4], acc[4] = {0.f, 0.f, 0.f, 0.f};
-  Vec<float>::load_keep(dinv + idx, di);
-  Vec<float>::load_keep(r + idx, ri);
-#define MPCG_JMF2_ROW(DY)                                                                           \
-  {                                                                                                 \
-    float cf[3][4];                                                                                 \
-    row_coefs2<DY>(kq, cf);                                                                         \
-    float ed[6], er[6];                                                                             \
-    row6(dinv + idx + (long long)(DY) * g.px, ed);                                                  \
-    row6(r + idx + (long long)(DY) * g.px, er);                                                     \
-    _Pragma("unroll") for (int w = 0; w < 4; ++w) {                                                \
-      acc[w] = fmaf(cf[0][w], ed[w] * er[w], acc[w]);                                               \
-      acc[w] = fmaf(cf[1][w], ed[w + 1] * er[w + 1], acc[w]);                                       \
-      acc[w] = fmaf(cf[2][w], ed[w + 2] * er[w + 2], acc[w]);                                       \
-    }                                                                                               \
-  }
-  MPCG_JMF2_ROW(-1) MPCG_JMF2_ROW(0) MPCG_JMF2_ROW(1)
-#undef MPCG_JMF2_ROW
+  edge_shift(acc, lane);
+  if (!store) return;
   float o[4];
 #pragma unroll
-  for (int w = 0; w < 4; ++w) o[w] = di[w] * ri[w] + di[w] * (ri[w] - acc[w]);
+  for (int i = 0; i < 4; ++i) o[i] = di[i] * ri[i] + di[i] * (ri[i] - acc[i + 1]);
   Vec<float>::store(out + idx, o);
 }
-
-inline int blocks_for(long long n) { return (int)((n + kBlock - 1) / kBlock); }
 
 }  // namespace
 
@@ -401,44 +292,35 @@ mpcg_status place_kappa(const GridDesc& g, const double* kappa, int ne, double h
   return MPCG_OK;
 }
 
-#define MPCG_MF_CASES(K, ...)                                                                      \
-  case 1: K<1><<<__VA_ARGS__>>>(g, k32, io, state); break;                                   \
-  case 2: K<2><<<__VA_ARGS__>>>(g, k32, io, state); break;                                   \
-  case 3: K<3><<<__VA_ARGS__>>>(g, k32, io, state); break;                                   \
-  case 4: K<4><<<__VA_ARGS__>>>(g, k32, io, state); break;                                   \
-  case 5: K<5><<<__VA_ARGS__>>>(g, k32, io, state); break;                                   \
-  case 6: K<6><<<__VA_ARGS__>>>(g, k32, io, state); break;                                   \
-  case 7: K<7><<<__VA_ARGS__>>>(g, k32, io, state); break;                                   \
-  case 8: K<8><<<__VA_ARGS__>>>(g, k32, io, state); break;                                   \
-  case 9: K<9><<<__VA_ARGS__>>>(g, k32, io, state); break;                                   \
-  case 10: K<10><<<__VA_ARGS__>>>(g, k32, io, state); break;                                 \
-  case 11: K<11><<<__VA_ARGS__>>>(g, k32, io, state); break;                                 \
-  case 12: K<12><<<__VA_ARGS__>>>(g, k32, io, state); break;
-
-bool launch_spmm_mf(const GridDesc& g, const float* k32, const SpmmIO<float>& io, int C, int nblocks,
-                    const DevState* state, cudaStream_t s) {
-  const dim3 grid(nblocks, g.nb);
-  const int threads = stream_threads(g);
-  if (g.dim == 3) {
-    switch (C) {
-      MPCG_MF_CASES(k_spmm_mf, grid, threads, 0, s)
-      default: return false;
-    }
-  } else {
-    switch (C) {
-      MPCG_MF_CASES(k_spmm_mf2d, grid, threads, 0, s)
-      default: return false;
-    }
+template <int DIM>
+static bool spmm_mf(const GridDesc& g, const float* k32, const SpmmIO<float>& io, int C, const DevState* state,
+                    cudaStream_t s) {
+  const RowMap map = row_map(g);
+  const int threads = spread_threads(32 * map.nwarps * g.nb);
+  const dim3 grid((unsigned)((32 * map.nwarps + threads - 1) / threads), g.nb);
+#define MPCG_MF_CASE(CC)                                                     \
+  case CC:                                                                   \
+    k_spmm_mf<DIM, CC><<<grid, threads, 0, s>>>(g, map, k32, io, state);     \
+    return true;
+  switch (C) {
+    MPCG_MF_CASE(1) MPCG_MF_CASE(2) MPCG_MF_CASE(3) MPCG_MF_CASE(4) MPCG_MF_CASE(5) MPCG_MF_CASE(6)
+    MPCG_MF_CASE(7) MPCG_MF_CASE(8) MPCG_MF_CASE(9) MPCG_MF_CASE(10) MPCG_MF_CASE(11) MPCG_MF_CASE(12)
+    default: return false;
   }
-  return true;
+#undef MPCG_MF_CASE
 }
-#undef MPCG_MF_CASES
+
+bool launch_spmm_mf(const GridDesc& g, const float* k32, const SpmmIO<float>& io, int C, const DevState* state,
+                    cudaStream_t s) {
+  return g.dim == 3 ? spmm_mf<3>(g, k32, io, C, state, s) : spmm_mf<2>(g, k32, io, C, state, s);
+}
 
 void launch_jacobi_mf(const GridDesc& g, const float* k32, const float* dinv, const float* r, float* out,
                       const DevState* state, cudaStream_t s) {
-  const dim3 grid(blocks_for(g.npts / 4), g.nb);
-  if (g.dim == 3) k_jacobi_mf<<<grid, kBlock, 0, s>>>(g, k32, dinv, r, out, state);
-  else k_jacobi_mf2d<<<grid, kBlock, 0, s>>>(g, k32, dinv, r, out, state);
+  const RowMap map = row_map(g);
+  const dim3 grid((unsigned)((32 * map.nwarps + kBlock - 1) / kBlock), g.nb);
+  if (g.dim == 3) k_jacobi_mf<3><<<grid, kBlock, 0, s>>>(g, map, k32, dinv, r, out, state);
+  else k_jacobi_mf<2><<<grid, kBlock, 0, s>>>(g, map, k32, dinv, r, out, state);
 }
 
 }  // namespace mpcg

@@ -11,6 +11,7 @@
 // test.  blockIdx.y selects the problem of a batch (offset b * len; columns
 // and stencil planes are cp = nb * len apart).
 #include "kernels.cuh"
+#include "rows.cuh"
 #include "tune.h"
 #include "vec.cuh"
 
@@ -206,7 +207,7 @@ __device__ __forceinline__ void stencil_group(const T* __restrict__ st, long lon
 // The FP32 3D instances with up to 6 columns run three blocks per SM (at most
 // 85 registers) in one wave of resident blocks (spmm_blocks): measured faster
 // than two blocks per SM over two waves, whose loads wait longer.
-template <typename T, int DIM, int C, bool SYM = false>
+template <typename T, int DIM, int C>
 __global__ void __launch_bounds__(kBlock, (sizeof(T) == 4 && DIM == 3 && C <= 6) ? 3 : (kIsDw<T> ? 2 : 1))
     k_spmm(GridDesc g, const T* __restrict__ st, SpmmIO<T> io, const DevState* state) {
   const int pb = blockIdx.y;
@@ -225,7 +226,7 @@ __global__ void __launch_bounds__(kBlock, (sizeof(T) == 4 && DIM == 3 && C <= 6)
     for (int c = 0; c < C; ++c)
 #pragma unroll
       for (int w = 0; w < W; ++w) acc[c][w] = 0;
-    stencil_group<T, DIM, C, SYM>(st, g.cp, X, idx, g.px, g.pxy, acc);
+    stencil_group<T, DIM, C>(st, g.cp, X, idx, g.px, g.pxy, acc);
 #pragma unroll
     for (int c = 0; c < C; ++c) Vec<T>::store(Y + (long long)c * g.cp + idx, acc[c]);
   }
@@ -455,6 +456,106 @@ __global__ void __launch_bounds__(kBlock, 4) k_jacobi(GridDesc g, const T* __res
     return;
   }
   if (active) VecN<T, W>::store(out + idx, o);
+}
+
+// The FP32 block SpMM on the symmetric half, rows read in aligned vectors only
+// (rows.cuh).  Bound by load latency (129^3, C = 6, ncu: DRAM 53 %, L1 41 %, long
+// scoreboard 7 of 11 stall cycles, 16 warps per SM), hence two rows in registers,
+// the next one's loads issued before the present one's products; C columns per
+// thread, because the columns share the row's coefficients.  Event-timed: 129^3
+// 69 -> 62 us, 1025^2 with C = 9 27 -> 23.6 us.  Slower: three columns per
+// thread on twice the warps (64-72 us), one row at a time (78-82 us), a bulk L2
+// prefetch of the planes (62 us), blocks tiled over y and z (63-65 us; 97^3 30
+// against 27 us).
+template <int DIM, int C>
+__global__ void __launch_bounds__(kBlock, C <= 3 ? 3 : 2) k_spmm_half(GridDesc g, RowMap map,
+                                                                      const float* __restrict__ st, SpmmIO<float> io,
+                                                                      const DevState* state) {
+  const int pb = blockIdx.y;
+  if (state && state[pb].done) return;
+  const float* X;
+  float* Y;
+  spmm_operands(io, state + pb, X, Y);
+  constexpr int R = DIM == 3 ? 9 : 3;
+  const int lane = threadIdx.x & 31;
+  const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (w >= map.nwarps) return;
+  long long q;
+  bool active, store;
+  row_group(map, w, lane, g.npts / 4, q, active, store);
+  const long long idx = (long long)pb * g.len + g.G + q * 4;
+  float acc[C][6];
+#pragma unroll
+  for (int c = 0; c < C; ++c)
+#pragma unroll
+    for (int k = 0; k < 6; ++k) acc[c][k] = 0.f;
+  if (active) {
+    float cl[2][4], cc[2][4], cr[2][4], x[2][C][4];
+    auto load = [&](int k) {
+      const long long ro = row_offset<DIM>(k, g.px, g.pxy);
+      half_row_coeffs<DIM>(st, g.cp, idx, ro, k, cl[k & 1], cc[k & 1], cr[k & 1]);
+#pragma unroll
+      for (int c = 0; c < C; ++c) Vec<float>::load_keep(X + (long long)c * g.cp + idx + ro, x[k & 1][c]);
+    };
+    load(0);
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+      if (k + 1 < R) load(k + 1);
+#pragma unroll
+      for (int c = 0; c < C; ++c) row_products(cl[k & 1], cc[k & 1], cr[k & 1], x[k & 1][c], acc[c]);
+    }
+  }
+#pragma unroll
+  for (int c = 0; c < C; ++c) {
+    edge_shift(acc[c], lane);
+    const float o[4] = {acc[c][1], acc[c][2], acc[c][3], acc[c][4]};
+    if (store) Vec<float>::store(Y + (long long)c * g.cp + idx, o);
+  }
+}
+
+// Two damped-Jacobi sweeps from zero on the symmetric half (mode 1 of
+// k_jacobi), rows read in aligned vectors only.
+template <int DIM>
+__global__ void __launch_bounds__(kBlock, 4) k_jacobi_half(GridDesc g, RowMap map, const float* __restrict__ st,
+                                                           const float* __restrict__ dinv, const float* __restrict__ r,
+                                                           float* __restrict__ out, const DevState* state) {
+  const int pb = blockIdx.y;
+  if (state && state[pb].done) return;
+  constexpr int R = DIM == 3 ? 9 : 3;
+  const int lane = threadIdx.x & 31;
+  const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  if (w >= map.nwarps) return;
+  long long q;
+  bool active, store;
+  row_group(map, w, lane, g.npts / 4, q, active, store);
+  const long long idx = (long long)pb * g.len + g.G + q * 4;
+  float acc[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f}, di[4] = {}, ri[4] = {};
+  if (active) {
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+      const long long ro = row_offset<DIM>(k, g.px, g.pxy);
+      float cl[4], cc[4], cr[4], d[4], x[4];
+      half_row_coeffs<DIM>(st, g.cp, idx, ro, k, cl, cc, cr);
+      Vec<float>::load_keep(dinv + idx + ro, d);
+      Vec<float>::load_keep(r + idx + ro, x);
+      if (k == R / 2) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          di[i] = d[i];
+          ri[i] = x[i];
+        }
+      }
+#pragma unroll
+      for (int i = 0; i < 4; ++i) x[i] *= d[i];
+      row_products(cl, cc, cr, x, acc);
+    }
+  }
+  edge_shift(acc, lane);
+  if (!store) return;
+  float o[4];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) o[i] = di[i] * ri[i] + di[i] * (ri[i] - acc[i + 1]);
+  Vec<float>::store(out + idx, o);
 }
 
 // Multicoloured SSOR (Section 3's smoother; the colouring is a reading):
@@ -1165,7 +1266,7 @@ template void launch_pack<float, float>(const GridDesc&, const float*, long long
 template void launch_unpack<float, float>(const GridDesc&, const float*, float*, long long, int, cudaStream_t);
 #endif
 
-template <typename T, int DIM, bool SYM = false>
+template <typename T, int DIM>
 static void spmm_dim(const GridDesc& g, const T* st, const SpmmIO<T>& io, int C, const DevState* state,
                      cudaStream_t s) {
   int threads = stream_threads(g), blocks = spmm_blocks<T>(g, C);
@@ -1176,7 +1277,7 @@ static void spmm_dim(const GridDesc& g, const T* st, const SpmmIO<T>& io, int C,
   const dim3 grid(blocks, g.nb);
 #define MPCG_SPMM_CASE(CC)                                                                      \
   case CC:                                                                                      \
-    k_spmm<T, DIM, CC, SYM><<<grid, threads, 0, s>>>(g, st, io, state);                         \
+    k_spmm<T, DIM, CC><<<grid, threads, 0, s>>>(g, st, io, state);                              \
     break;
   switch (C) {
     MPCG_SPMM_CASE(1) MPCG_SPMM_CASE(2) MPCG_SPMM_CASE(3) MPCG_SPMM_CASE(4) MPCG_SPMM_CASE(5)
@@ -1300,6 +1401,15 @@ static void jacobi_impl(const GridDesc& g, const T* st, const T* dinv, const T* 
     return;
   }
   const dim3 grid(blocks_for(g.npts / vw<T>()), g.nb);
+  if constexpr (SYM) {
+    if (mode == 1) {
+      const RowMap map = row_map(g);
+      const dim3 rows((unsigned)((32 * map.nwarps + kBlock - 1) / kBlock), g.nb);
+      if (g.dim == 3) k_jacobi_half<3><<<rows, kBlock, 0, s>>>(g, map, st, dinv, r, out, state);
+      else k_jacobi_half<2><<<rows, kBlock, 0, s>>>(g, map, st, dinv, r, out, state);
+      return;
+    }
+  }
   if (g.dim == 3) k_jacobi<T, 3, Vec<T>::W, SYM><<<grid, kBlock, 0, s>>>(g, st, dinv, r, sin, out, mode, state);
   else k_jacobi<T, 2, Vec<T>::W, SYM><<<grid, kBlock, 0, s>>>(g, st, dinv, r, sin, out, mode, state);
 }
@@ -1591,11 +1701,30 @@ void launch_sym_half(const GridDesc& g, const double* st, float* half, cudaStrea
   else k_sym_half<2><<<grid_for(g.cp, 4096), kBlock, 0, s>>>(g, st, half);
 }
 
+template <int DIM>
+static void spmm_half(const GridDesc& g, const float* half, const SpmmIO<float>& io, int C, const DevState* state,
+                      cudaStream_t s) {
+  const RowMap map = row_map(g);
+  const int threads = spread_threads(32 * map.nwarps * g.nb);
+  const dim3 grid((unsigned)((32 * map.nwarps + threads - 1) / threads), g.nb);
+#define MPCG_SPMM_CASE(CC)                                                   \
+  case CC:                                                                   \
+    k_spmm_half<DIM, CC><<<grid, threads, 0, s>>>(g, map, half, io, state);  \
+    break;
+  switch (C) {
+    MPCG_SPMM_CASE(1) MPCG_SPMM_CASE(2) MPCG_SPMM_CASE(3) MPCG_SPMM_CASE(4) MPCG_SPMM_CASE(5)
+    MPCG_SPMM_CASE(6) MPCG_SPMM_CASE(7) MPCG_SPMM_CASE(8) MPCG_SPMM_CASE(9) MPCG_SPMM_CASE(10)
+    MPCG_SPMM_CASE(11) MPCG_SPMM_CASE(12)
+    default: break;
+  }
+#undef MPCG_SPMM_CASE
+}
+
 void launch_spmm_sym(const GridDesc& g, const float* half, const SpmmIO<float>& io, int C, const DevState* state,
                      cudaStream_t s) {
   if (g.ncomp != 1) return;
-  if (g.dim == 3) spmm_dim<float, 3, true>(g, half, io, C, state, s);
-  else spmm_dim<float, 2, true>(g, half, io, C, state, s);
+  if (g.dim == 3) spmm_half<3>(g, half, io, C, state, s);
+  else spmm_half<2>(g, half, io, C, state, s);
 }
 
 void launch_jacobi_sym(const GridDesc& g, const float* half, const float* dinv, const float* r, const float* sin,

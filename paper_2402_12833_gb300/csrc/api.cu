@@ -383,7 +383,9 @@ mpcg_status build_solver(mg_hierarchy* h, Solver<T>& S) {
   const size_t sbc = (size_t)stream_blocks_cap(gf), gcc = (size_t)gram_chunks_cap(gf);
   CKS(S.mem.get(&S.part_res, nb * 2 * sbc, s));
   CKS(S.mem.get(&S.part_W, nb * S.m * C * C * gcc, s));
-  CKS(S.mem.get(&S.part_G, nb * (C * (C + 1) / 2 + C) * sbc, s));
+  // at least the row kernels' slots: two blocks per SM of 256 threads, or as many smaller ones
+  const size_t gsl = std::max(sbc, (size_t)16 * (size_t)std::max(sm_count(), 152));
+  CKS(S.mem.get(&S.part_G, nb * (C * (C + 1) / 2 + C) * gsl, s));
   CKS(S.mem.get(&S.part_r, nb * sbc, s));
   CKS(S.mem.get(&S.small_scratch, nb * kSmallScratch, s));
   CKS(S.mem.get(&S.counters, 2 * nb + 1, s));
@@ -758,28 +760,35 @@ void enqueue_prologue(mg_hierarchy* h, Solver<T>& S, cudaGraphConditionalHandle 
                                    loop_cond(h, S, cond, use_cond), s));
 }
 
-// A P of the block being built (the ring slot after the newest).
+// A P of the block being built (the ring slot after the newest) and the partial
+// sums of P^T A P and P^T r: with the product where its kernel forms them (the
+// FP32 scalar stencils), else in a launch of their own.  Returns the slots per
+// value of part_G.
 template <typename T>
-void enqueue_block_spmm(mg_hierarchy* h, Solver<T>& S, cudaStream_t s) {
+int enqueue_block_product(mg_hierarchy* h, Solver<T>& S, cudaStream_t s) {
   const Level& L = h->lev[h->levels - 1];
   const int C = S.C;
+  int slots = 0;
   if (h->algebraic) {
     LAUNCH(h, K_SPMM, s,
            launch_ell_spmm<T>(ell_of<T>(L.eA), spmm_ring(S.win, S.m, L.g.G), L.g.cp, L.g.cp, C, S.state, s));
-    return;
-  }
-  const SpmmIO<T> io = spmm_ring(S.win, S.m);
-  if constexpr (std::is_same<T, float>::value) {
-    if (L.kq32) {   // fine operator rebuilt from the element coefficients
-      LAUNCH(h, K_SPMM, s, launch_spmm_mf(L.g, L.kq32, io, C, S.state, s));
-      return;
+  } else {
+    const SpmmIO<T> io = spmm_ring(S.win, S.m);
+    bool done = false;
+    if constexpr (std::is_same<T, float>::value) {
+      if (L.kq32) {   // fine operator rebuilt from the element coefficients
+        LAUNCH(h, K_SPMM, s, slots = launch_spmm_mf(L.g, L.kq32, io, C, S.r, S.part_G, S.state, s));
+        done = true;
+      } else if (L.sth32) {   // the symmetric half of the stored stencil
+        LAUNCH(h, K_SPMM, s, slots = launch_spmm_sym(L.g, L.sth32, io, C, S.r, S.part_G, S.state, s));
+        done = true;
+      }
     }
-    if (L.sth32) {   // the symmetric half of the stored stencil
-      LAUNCH(h, K_SPMM, s, launch_spmm_sym(L.g, L.sth32, io, C, S.state, s));
-      return;
-    }
+    if (!done) LAUNCH(h, K_SPMM, s, launch_spmm<T>(L.g, st_of<T>(L), io, C, S.state, s));
   }
-  LAUNCH(h, K_SPMM, s, launch_spmm<T>(L.g, st_of<T>(L), io, C, S.state, s));
+  if (slots) return slots;
+  LAUNCH(h, K_OGRAM, s, launch_block_gram<T>(L.g, S.win, S.r, C, S.part_G, S.state, s));
+  return stream_blocks(L.g);
 }
 
 template <typename T>
@@ -808,9 +817,8 @@ void enqueue_body(mg_hierarchy* h, Solver<T>& S, cudaGraphConditionalHandle cond
   LAUNCH(h, K_BETA, s, launch_small_beta(S.state, h->nb, S.part_W, gram_shape<T>(L.g, C, S.m), C, S.small_scratch,
                                          S.counters, s));
   LAUNCH(h, K_ORTH, s, launch_orth_update<T>(L.g, S.win, S.Z, C, S.state, s));
-  enqueue_block_spmm<T>(h, S, s);
-  LAUNCH(h, K_OGRAM, s, launch_block_gram<T>(L.g, S.win, S.r, C, S.part_G, S.state, s));
-  LAUNCH(h, K_ALPHA, s, launch_small_alpha(S.state, h->nb, S.part_G, stream_blocks(L.g), C, S.alpha_hist,
+  const int slots = enqueue_block_product<T>(h, S, s);
+  LAUNCH(h, K_ALPHA, s, launch_small_alpha(S.state, h->nb, S.part_G, slots, C, S.alpha_hist,
                                           (long long)S.hist_cap * C, S.small_scratch, S.counters, s));
   // the new block's inverse Gram, which the next beta reads, beside the update
   cudaStream_t si = h->prof.on ? s : h->side[0];
@@ -2546,7 +2554,7 @@ mpcg_status mg_apply_operator_f32(mg_hierarchy* h, int level, const double* X, d
   for (int c0 = 0; c0 < ncols; c0 += chunk) {
     const int nc = ncols - c0 < chunk ? ncols - c0 : chunk;
     launch_pack<double, float>(L.g, X + (size_t)c0 * L.g.n, L.g.n, xp, nc, s);
-    if (L.sth32) launch_spmm_sym(L.g, L.sth32, spmm_io<float>(xp, yp), nc, nullptr, s);
+    if (L.sth32) launch_spmm_sym(L.g, L.sth32, spmm_io<float>(xp, yp), nc, nullptr, nullptr, nullptr, s);
     else launch_spmm<float>(L.g, L.st32, spmm_io<float>(xp, yp), nc, nullptr, s);
     launch_unpack<float, double>(L.g, yp, Y + (size_t)c0 * L.g.n, L.g.n, nc, s);
   }

@@ -129,9 +129,11 @@ int sym_planes(int dim);
 // half (sym_planes(g.dim) * g.cp floats) from the full FP64 planes st;
 // couplings with a pad row or column stored as zero
 void launch_sym_half(const GridDesc& g, const double* st, float* half, cudaStream_t s);
-// launch_spmm<float> and launch_jacobi<float> (scalar grids) reading the half
-void launch_spmm_sym(const GridDesc& g, const float* half, const SpmmIO<float>& io, int C, const DevState* state,
-                     cudaStream_t s);
+// launch_spmm<float> and launch_jacobi<float> (scalar grids) reading the half;
+// with part the partial sums of launch_block_gram for X = P as well (residual r),
+// in the returned number of slots per value; 0: not formed
+int launch_spmm_sym(const GridDesc& g, const float* half, const SpmmIO<float>& io, int C, const float* r, double* part,
+                    const DevState* state, cudaStream_t s);
 void launch_jacobi_sym(const GridDesc& g, const float* half, const float* dinv, const float* r, const float* sin,
                        float* out, int mode, const DevState* state, cudaStream_t s);
 // Vector operators (3 unknowns per node): t = r - A x (one sweep's residual)
@@ -214,9 +216,11 @@ void launch_update_xr(const GridDesc& g, Window<T> win, T* x, T* r, int C, doubl
 mpcg_status place_kappa(const GridDesc& g, const double* kappa, int ne, double h, float* k32, double* k64,
                         unsigned long long* check, const double* st64, double* maxdiff, double* maxabs,
                         cudaStream_t s);
-// Y = A X (C <= 12 columns; false for other C) and the fused two-sweep Jacobi, A rebuilt from k32 (2D / 3D scalar, FP32).
-bool launch_spmm_mf(const GridDesc& g, const float* k32, const SpmmIO<float>& io, int C, const DevState* state,
-                    cudaStream_t s);
+// Y = A X (C <= 12 columns) with launch_block_gram's partial sums (returns the
+// slots per value), and the fused two-sweep Jacobi, A rebuilt from k32 (2D / 3D
+// scalar, FP32).
+int launch_spmm_mf(const GridDesc& g, const float* k32, const SpmmIO<float>& io, int C, const float* r, double* part,
+                   const DevState* state, cudaStream_t s);
 void launch_jacobi_mf(const GridDesc& g, const float* k32, const float* dinv, const float* r, float* out,
                       const DevState* state, cudaStream_t s);
 

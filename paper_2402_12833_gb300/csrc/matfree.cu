@@ -171,57 +171,83 @@ __device__ __forceinline__ void mf_row_products(int k, const float (&cl)[4], con
 // (rows.cuh; the next row's loads are issued before the present one's
 // products): 113^3, C = 5, 36.8 -> 28.6 us, the fused Jacobi 21 -> 15 us against
 // gathering the neighbours (event-timed).
+// The Gram partial sums of the new block X = P go to part.
 template <int DIM, int C>
-__global__ void __launch_bounds__(kBlock, C <= 4 ? 3 : 2) k_spmm_mf(GridDesc g, RowMap map,
+__global__ void __launch_bounds__(kBlock, C <= 3 ? 3 : 2) k_spmm_mf(GridDesc g, RowMap map,
                                                                     const float* __restrict__ k32, SpmmIO<float> io,
+                                                                    const float* __restrict__ r, double* part,
                                                                     const DevState* state) {
   const int pb = blockIdx.y;
   if (state && state[pb].done) return;
   const float* X;
   float* Y;
   spmm_operands(io, state + pb, X, Y);
-  constexpr int R = DIM == 3 ? 9 : 3;
+  constexpr int R = DIM == 3 ? 9 : 3, NV = C * (C + 1) / 2 + C;
   const int lane = threadIdx.x & 31;
-  const long long wid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (wid >= map.nwarps) return;
-  long long q;
-  bool active, store;
-  row_group(map, wid, lane, g.npts / 4, q, active, store);
-  const long long idx = (long long)pb * g.len + g.G + q * 4;
-  float acc[C][6];
+  const long long ngroups = g.npts / 4, bo = (long long)pb * g.len + g.G;
+  double hold[rs_count(NV, 5)] = {};
+  int base = 0, nvalid = 0;
+  for (long long wid = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; wid < map.nwarps;
+       wid += (long long)gridDim.x * (blockDim.x >> 5)) {
+    long long q;
+    bool active, store;
+    row_group(map, wid, lane, ngroups, q, active, store);
+    const long long idx = bo + q * 4;
+    float acc[C][6];
 #pragma unroll
-  for (int c = 0; c < C; ++c)
+    for (int c = 0; c < C; ++c)
 #pragma unroll
-    for (int i = 0; i < 6; ++i) acc[c][i] = 0.f;
-  if (active) {
-    float x[2][C][4], kq[DIM == 3 ? 4 : 2][5];
-    auto load = [&](int k) {
-      const long long ro = (k % 3 - 1) * (long long)g.px + (DIM == 3 ? (k / 3 - 1) * g.pxy : 0);
+      for (int i = 0; i < 6; ++i) acc[c][i] = 0.f;
+    float x[2][C][4], rv[4];
+    constexpr bool kP = C <= kGramRegs;
+    auto own_rows = [&]() {   // P's own rows and r, for the Gram sums
 #pragma unroll
-      for (int c = 0; c < C; ++c) Vec<float>::load_keep(X + (long long)c * g.cp + idx + ro, x[k & 1][c]);
+      for (int c = 0; c < C; ++c) Vec<float>::load_keep(X + (long long)c * g.cp + idx, x[R & 1][c]);
+      Vec<float>::load_keep(r + idx, rv);
     };
-    load_kappa<DIM>(k32, idx, g.px, g.pxy, kq);
-    load(0);
+    if (active) {
+      float kq[DIM == 3 ? 4 : 2][5];
+      auto load = [&](int k) {
+        const long long ro = (k % 3 - 1) * (long long)g.px + (DIM == 3 ? (k / 3 - 1) * g.pxy : 0);
 #pragma unroll
-    for (int k = 0; k < R; ++k) {
-      if (k + 1 < R) load(k + 1);
-      float cl[4], cc[4], cr[4];
-      mf_row_coeffs<DIM>(kq, k, cl, cc, cr);
+        for (int c = 0; c < C; ++c) Vec<float>::load_keep(X + (long long)c * g.cp + idx + ro, x[k & 1][c]);
+      };
+      load_kappa<DIM>(k32, idx, g.px, g.pxy, kq);
+      load(0);
 #pragma unroll
-      for (int c = 0; c < C; ++c) mf_row_products<DIM>(k, cl, cc, cr, x[k & 1][c], acc[c]);
+      for (int k = 0; k < R; ++k) {
+        if (k + 1 < R) load(k + 1);
+        else if (kP) own_rows();
+        float cl[4], cc[4], cr[4];
+        mf_row_coeffs<DIM>(kq, k, cl, cc, cr);
+#pragma unroll
+        for (int c = 0; c < C; ++c) mf_row_products<DIM>(k, cl, cc, cr, x[k & 1][c], acc[c]);
+      }
     }
-  }
-  int x0 = 0, y = 0, z = 0, a;
-  if (store) decode(g, q * 4, x0, y, z, a);
-  const bool row_in = y < g.ny && (DIM == 2 || z < g.nz);
+    int x0 = 0, y = 0, z = 0, a;
+    if (store) decode(g, q * 4, x0, y, z, a);
+    const bool row_in = y < g.ny && (DIM == 2 || z < g.nz);
+    float o[C][4];
 #pragma unroll
-  for (int c = 0; c < C; ++c) {
-    edge_shift(acc[c], lane);
-    float o[4];
+    for (int c = 0; c < C; ++c) {
+      edge_shift(acc[c], lane);
 #pragma unroll
-    for (int w = 0; w < 4; ++w) o[w] = row_in && x0 + w < g.nx ? acc[c][w + 1] : 0.f;   // pad points: zero rows
-    if (store) Vec<float>::store(Y + (long long)c * g.cp + idx, o);
+      for (int w = 0; w < 4; ++w) o[c][w] = row_in && x0 + w < g.nx ? acc[c][w + 1] : 0.f;   // pad points: zero rows
+      if (store) Vec<float>::store(Y + (long long)c * g.cp + idx, o[c]);
+    }
+    if (!kP && store) Vec<float>::load_keep(r + idx, rv);
+    gram_add<C>(
+        [&](int a, float(&v)[4]) {
+          if constexpr (kP) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i) v[i] = x[R & 1][a][i];
+          } else {
+            Vec<float>::load_keep(X + (long long)a * g.cp + idx, v);
+          }
+        },
+        rv, o, store, hold, base, nvalid, lane);
   }
+  gram_store<NV>(hold, base, nvalid, part + (long long)pb * NV * gridDim.x);
 }
 
 // Two damped-Jacobi sweeps from zero on the fine grid, fused (as k_jacobi
@@ -293,26 +319,27 @@ mpcg_status place_kappa(const GridDesc& g, const double* kappa, int ne, double h
 }
 
 template <int DIM>
-static bool spmm_mf(const GridDesc& g, const float* k32, const SpmmIO<float>& io, int C, const DevState* state,
-                    cudaStream_t s) {
+static int spmm_mf(const GridDesc& g, const float* k32, const SpmmIO<float>& io, int C, const float* r, double* part,
+                   const DevState* state, cudaStream_t s) {
   const RowMap map = row_map(g);
-  const int threads = spread_threads(32 * map.nwarps * g.nb);
-  const dim3 grid((unsigned)((32 * map.nwarps + threads - 1) / threads), g.nb);
-#define MPCG_MF_CASE(CC)                                                     \
-  case CC:                                                                   \
-    k_spmm_mf<DIM, CC><<<grid, threads, 0, s>>>(g, map, k32, io, state);     \
-    return true;
+  const RowLaunch l = row_launch(map);
+  const dim3 grid(l.blocks, g.nb);
+#define MPCG_MF_CASE(CC)                                                                     \
+  case CC:                                                                                   \
+    k_spmm_mf<DIM, CC><<<grid, l.threads, 0, s>>>(g, map, k32, io, r, part, state);          \
+    break;
   switch (C) {
     MPCG_MF_CASE(1) MPCG_MF_CASE(2) MPCG_MF_CASE(3) MPCG_MF_CASE(4) MPCG_MF_CASE(5) MPCG_MF_CASE(6)
     MPCG_MF_CASE(7) MPCG_MF_CASE(8) MPCG_MF_CASE(9) MPCG_MF_CASE(10) MPCG_MF_CASE(11) MPCG_MF_CASE(12)
-    default: return false;
+    default: break;
   }
 #undef MPCG_MF_CASE
+  return l.blocks;
 }
 
-bool launch_spmm_mf(const GridDesc& g, const float* k32, const SpmmIO<float>& io, int C, const DevState* state,
-                    cudaStream_t s) {
-  return g.dim == 3 ? spmm_mf<3>(g, k32, io, C, state, s) : spmm_mf<2>(g, k32, io, C, state, s);
+int launch_spmm_mf(const GridDesc& g, const float* k32, const SpmmIO<float>& io, int C, const float* r, double* part,
+                   const DevState* state, cudaStream_t s) {
+  return g.dim == 3 ? spmm_mf<3>(g, k32, io, C, r, part, state, s) : spmm_mf<2>(g, k32, io, C, r, part, state, s);
 }
 
 void launch_jacobi_mf(const GridDesc& g, const float* k32, const float* dinv, const float* r, float* out,

@@ -18,6 +18,7 @@
 // sum has the same products in the same order either way.
 #pragma once
 
+#include "kernels.cuh"
 #include "vec.cuh"
 
 namespace mpcg {
@@ -39,6 +40,83 @@ __device__ __forceinline__ void row_group(const RowMap& m, long long w, int lane
   q = m.stride == 32 ? w * 32 + lane : w * 30 + lane - 1;
   active = q >= 0 && q < ngroups;
   store = active && (m.stride == 32 || (lane > 0 && lane < 31));
+}
+
+// Warps of one problem's launch (the same for a problem alone and in a batch:
+// the partial sums below follow them): a warp per segment up to two blocks of
+// eight per SM, which then walk the segments (with sixteen blocks per SM the
+// block sums cost more than the balance gains: 1025^2, C = 9 32.7 against 28.6
+// us, matrix-free 113^3 35.9 against 28.8).
+struct RowLaunch {
+  int blocks, threads;
+};
+inline RowLaunch row_launch(const RowMap& m) {
+  RowLaunch l;
+  l.threads = spread_threads(32 * m.nwarps);
+  const long long need = (32 * m.nwarps + l.threads - 1) / l.threads;
+  const int cap = 2 * (sm_count() > 0 ? sm_count() : 152) * (kBlock / l.threads);
+  l.blocks = (int)(need < cap ? need : cap);
+  return l;
+}
+
+// Gram sums of the new block beside the product that forms it: with the lane's
+// four values of every A p_c in o, the upper triangle of P^T A P and P^T r over
+// its points, summed over the warp in FP32 and added to `hold` in FP64 (value
+// base + i of the lane's i-th, as warp_reduce_scatter deals them).  p(a, v)
+// gives the values of P's column a.  A kernel of its own reads P, A P and r from
+// memory again (1025^2, C = 9: 23.5 + 16.3 us against 28.6 together, 257^2 batch,
+// C = 7: 20.4 + 18.4 against 28.6, matrix-free 113^3, C = 5: 28.6 + 12.2 against
+// 28.7, 33^3 8 + 6 against 8).
+template <int C, typename P>
+__device__ __forceinline__ void gram_add(P p, const float (&rv)[4], const float (&o)[C][4], bool store,
+                                         double (&hold)[rs_count(C * (C + 1) / 2 + C, 5)], int& base, int& nvalid,
+                                         int lane) {
+  constexpr int NG = C * (C + 1) / 2;
+  float v[NG + C];
+#pragma unroll
+  for (int i = 0; i < NG + C; ++i) v[i] = 0.f;
+  if (store) {
+    int k = 0;
+#pragma unroll
+    for (int a = 0; a < C; ++a) {
+      float pa[4];
+      p(a, pa);
+#pragma unroll
+      for (int b = a; b < C; ++b) {
+#pragma unroll
+        for (int w = 0; w < 4; ++w) v[k] = fmaf(pa[w], o[b][w], v[k]);
+        ++k;
+      }
+#pragma unroll
+      for (int w = 0; w < 4; ++w) v[NG + a] = fmaf(pa[w], rv[w], v[NG + a]);
+    }
+  }
+  warp_reduce_scatter<float, NG + C>(v, base, nvalid, lane);
+#pragma unroll
+  for (int i = 0; i < rs_count(NG + C, 5); ++i) hold[i] += (double)v[i];
+}
+// Columns up to which P's own rows are loaded again as one more row of the
+// product's pipeline and kept in registers for gram_add; wider blocks would
+// spill and read them one column at a time.
+constexpr int kGramRegs = 6;
+
+// the block's sums of the warps' `hold` to part[value * gridDim.x + blockIdx.x];
+// every thread of the block calls it
+template <int NV>
+__device__ __forceinline__ void gram_store(const double (&hold)[rs_count(NV, 5)], int base, int nvalid, double* part) {
+  __shared__ double sh[kBlock / 32][NV];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  for (int i = lane; i < NV; i += 32) sh[warp][i] = 0.0;   // a warp without a segment holds nothing
+  __syncwarp();
+#pragma unroll
+  for (int i = 0; i < rs_count(NV, 5); ++i)
+    if (i < nvalid) sh[warp][base + i] = hold[i];
+  __syncthreads();
+  for (int i = threadIdx.x; i < NV; i += blockDim.x) {
+    double s = 0.0;
+    for (int w = 0; w < nw; ++w) s += sh[w][i];
+    part[(long long)i * gridDim.x + blockIdx.x] = s;
+  }
 }
 
 // acc[1], acc[4] get the sums of the neighbour lanes

@@ -467,50 +467,81 @@ __global__ void __launch_bounds__(kBlock, 4) k_jacobi(GridDesc g, const T* __res
 // thread on twice the warps (64-72 us), one row at a time (78-82 us), a bulk L2
 // prefetch of the planes (62 us), blocks tiled over y and z (63-65 us; 97^3 30
 // against 27 us).
-template <int DIM, int C>
+// GRAM: X is the new block P and the partial sums of P^T A P and P^T r go to
+// part.
+template <int DIM, int C, bool GRAM>
 __global__ void __launch_bounds__(kBlock, C <= 3 ? 3 : 2) k_spmm_half(GridDesc g, RowMap map,
                                                                       const float* __restrict__ st, SpmmIO<float> io,
+                                                                      const float* __restrict__ r, double* part,
                                                                       const DevState* state) {
   const int pb = blockIdx.y;
   if (state && state[pb].done) return;
   const float* X;
   float* Y;
   spmm_operands(io, state + pb, X, Y);
-  constexpr int R = DIM == 3 ? 9 : 3;
+  constexpr int R = DIM == 3 ? 9 : 3, NV = C * (C + 1) / 2 + C;
   const int lane = threadIdx.x & 31;
-  const long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  if (w >= map.nwarps) return;
-  long long q;
-  bool active, store;
-  row_group(map, w, lane, g.npts / 4, q, active, store);
-  const long long idx = (long long)pb * g.len + g.G + q * 4;
-  float acc[C][6];
+  const long long ngroups = g.npts / 4, bo = (long long)pb * g.len + g.G;
+  double hold[rs_count(NV, 5)] = {};
+  int base = 0, nvalid = 0;
+  for (long long w = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5; w < map.nwarps;
+       w += (long long)gridDim.x * (blockDim.x >> 5)) {
+    long long q;
+    bool active, store;
+    row_group(map, w, lane, ngroups, q, active, store);
+    const long long idx = bo + q * 4;
+    float acc[C][6];
 #pragma unroll
-  for (int c = 0; c < C; ++c)
+    for (int c = 0; c < C; ++c)
 #pragma unroll
-    for (int k = 0; k < 6; ++k) acc[c][k] = 0.f;
-  if (active) {
-    float cl[2][4], cc[2][4], cr[2][4], x[2][C][4];
-    auto load = [&](int k) {
-      const long long ro = row_offset<DIM>(k, g.px, g.pxy);
-      half_row_coeffs<DIM>(st, g.cp, idx, ro, k, cl[k & 1], cc[k & 1], cr[k & 1]);
+      for (int k = 0; k < 6; ++k) acc[c][k] = 0.f;
+    float x[2][C][4], rv[4];
+    constexpr bool kP = GRAM && C <= kGramRegs;
+    auto own_rows = [&]() {   // P's own rows and r, for the Gram sums
 #pragma unroll
-      for (int c = 0; c < C; ++c) Vec<float>::load_keep(X + (long long)c * g.cp + idx + ro, x[k & 1][c]);
+      for (int c = 0; c < C; ++c) Vec<float>::load_keep(X + (long long)c * g.cp + idx, x[R & 1][c]);
+      Vec<float>::load_keep(r + idx, rv);
     };
-    load(0);
+    if (active) {
+      float cl[2][4], cc[2][4], cr[2][4];
+      auto load = [&](int k) {
+        const long long ro = row_offset<DIM>(k, g.px, g.pxy);
+        half_row_coeffs<DIM>(st, g.cp, idx, ro, k, cl[k & 1], cc[k & 1], cr[k & 1]);
 #pragma unroll
-    for (int k = 0; k < R; ++k) {
-      if (k + 1 < R) load(k + 1);
+        for (int c = 0; c < C; ++c) Vec<float>::load_keep(X + (long long)c * g.cp + idx + ro, x[k & 1][c]);
+      };
+      load(0);
 #pragma unroll
-      for (int c = 0; c < C; ++c) row_products(cl[k & 1], cc[k & 1], cr[k & 1], x[k & 1][c], acc[c]);
+      for (int k = 0; k < R; ++k) {
+        if (k + 1 < R) load(k + 1);
+        else if (kP) own_rows();
+#pragma unroll
+        for (int c = 0; c < C; ++c) row_products(cl[k & 1], cc[k & 1], cr[k & 1], x[k & 1][c], acc[c]);
+      }
+    }
+    float o[C][4];
+#pragma unroll
+    for (int c = 0; c < C; ++c) {
+      edge_shift(acc[c], lane);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) o[c][i] = acc[c][i + 1];
+      if (store) Vec<float>::store(Y + (long long)c * g.cp + idx, o[c]);
+    }
+    if constexpr (GRAM) {
+      if (!kP && store) Vec<float>::load_keep(r + idx, rv);
+      gram_add<C>(
+          [&](int a, float(&v)[4]) {
+            if constexpr (kP) {
+#pragma unroll
+              for (int i = 0; i < 4; ++i) v[i] = x[R & 1][a][i];
+            } else {
+              Vec<float>::load_keep(X + (long long)a * g.cp + idx, v);
+            }
+          },
+          rv, o, store, hold, base, nvalid, lane);
     }
   }
-#pragma unroll
-  for (int c = 0; c < C; ++c) {
-    edge_shift(acc[c], lane);
-    const float o[4] = {acc[c][1], acc[c][2], acc[c][3], acc[c][4]};
-    if (store) Vec<float>::store(Y + (long long)c * g.cp + idx, o);
-  }
+  if constexpr (GRAM) gram_store<NV>(hold, base, nvalid, part + (long long)pb * NV * gridDim.x);
 }
 
 // Two damped-Jacobi sweeps from zero on the symmetric half (mode 1 of
@@ -1702,14 +1733,20 @@ void launch_sym_half(const GridDesc& g, const double* st, float* half, cudaStrea
 }
 
 template <int DIM>
-static void spmm_half(const GridDesc& g, const float* half, const SpmmIO<float>& io, int C, const DevState* state,
-                      cudaStream_t s) {
+static int spmm_half(const GridDesc& g, const float* half, const SpmmIO<float>& io, int C, const float* r, double* part,
+                     const DevState* state, cudaStream_t s) {
   const RowMap map = row_map(g);
-  const int threads = spread_threads(32 * map.nwarps * g.nb);
-  const dim3 grid((unsigned)((32 * map.nwarps + threads - 1) / threads), g.nb);
-#define MPCG_SPMM_CASE(CC)                                                   \
-  case CC:                                                                   \
-    k_spmm_half<DIM, CC><<<grid, threads, 0, s>>>(g, map, half, io, state);  \
+  const RowLaunch l = row_launch(map);
+  // With the 14 planes of a large 3D grid the product's loads fill the registers
+  // and the Gram sums cost as much as a launch of their own (129^3, C = 6: 88 us
+  // against 62 + 22); up to a segment per warp, two blocks per SM, they are free.
+  const bool alone = part && DIM == 3 && map.nwarps > 16LL * (sm_count() > 0 ? sm_count() : 152);
+  if (alone) part = nullptr;
+  const dim3 grid((unsigned)(part ? l.blocks : (32 * map.nwarps + l.threads - 1) / l.threads), g.nb);
+#define MPCG_SPMM_CASE(CC)                                                                                \
+  case CC:                                                                                                \
+    if (part) k_spmm_half<DIM, CC, true><<<grid, l.threads, 0, s>>>(g, map, half, io, r, part, state);    \
+    else k_spmm_half<DIM, CC, false><<<grid, l.threads, 0, s>>>(g, map, half, io, r, part, state);        \
     break;
   switch (C) {
     MPCG_SPMM_CASE(1) MPCG_SPMM_CASE(2) MPCG_SPMM_CASE(3) MPCG_SPMM_CASE(4) MPCG_SPMM_CASE(5)
@@ -1718,13 +1755,14 @@ static void spmm_half(const GridDesc& g, const float* half, const SpmmIO<float>&
     default: break;
   }
 #undef MPCG_SPMM_CASE
+  return part ? l.blocks : 0;
 }
 
-void launch_spmm_sym(const GridDesc& g, const float* half, const SpmmIO<float>& io, int C, const DevState* state,
-                     cudaStream_t s) {
-  if (g.ncomp != 1) return;
-  if (g.dim == 3) spmm_half<3>(g, half, io, C, state, s);
-  else spmm_half<2>(g, half, io, C, state, s);
+int launch_spmm_sym(const GridDesc& g, const float* half, const SpmmIO<float>& io, int C, const float* r, double* part,
+                    const DevState* state, cudaStream_t s) {
+  if (g.ncomp != 1) return 0;
+  return g.dim == 3 ? spmm_half<3>(g, half, io, C, r, part, state, s)
+                    : spmm_half<2>(g, half, io, C, r, part, state, s);
 }
 
 void launch_jacobi_sym(const GridDesc& g, const float* half, const float* dinv, const float* r, const float* sin,

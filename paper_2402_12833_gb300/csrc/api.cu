@@ -344,6 +344,17 @@ const float* dinv_of<float>(const Level& L) { return L.dinv32; }
 template <>
 const dw* dinv_of<dw>(const Level& L) { return L.dinvdw; }
 
+// The two damped-Jacobi sweeps of a scalar stencil grid in two launches, s1 =
+// dinv r and then the sweep from s1, instead of the fused one that forms s1 at
+// every neighbour (same values): the fused form does twice the arithmetic,
+// which bounds FP64 and double-word on all but small grids (fine grid of 97^3
+// FP64: 87 -> 65 us, of 129^3 double-word: 114 -> 88 us); below 2^16 points the
+// second launch costs as much as it saves.
+template <typename T>
+bool smooth_in_two(const GridDesc& g) {
+  return sizeof(T) == 8 && g.ncomp == 1 && g.npts >= (1LL << 16);
+}
+
 template <typename T>
 mpcg_status build_solver(mg_hierarchy* h, Solver<T>& S) {
   if (S.built) return MPCG_OK;
@@ -372,10 +383,9 @@ mpcg_status build_solver(mg_hierarchy* h, Solver<T>& S) {
       CKS(S.mem.get(&S.rlev[j], g.cp, s));
       CKS(S.mem.get(&S.zc[j], (size_t)(j + 1) * g.cp, s));
     }
-    if (h->opt.nu > 2 || (g.ncomp > 1 && h->opt.nu > 1) || h->opt.vcycle) {   // V-cycle: defects
-      CKS(S.mem.get(&S.tmp[j], g.cp, s));
-      CKS(S.mem.get(&S.tmp2[j], g.cp, s));
-    }
+    const bool both = h->opt.nu > 2 || (g.ncomp > 1 && h->opt.nu > 1) || h->opt.vcycle;   // V-cycle: defects
+    if (both || (!h->algebraic && smooth_in_two<T>(g))) CKS(S.mem.get(&S.tmp[j], g.cp, s));
+    if (both) CKS(S.mem.get(&S.tmp2[j], g.cp, s));
   }
   CKS(S.mem.get(&S.state, nb, s));
   // partial-sum slots for the most blocks a tuned launch shape may take
@@ -507,6 +517,9 @@ void enqueue_smooth(mg_hierarchy* h, Solver<T>& S, int j, const T* rr, T* out, c
   }
   if (nu == 1) {
     LAUNCH(h, K_JACOBI, s, jacobi_of<T>(L, st, di, rr, nullptr, out, 0, state, s));
+  } else if (nu == 2 && smooth_in_two<T>(L.g)) {
+    LAUNCH(h, K_JACOBI, s, jacobi_of<T>(L, st, di, rr, nullptr, S.tmp[j], 0, state, s));
+    LAUNCH(h, K_JACOBI, s, jacobi_of<T>(L, st, di, rr, S.tmp[j], out, 2, state, s));
   } else if (nu == 2) {
     LAUNCH(h, K_JACOBI, s, jacobi_of<T>(L, st, di, rr, nullptr, out, 1, state, s));
   } else {

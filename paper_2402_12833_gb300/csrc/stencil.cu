@@ -694,15 +694,16 @@ __global__ void __launch_bounds__(kBlock) k_add_to(GridDesc g, const T* __restri
 // and (g >> m) + 1 with weights 1 - f/s and f/s, f = g mod s (exact binary
 // fractions); coarse parents outside the grid are pad entries (zero).  One
 // launch writes columns 0 .. J-1 of Z (column J is the fine smoothing),
-// equal to successive two-grid prolongation up to the summation order.  The
-// grid count is a template parameter, so that every column's ratio s and
-// weights fold to constants (the kernel is bound by instruction issue).
+// equal to successive two-grid prolongation up to the summation order.
 template <typename T>
 struct CoarseSrc {
   const T* v[kMaxLevels];      // grid j's correction (padded, problem 0)
   GridDesc g[kMaxLevels];
 };
 
+// FP32: four points per thread (the grid count is a template parameter, so that
+// every column's ratio and weights fold to constants; bound by instruction
+// issue).
 template <typename T, int DIM, int JJ>
 __global__ void __launch_bounds__(kBlock) k_prolong_all(GridDesc gf, CoarseSrc<T> src, T* __restrict__ Z,
                                                         const DevState* state) {
@@ -762,6 +763,94 @@ __global__ void __launch_bounds__(kBlock) k_prolong_all(GridDesc gf, CoarseSrc<T
       o[w] = x0 + w < gf.nx ? v : (T)0;
     }
     Vec<T>::store(Z + (long long)j * gf.cp + idf, o);
+  }
+}
+
+// FP64 and double-word: the interpolation's arithmetic is the bound, so a warp
+// takes a segment of a fine row and first interpolates every coarse grid along y
+// and z at that row, once per coarse node (nx / s of them on grid j, about nx
+// over all grids), into shared memory together with the differences of
+// consecutive nodes; a fine point then is one multiply-add per column instead of
+// 8 to 12 (97^3 FP64 114 -> 29 us, 129^3 double-word 70 -> 33 us, 65^2 FP64 10
+// -> 8 us, event-timed; FP32 lost, 17 -> 24 us at 129^3, and keeps the form
+// above).  The same values as the form above.  Pad rows of Z are zero from its
+// allocation and stay so.
+constexpr int kProlongSeg = 256;                      // fine points of a warp's segment
+constexpr int kProlongBuf = kProlongSeg + 3 * kMaxLevels;
+constexpr int kFracLevels = 7;                        // fractions f / 2^m, m <= 7, from a table
+
+template <typename T, int DIM, int JJ>
+__global__ void __launch_bounds__(kBlock) k_prolong_rows(GridDesc gf, CoarseSrc<T> src, T* __restrict__ Z,
+                                                        const DevState* state) {
+  const int pb = blockIdx.y;
+  if (state && state[pb].done) return;
+  __shared__ T rows[kBlock / 32][kProlongBuf], diff[kBlock / 32][kProlongBuf];
+  __shared__ T frac[(2 << kFracLevels) - 2];          // f / 2^m at 2^m - 2 + f
+  constexpr int MT = JJ < kFracLevels ? JJ : kFracLevels;
+  for (int e = threadIdx.x; e < (2 << MT) - 2; e += blockDim.x) {
+    const int m = 31 - __clz(e + 2);
+    frac[e] = (T)((float)(e + 2 - (1 << m)) * (1.f / (float)(1 << m)));
+  }
+  __syncthreads();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  T* R = rows[warp];
+  T* D = diff[warp];
+  const unsigned nseg = (unsigned)((gf.nx + kProlongSeg - 1) / kProlongSeg);
+  const unsigned items = nseg * (unsigned)gf.ny * (unsigned)gf.nz * (unsigned)gf.ncomp;
+  for (unsigned it = blockIdx.x * (kBlock / 32) + warp; it < items; it += gridDim.x * (kBlock / 32)) {
+    const unsigned row = it / nseg;
+    const int x0 = (int)(it - row * nseg) * kProlongSeg;
+    const unsigned yz = row / (unsigned)gf.ny;
+    const int y = (int)(row - yz * (unsigned)gf.ny);
+    const int comp = (int)(yz / (unsigned)gf.nz), z = (int)(yz - (unsigned)comp * (unsigned)gf.nz);
+    const int x1 = x0 + kProlongSeg < gf.nx ? x0 + kProlongSeg : gf.nx;
+    const int gx0 = x0 + gf.lox, gx1 = x1 - 1 + gf.lox;   // first and last global node
+    const int gy = y + gf.loy, gz = DIM == 3 ? z + gf.loz : 0;
+    // grid j's nodes gx0 >> m .. (gx1 >> m) + 1 at off[j] .. off[j + 1] - 1
+    int off[JJ + 1];
+    off[0] = 0;
+#pragma unroll
+    for (int j = 0; j < JJ; ++j) off[j + 1] = off[j] + (gx1 >> (JJ - j)) - (gx0 >> (JJ - j)) + 2;
+    for (int e = lane; e < off[JJ]; e += 32) {
+      int j = 0, o = 0;
+#pragma unroll
+      for (int k = 1; k < JJ; ++k)
+        if (e >= off[k]) {
+          j = k;
+          o = off[k];
+        }
+      const int m = JJ - j, sm1 = (1 << m) - 1;
+      const float inv_s = 1.f / (float)(1 << m);          // exact: a power of two
+      const GridDesc& gc = src.g[j];
+      const float wy1 = (float)(gy & sm1) * inv_s, wz1 = DIM == 3 ? (float)(gz & sm1) * inv_s : 0.f;
+      const T* p = src.v[j] + (long long)pb * gc.len + gc.G + (long long)comp * gc.cstride +
+                   ((gx0 >> m) + (e - o) - gc.lox) + gc.px * (long long)((gy >> m) - gc.loy) +
+                   (DIM == 3 ? gc.pxy * (long long)((gz >> m) - gc.loz) : 0);
+      T v = 0;
+#pragma unroll
+      for (int kz = 0; kz < (DIM == 3 ? 2 : 1); ++kz) {
+        const float wz = DIM == 3 ? (kz ? wz1 : 1.f - wz1) : 1.f;
+#pragma unroll
+        for (int ky = 0; ky < 2; ++ky)   // the weights' products are exact in FP32
+          v = fma((T)(wz * (ky ? wy1 : 1.f - wy1)), p[gc.px * (long long)ky + (DIM == 3 ? gc.pxy * (long long)kz : 0)], v);
+      }
+      R[e] = v;
+    }
+    __syncwarp();
+    for (int e = lane; e < off[JJ] - 1; e += 32) D[e] = R[e + 1] - R[e];   // unused between two grids
+    __syncwarp();
+    T* zp = Z + (long long)pb * gf.len + gf.G + (long long)comp * gf.cstride + (long long)gf.px * y +
+            (DIM == 3 ? gf.pxy * z : 0);
+    for (int x = x0 + lane; x < x1; x += 32) {
+      const int gx = x + gf.lox;
+#pragma unroll
+      for (int j = 0; j < JJ; ++j) {
+        const int m = JJ - j, f = gx & ((1 << m) - 1), e = off[j] + (gx >> m) - (gx0 >> m);
+        const T fr = m <= kFracLevels ? frac[(1 << m) - 2 + f] : (T)((float)f * (1.f / (float)(1 << m)));
+        zp[(long long)j * gf.cp + x] = fma(fr, D[e], R[e]);
+      }
+    }
+    __syncwarp();
   }
 }
 
@@ -1628,12 +1717,24 @@ void launch_prolong_all(const GridDesc& gf, const T* const* coarse, const GridDe
     src.v[j] = coarse[j];
     src.g[j] = gcs[j];
   }
-  const dim3 grid(blocks_for(gf.npts / vw<T>()), gf.nb);
+  unsigned blocks = (unsigned)blocks_for(gf.npts / vw<T>());
+  if (sizeof(T) == 8) {
+    const long long items = (long long)((gf.nx + kProlongSeg - 1) / kProlongSeg) * gf.ny * gf.nz * gf.ncomp;
+    const long long need = (items + kBlock / 32 - 1) / (kBlock / 32);
+    const int cap = 8 * (sm_count() > 0 ? sm_count() : 152);
+    blocks = (unsigned)(need < cap ? need : cap);
+  }
+  const dim3 grid(blocks, gf.nb);
   static_assert(kMaxLevels <= 12, "the switch below covers up to 11 coarse grids");
 #define MPCG_PROLONG_CASE(JJ)                                                                   \
   case JJ:                                                                                      \
-    if (gf.dim == 3) k_prolong_all<T, 3, JJ><<<grid, kBlock, 0, s>>>(gf, src, Z, state);       \
-    else k_prolong_all<T, 2, JJ><<<grid, kBlock, 0, s>>>(gf, src, Z, state);                   \
+    if constexpr (sizeof(T) == 8) {                                                             \
+      if (gf.dim == 3) k_prolong_rows<T, 3, JJ><<<grid, kBlock, 0, s>>>(gf, src, Z, state);    \
+      else k_prolong_rows<T, 2, JJ><<<grid, kBlock, 0, s>>>(gf, src, Z, state);                \
+    } else {                                                                                    \
+      if (gf.dim == 3) k_prolong_all<T, 3, JJ><<<grid, kBlock, 0, s>>>(gf, src, Z, state);     \
+      else k_prolong_all<T, 2, JJ><<<grid, kBlock, 0, s>>>(gf, src, Z, state);                 \
+    }                                                                                           \
     break;
   switch (J) {
     MPCG_PROLONG_CASE(1) MPCG_PROLONG_CASE(2) MPCG_PROLONG_CASE(3) MPCG_PROLONG_CASE(4) MPCG_PROLONG_CASE(5)

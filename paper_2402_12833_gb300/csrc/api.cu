@@ -775,7 +775,7 @@ void enqueue_prologue(mg_hierarchy* h, Solver<T>& S, cudaGraphConditionalHandle 
 
 // A P of the block being built (the ring slot after the newest) and the partial
 // sums of P^T A P and P^T r: with the product where its kernel forms them (the
-// FP32 scalar stencils), else in a launch of their own.  Returns the slots per
+// FP32 scalar stencils and sparse operators), else in a launch of their own.  Returns the slots per
 // value of part_G.
 template <typename T>
 int enqueue_block_product(mg_hierarchy* h, Solver<T>& S, cudaStream_t s) {
@@ -783,8 +783,12 @@ int enqueue_block_product(mg_hierarchy* h, Solver<T>& S, cudaStream_t s) {
   const int C = S.C;
   int slots = 0;
   if (h->algebraic) {
-    LAUNCH(h, K_SPMM, s,
-           launch_ell_spmm<T>(ell_of<T>(L.eA), spmm_ring(S.win, S.m, L.g.G), L.g.cp, L.g.cp, C, S.state, s));
+    const SpmmIO<T> io = spmm_ring(S.win, S.m, L.g.G);
+    if constexpr (std::is_same<T, float>::value)
+      LAUNCH(h, K_SPMM, s,
+             slots = launch_ell_spmm_gram(ell_of<T>(L.eA), io, L.g.cp, C, S.r + L.g.G, S.part_G, S.state, s));
+    else
+      LAUNCH(h, K_SPMM, s, launch_ell_spmm<T>(ell_of<T>(L.eA), io, L.g.cp, L.g.cp, C, S.state, s));
   } else {
     const SpmmIO<T> io = spmm_ring(S.win, S.m);
     bool done = false;

@@ -29,14 +29,22 @@ __device__ __forceinline__ T group_sum(T v, int lg) {
 }
 
 // Y[:, c] = A X[:, c] (ADD: Y[:, c] += A X[:, c]) for C columns (column
-// pitches ldx, ldy).
-template <typename T, int C, bool ADD = false>
+// pitches ldx, ldy).  GRAM: X is the new block P, and the partial sums of P^T A P
+// (upper triangle) and P^T r go to part, value-major, a slot per block: the row's
+// lane holds A p and needs one load per column and r (a launch of its own: 8 us
+// on the 296,480-unknown fracture matrix, whose iteration is a chain of
+// launches that short).
+template <typename T, int C, bool ADD = false, bool GRAM = false>
 __global__ void __launch_bounds__(kBlock) k_ell_spmm(EllDev<T> A, SpmmIO<T> io, long long ldx, long long ldy,
-                                                     const DevState* state) {
+                                                     const T* __restrict__ rv, double* part, const DevState* state) {
   if (state && state[0].done) return;
   const T* X;
   T* Y;
   spmm_operands(io, state, X, Y);
+  constexpr int NG = C * (C + 1) / 2, NV = GRAM ? NG + C : 1;
+  T sum[NV];
+#pragma unroll
+  for (int i = 0; i < NV; ++i) sum[i] = 0;
   const long long nt = (long long)A.nslices * 32;
   for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < nt; t += (long long)gridDim.x * blockDim.x) {
     const int s = (int)(t >> 5), lane = (int)(t & 31);
@@ -62,8 +70,23 @@ __global__ void __launch_bounds__(kBlock) k_ell_spmm(EllDev<T> A, SpmmIO<T> io, 
         if (ADD) Y[c * ldy + r] += acc[c];
         else Y[c * ldy + r] = acc[c];
       }
+      if constexpr (GRAM) {
+        const T rr = rv[r];
+        int k = 0;
+#pragma unroll
+        for (int a = 0; a < C; ++a) {
+          const T p = X[a * ldx + r];
+#pragma unroll
+          for (int c = a; c < C; ++c) {
+            sum[k] = fma(p, acc[c], sum[k]);
+            ++k;
+          }
+          sum[NG + a] = fma(p, rr, sum[NG + a]);
+        }
+      }
     }
   }
+  if constexpr (GRAM) block_sum_store<T, NV>(sum, part, gridDim.x, blockIdx.x);
 }
 
 // r = b - A x with the partials of |r|^2 and |b|^2 (NORMS; without them it
@@ -147,7 +170,7 @@ void launch_ell_spmm(const EllDev<T>& A, const SpmmIO<T>& io, long long ldx, lon
   const int grid = ell_threads_blocks(A);
 #define MPCG_ELL_CASE(CC)                                                                                \
   case CC:                                                                                               \
-    k_ell_spmm<T, CC><<<grid, kBlock, 0, s>>>(A, io, ldx, ldy, state);                                   \
+    k_ell_spmm<T, CC><<<grid, kBlock, 0, s>>>(A, io, ldx, ldy, nullptr, nullptr, state);                 \
     break;
   switch (C) {
     MPCG_ELL_CASE(1) MPCG_ELL_CASE(2) MPCG_ELL_CASE(3) MPCG_ELL_CASE(4) MPCG_ELL_CASE(5) MPCG_ELL_CASE(6)
@@ -162,6 +185,24 @@ template void launch_ell_spmm<float>(const EllDev<float>&, const SpmmIO<float>&,
                                      const DevState*, cudaStream_t);
 template void launch_ell_spmm<dw>(const EllDev<dw>&, const SpmmIO<dw>&, long long, long long, int, const DevState*,
                                   cudaStream_t);
+
+int launch_ell_spmm_gram(const EllDev<float>& A, const SpmmIO<float>& io, long long ld, int C, const float* r,
+                         double* part, const DevState* state, cudaStream_t s) {
+  // at most eight blocks per SM: the slots the solver reserves
+  const int cap = 8 * (sm_count() > 0 ? sm_count() : 152), need = ell_threads_blocks(A);
+  const int grid = need < cap ? need : cap;
+#define MPCG_ELL_CASE(CC)                                                                                \
+  case CC:                                                                                               \
+    k_ell_spmm<float, CC, false, true><<<grid, kBlock, 0, s>>>(A, io, ld, ld, r, part, state);           \
+    break;
+  switch (C) {
+    MPCG_ELL_CASE(1) MPCG_ELL_CASE(2) MPCG_ELL_CASE(3) MPCG_ELL_CASE(4) MPCG_ELL_CASE(5) MPCG_ELL_CASE(6)
+    MPCG_ELL_CASE(7) MPCG_ELL_CASE(8) MPCG_ELL_CASE(9) MPCG_ELL_CASE(10) MPCG_ELL_CASE(11) MPCG_ELL_CASE(12)
+    default: break;
+  }
+#undef MPCG_ELL_CASE
+  return grid;
+}
 
 template <typename T>
 void launch_ell_residual(const EllDev<T>& A, const T* b, const T* x, T* r, double* part, int nblocks, int threads,
@@ -181,7 +222,7 @@ template void launch_ell_defect<float>(const EllDev<float>&, const float*, const
 
 template <typename T>
 void launch_ell_spmv_add(const EllDev<T>& A, const T* X, T* Y, const DevState* state, cudaStream_t s) {
-  k_ell_spmm<T, 1, true><<<ell_threads_blocks(A), kBlock, 0, s>>>(A, spmm_io(X, Y), 0, 0, state);
+  k_ell_spmm<T, 1, true><<<ell_threads_blocks(A), kBlock, 0, s>>>(A, spmm_io(X, Y), 0, 0, nullptr, nullptr, state);
 }
 template void launch_ell_spmv_add<double>(const EllDev<double>&, const double*, double*, const DevState*,
                                           cudaStream_t);

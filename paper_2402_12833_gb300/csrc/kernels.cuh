@@ -69,6 +69,10 @@ inline int grid_for(long long work, int cap) {
 template <typename T>
 void launch_ell_spmm(const EllDev<T>& A, const SpmmIO<T>& io, long long ldx, long long ldy, int C,
                      const DevState* state, cudaStream_t s);
+// the FP32 product with launch_block_gram's partial sums for X = P (column pitch
+// ld for both); returns the slots per value
+int launch_ell_spmm_gram(const EllDev<float>& A, const SpmmIO<float>& io, long long ld, int C, const float* r,
+                         double* part, const DevState* state, cudaStream_t s);
 // r = b - A x, partials [|r|^2, |b|^2] over nblocks blocks; xnz as launch_residual
 template <typename T>
 void launch_ell_residual(const EllDev<T>& A, const T* b, const T* x, T* r, double* part, int nblocks, int threads,

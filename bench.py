@@ -1079,7 +1079,9 @@ def amg_roofline(trace, ns, nnzA, nnzP, C, m, w, peaks):
     padding excluded) plus the vectors it reads and writes once.  Launch
     order per iteration (one stream): Jacobi J, restriction J, Jacobi J-1,
     restriction J-1, ..., Jacobi 1, restriction 1, coarse solve,
-    prolongations P_1 .. P_J (k columns each), then the block kernels."""
+    prolongations P_1 .. P_J (k columns each), then the block kernels; a small
+    grid 1 has the coarse solve and its transfers as one launch and the
+    prolongations start at P_2."""
     J = len(ns) - 1
     tot = {}
     for cls, ms in trace:

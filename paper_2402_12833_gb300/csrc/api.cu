@@ -3094,9 +3094,11 @@ mpcg_status mg_learned_train(mg_hierarchy* const* hs, int nprob, const int* pair
   // training set in the padded layout, and A e per pair (FP32 operators)
   launch_pack<float, float>(g, rhat_dev, g.n, R, npairs, s);
   launch_pack<float, float>(g, e_dev, g.n, E, npairs, s);
-  for (int i = 0; i < npairs; ++i) {
+  for (int i = 0, n = 0; i < npairs; i += n) {   // consecutive pairs of a problem are columns of one product
+    n = 1;
+    while (i + n < npairs && n < (net3 ? kMaxVecCols : MPCG_MAX_COLS) && pair_prob[i + n] == pair_prob[i]) ++n;
     const Level& Lp = hs[pair_prob[i]]->lev[hs[pair_prob[i]]->levels - 1];
-    launch_spmm<float>(g, Lp.st32, spmm_io<float>(E + (size_t)i * L, AE + (size_t)i * L), 1, nullptr, s);
+    launch_spmm<float>(g, Lp.st32, spmm_io<float>(E + (size_t)i * L, AE + (size_t)i * L), n, nullptr, s);
   }
   // batches: pairs grouped by problem, shuffled within a problem and across
   // batches by a seeded 64-bit LCG (Knuth's MMIX constants)
@@ -3119,11 +3121,7 @@ mpcg_status mg_learned_train(mg_hierarchy* const* hs, int nprob, const int* pair
     cudaMemsetAsync(loss, 0, sizeof(double), s);
     for (auto& bt : batches) {
       const int nb = (int)bt.size();
-      for (int k = 0; k < nb; ++k) {
-        cudaMemcpyAsync(nbt.rb + k * L, R + (size_t)bt[k] * L, sizeof(float) * L, cudaMemcpyDeviceToDevice, s);
-        cudaMemcpyAsync(nbt.eb + k * L, E + (size_t)bt[k] * L, sizeof(float) * L, cudaMemcpyDeviceToDevice, s);
-        cudaMemcpyAsync(nbt.aeb + k * L, AE + (size_t)bt[k] * L, sizeof(float) * L, cudaMemcpyDeviceToDevice, s);
-      }
+      launch_net_gather(bt.data(), nb, (long long)L, R, E, AE, nbt.rb, nbt.eb, nbt.aeb, s);
       mg_hierarchy* hp = hs[pair_prob[bt[0]]];
       net_batch_step(nbt, g, nb, hp->net_c, hp->lev[hp->levels - 1].st32, wq, loss, s);
       ++step;

@@ -366,6 +366,10 @@ void launch_net_loss_grad(const GridDesc& g, int B, const float* y, const float*
 void launch_net_adam(const double* const* parts_dev, int nblk, int net3, float* master, float* m, float* v, float* wq,
                      int step, float lr, float b1, float b2, float eps, cudaStream_t s);
 void launch_round_bf16(const float* src, float* dst, int n, cudaStream_t s);
+// pairs idx[0 .. nb - 1] of the training set (len floats each) into the batch's
+// buffers
+void launch_net_gather(const int* idx, int nb, long long len, const float* R, const float* E, const float* AE,
+                       float* rb, float* eb, float* aeb, cudaStream_t s);
 // grad[i] = sum of the weight-gradient partials of parameter i (all layers)
 void launch_net_grad_sum(const double* const* parts_dev, int nblk, int net3, double* grad, cudaStream_t s);
 // activations a0..a3 of the training forward ([B][len][C] bfloat16, padded)

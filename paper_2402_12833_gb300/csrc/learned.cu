@@ -43,16 +43,20 @@ __global__ void __launch_bounds__(kBlock) k_net_dots(GridDesc g, const float* __
   block_sum_store<float, 3>(s, part + (long long)b * 3 * gridDim.x, gridDim.x, blockIdx.x);
 }
 
-// Loss per item and coefficients of dL/dy = -k1 (Ae - k2 Ay) / B.
+// Loss per item and coefficients of dL/dy = -k1 (Ae - k2 Ay) / B: a warp per
+// item, lanes over the partials (one thread per item: 17 us at 8 items of 64 partials; now 9).
 __global__ void k_net_loss(const double* part, int nblk, int B, double* coef, double* loss_sum) {
-  const int b = threadIdx.x;
-  if (b >= B) return;
+  const int b = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double d[3];
+#pragma unroll
   for (int v = 0; v < 3; ++v) {
     double a = 0.0;
-    for (int k = 0; k < nblk; ++k) a += part[((long long)b * 3 + v) * nblk + k];
+    for (int k = lane; k < nblk; k += 32) a += part[((long long)b * 3 + v) * nblk + k];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
     d[v] = a;
   }
+  if (lane != 0) return;
   const double eAy = d[0], eAe = d[1], yAy = d[2];
   const bool ok = eAe > 0.0 && yAy > 0.0;
   const double L = ok ? 1.0 - eAy * eAy / (eAe * yAy) : 1.0;
@@ -81,18 +85,28 @@ __device__ __forceinline__ int net_layer_size(int net3, int layer) {
   return layer == 0 ? kNetC1 * kNetIn * 9 : (layer == 3 ? kNetW * 9 : kNetW * kNetW * 9);
 }
 
-__global__ void k_net_adam(const double* const* parts, int nblk, int nparams, int net3, float* master, float* m,
-                           float* v, float* wq, int step, float lr, float b1, float b2, float eps) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nparams) return;
+// Sum of the partials of parameter i, over the warp (a thread per parameter
+// walked its partials one by one: 23 us for 5,040 parameters of 128 partials;
+// now 11 us for 296).
+__device__ __forceinline__ double net_grad_of(const double* const* parts, int nblk, int net3, int i, int lane) {
   int layer = 0, off = i;
   const int sizes[4] = {net_layer_size(net3, 0), net_layer_size(net3, 1), net_layer_size(net3, 2),
                         net_layer_size(net3, 3)};
   while (off >= sizes[layer]) off -= sizes[layer], ++layer;
-  double gsum = 0.0;
   const double* p = parts[layer] + (long long)off * nblk;
-  for (int k = 0; k < nblk; ++k) gsum += p[k];
-  const float gr = (float)gsum;
+  double a = 0.0;
+  for (int k = lane; k < nblk; k += 32) a += p[k];
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
+  return a;
+}
+
+__global__ void k_net_adam(const double* const* parts, int nblk, int nparams, int net3, float* master, float* m,
+                           float* v, float* wq, int step, float lr, float b1, float b2, float eps) {
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+  if (i >= nparams) return;
+  const float gr = (float)net_grad_of(parts, nblk, net3, i, lane);
+  if (lane != 0) return;
   const float mi = b1 * m[i] + (1.f - b1) * gr;
   const float vi = b2 * v[i] + (1.f - b2) * gr * gr;
   m[i] = mi;
@@ -105,16 +119,25 @@ __global__ void k_net_adam(const double* const* parts, int nblk, int nparams, in
 }
 
 __global__ void k_net_grad_sum(const double* const* parts, int nblk, int nparams, int net3, double* grad) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
   if (i >= nparams) return;
-  int layer = 0, off = i;
-  const int sizes[4] = {net_layer_size(net3, 0), net_layer_size(net3, 1), net_layer_size(net3, 2),
-                        net_layer_size(net3, 3)};
-  while (off >= sizes[layer]) off -= sizes[layer], ++layer;
-  double gsum = 0.0;
-  const double* p = parts[layer] + (long long)off * nblk;
-  for (int k = 0; k < nblk; ++k) gsum += p[k];
-  grad[i] = gsum;
+  const double a = net_grad_of(parts, nblk, net3, i, lane);
+  if (lane == 0) grad[i] = a;
+}
+
+// One batch of the training set, pairs idx[0 .. nb - 1] of R, E and A E (len
+// floats each, a multiple of 32), side by side: blockIdx.y = 3 k + array.
+struct BatchIndex {
+  int i[MPCG_MAX_COLS];
+};
+__global__ void k_net_gather(BatchIndex idx, long long len, const float* __restrict__ R, const float* __restrict__ E,
+                             const float* __restrict__ AE, float* __restrict__ rb, float* __restrict__ eb,
+                             float* __restrict__ aeb) {
+  const int k = blockIdx.y / 3, w = blockIdx.y % 3;
+  const float4* src = reinterpret_cast<const float4*>((w == 0 ? R : w == 1 ? E : AE) + idx.i[k] * len);
+  float4* dst = reinterpret_cast<float4*>((w == 0 ? rb : w == 1 ? eb : aeb) + k * len);
+  for (long long t = blockIdx.x * (long long)blockDim.x + threadIdx.x; t < len / 4; t += (long long)gridDim.x * blockDim.x)
+    dst[t] = src[t];
 }
 
 __global__ void k_net_acts_export(GridDesc g, int B, NetActs a, float* out) {
@@ -185,20 +208,27 @@ void launch_net_loss_grad(const GridDesc& g, int B, const float* y, const float*
                           const float* Ae, double* part, double* coef, double* loss_sum, float* dy, cudaStream_t s) {
   const int nblk = 64;
   k_net_dots<<<dim3(nblk, B), kBlock, 0, s>>>(g, y, Ay, e, Ae, part);
-  k_net_loss<<<1, 32, 0, s>>>(part, nblk, B, coef, loss_sum);
+  k_net_loss<<<1, 32 * B, 0, s>>>(part, nblk, B, coef, loss_sum);
   k_net_dy<<<grid_for((long long)B * g.len, 4096), kBlock, 0, s>>>(g, B, Ay, Ae, coef, dy);
 }
 
 void launch_net_adam(const double* const* parts_dev, int nblk, int net3, float* master, float* m, float* v, float* wq,
                      int step, float lr, float b1, float b2, float eps, cudaStream_t s) {
   const int np = net3 ? kNet3Params : kNetParams;
-  k_net_adam<<<(np + kBlock - 1) / kBlock, kBlock, 0, s>>>(parts_dev, nblk, np, net3, master, m, v, wq,
-                                                                   step, lr, b1, b2, eps);
+  k_net_adam<<<(32 * np + kBlock - 1) / kBlock, kBlock, 0, s>>>(parts_dev, nblk, np, net3, master, m, v, wq, step, lr,
+                                                                b1, b2, eps);
+}
+
+void launch_net_gather(const int* idx, int nb, long long len, const float* R, const float* E, const float* AE,
+                       float* rb, float* eb, float* aeb, cudaStream_t s) {
+  BatchIndex bi = {};
+  for (int k = 0; k < nb; ++k) bi.i[k] = idx[k];
+  k_net_gather<<<dim3(grid_for(len / 4, 256), 3 * nb), kBlock, 0, s>>>(bi, len, R, E, AE, rb, eb, aeb);
 }
 
 void launch_net_grad_sum(const double* const* parts_dev, int nblk, int net3, double* grad, cudaStream_t s) {
   const int np = net3 ? kNet3Params : kNetParams;
-  k_net_grad_sum<<<(np + kBlock - 1) / kBlock, kBlock, 0, s>>>(parts_dev, nblk, np, net3, grad);
+  k_net_grad_sum<<<(32 * np + kBlock - 1) / kBlock, kBlock, 0, s>>>(parts_dev, nblk, np, net3, grad);
 }
 
 void launch_net_acts_export(const GridDesc& g, int B, NetActs acts, float* out, cudaStream_t s) {

@@ -365,11 +365,21 @@ void launch_net_dgrad_tc(const GridDesc& g, int B, int cout, const float* dOut, 
   else k_net_dgrad_tc<16><<<grid, kWT, kDSmem, s>>>(g, dOut, W, act_in, dIn, err);
 }
 
-int net_wgrad_tc_chunks_per_block() { return 16; }
+// Chunks of a CTA: as many as give a batch of eight images two CTAs per SM (the
+// tensor memory's limit), at least two, at most 16.  A chunk is a serial chain
+// of staging and MMAs, so one CTA per SM with 16 chunks left the staging's
+// latency bare (129^2, batch of 8: 79 us a layer with 128 CTAs of 16, 52 us with
+// 296 of 7).  The rule depends on the grid alone, so that a short last batch
+// launches a part of the same CTAs.
+int net_wgrad_tc_chunks_per_block(long long nchunks) {
+  const int ctas = 2 * (sm_count() > 0 ? sm_count() : 152);
+  const long long c = (8 * nchunks + ctas - 1) / ctas;
+  return (int)(c < 2 ? 2 : (c > 16 ? 16 : c));
+}
 
 int net_wgrad_tc_blocks(const GridDesc& g, int B) {
   const long long nchunks = (g.npts + kChunk - 1) / kChunk;
-  const int cpb = net_wgrad_tc_chunks_per_block();
+  const int cpb = net_wgrad_tc_chunks_per_block(nchunks);
   return B * (int)((nchunks + cpb - 1) / cpb);
 }
 
@@ -388,7 +398,7 @@ void net_train_tc_prepare_attributes() {
 void launch_net_wgrad_tc(const GridDesc& g, int B, int layer, const float* dOut, const __nv_bfloat16* act,
                          double* part, int* err, cudaStream_t s) {
   const long long nchunks = (g.npts + kChunk - 1) / kChunk;
-  const int cpb = net_wgrad_tc_chunks_per_block();
+  const int cpb = net_wgrad_tc_chunks_per_block(nchunks);
   const int bpi = (int)((nchunks + cpb - 1) / cpb);
   const dim3 grid((unsigned)(B * bpi));
   if (layer == 3) k_net_wgrad_tc<kNetW, 1><<<grid, kWT, kWSmem, s>>>(g, cpb, bpi, dOut, act, part, err);

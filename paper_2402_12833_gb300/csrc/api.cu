@@ -108,6 +108,24 @@ struct Alloc {
     *p = (P*)q;
     return MPCG_OK;
   }
+  // Several arrays from one allocation, each on a 256-byte boundary and zeroed:
+  // calls that need many buffers pay for one cudaMalloc, memset and cudaFree.
+  struct Plan {
+    std::vector<std::pair<void**, size_t>> items;
+    size_t bytes = 0;
+    template <typename P>
+    void add(P** p, size_t count) {
+      items.emplace_back(reinterpret_cast<void**>(p), bytes);
+      bytes += (count * sizeof(P) + 255) / 256 * 256;
+    }
+  };
+  mpcg_status commit(const Plan& plan, cudaStream_t s) {
+    char* q = nullptr;
+    const mpcg_status st = get(&q, plan.bytes, s);
+    if (st == MPCG_OK)
+      for (const auto& it : plan.items) *it.first = q + it.second;
+    return st;
+  }
   void release() {
     for (void* p : ptrs) cudaFree(p);
     ptrs.clear();
@@ -281,6 +299,11 @@ struct mg_hierarchy {
   int* net_err = nullptr;      // set by the tensor-core inference kernel on a timed-out wait
   unsigned char* net_wtc = nullptr;   // weights packed for the tensor-core kernel
   Alloc net_mem;
+  // forward calls' residuals and outputs in the padded layout, kept up to
+  // kNetKeep bytes (larger calls allocate their own); given back on detach
+  Alloc net_ws;
+  float *net_r = nullptr, *net_y = nullptr;
+  int net_imgs = 0;
   // algebraic hierarchy (flat grids, ELL operators); host copies of its
   // matrices by grid index: A[j], P[j] (j >= 1), aggregates of grid j (j >= 1)
   bool algebraic = false;
@@ -1172,6 +1195,7 @@ void mg_hierarchy_destroy(mg_hierarchy* h) {
   h->mem.release();
   h->prof.release();
   h->net_mem.release();
+  h->net_ws.release();
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
   for (auto sd : h->side)
     if (sd) cudaStreamDestroy(sd);
@@ -2715,13 +2739,10 @@ int net_batch_blocks(const NetBatch& nb, const GridDesc& g, int nimg) {
   return nb.net3 ? net3_wgrad_blocks(g, nimg) : net_wgrad_tc_blocks(g, nimg);
 }
 
-mpcg_status net_batch_alloc(bool net3, const GridDesc& g, int B, Alloc& mem, cudaStream_t s, NetBatch& nb) {
+void net_batch_plan(bool net3, const GridDesc& g, int B, Alloc::Plan& plan, NetBatch& nb) {
   nb.net3 = net3;
   nb.np = net3 ? kNet3Params : kNetParams;
-  mpcg_status st = MPCG_OK;
-  auto get = [&](auto** p, size_t n) {
-    if (st == MPCG_OK) st = mem.get(p, n, s);
-  };
+  auto get = [&](auto** p, size_t n) { plan.add(p, n); };
   const size_t L = g.len;
   const size_t A = net3 ? (size_t)net3_act_len(g) : L;   // points of one activation image
   const int nw = net_batch_blocks(nb, g, B);
@@ -2747,8 +2768,10 @@ mpcg_status net_batch_alloc(bool net3, const GridDesc& g, int B, Alloc& mem, cud
   get(&nb.wtc, (size_t)(net3 ? net3_pack_bytes() : net_tc_weight_bytes()));
   get(&nb.terr, 1);
   get(&nb.parts_dev, 4);
-  if (st != MPCG_OK) return st;
-  if (net3) net3_prepare_attributes();
+}
+// after the plan's allocation
+mpcg_status net_batch_ready(const NetBatch& nb, cudaStream_t s) {
+  if (nb.net3) net3_prepare_attributes();
   else net_train_tc_prepare_attributes();
   CK(cudaMemcpyAsync(nb.parts_dev, nb.gr.part, sizeof(nb.gr.part), cudaMemcpyHostToDevice, s));
   return MPCG_OK;
@@ -2849,6 +2872,8 @@ mpcg_status mg_learned_detach(mg_hierarchy* h) {
   CK(cudaSetDevice(h->device));
   if (h->net_on) {
     h->net_on = false;
+    h->net_ws.release();
+    h->net_imgs = 0;
     CKS(rebuild_solvers(h));
   }
   return MPCG_OK;
@@ -2909,6 +2934,9 @@ mpcg_status mg_detach_q1_kappa(mg_hierarchy* h) {
   return MPCG_OK;
 }
 
+// workspace a hierarchy keeps for forward calls (a call of four 1025^2 images: 34 MB)
+static constexpr size_t kNetKeep = (size_t)256 << 20;
+
 mpcg_status mg_learned_forward_acts(mg_hierarchy* h, const float* rhat_dev, float* y_dev, float* acts_dev,
                                    int nimg) {
   g_err.clear();
@@ -2924,14 +2952,29 @@ mpcg_status mg_learned_forward_acts(mg_hierarchy* h, const float* rhat_dev, floa
   Alloc tmp;
   float *r = nullptr, *y = nullptr;
   mpcg_status st = MPCG_OK;
+  if (sizeof(float) * 2 * nimg * g.len > kNetKeep) {
+    st = tmp.get(&r, (size_t)nimg * g.len, s);
+    if (st == MPCG_OK) st = tmp.get(&y, (size_t)nimg * g.len, s);
+  } else {
+    // only the unknowns' entries are written: the zeroed pads hold for every call
+    if (nimg > h->net_imgs) {
+      h->net_ws.release();
+      h->net_imgs = 0;
+      st = h->net_ws.get(&h->net_r, (size_t)nimg * g.len, s);
+      if (st == MPCG_OK) st = h->net_ws.get(&h->net_y, (size_t)nimg * g.len, s);
+      if (st == MPCG_OK) h->net_imgs = nimg;
+      else h->net_ws.release();
+    }
+    r = h->net_r;
+    y = h->net_y;
+  }
   NetActs a3 = {};
   if (net3_of(h)) {   // activations for nimg images
     const size_t A = (size_t)net3_act_len(g) * nimg * 16;
     for (__nv_bfloat16** p : {&a3.a0, &a3.a1, &a3.a2, &a3.a3})
       if (st == MPCG_OK) st = tmp.get(p, A, s);
   }
-  if (st == MPCG_OK && (st = tmp.get(&r, (size_t)nimg * g.len, s)) == MPCG_OK &&
-      (st = tmp.get(&y, (size_t)nimg * g.len, s)) == MPCG_OK) {
+  if (st == MPCG_OK) {
     cudaMemsetAsync(h->net_err, 0, sizeof(int), s);
     launch_pack<float, float>(g, rhat_dev, g.n, r, nimg, s);
     if (net3_of(h)) {
@@ -2982,13 +3025,16 @@ mpcg_status mg_learned_grad(mg_hierarchy* h, const float* params, const float* r
   CKS(net_prepare(h));
   Alloc mem;
   NetBatch nbt;
-  mpcg_status st = net_batch_alloc(net3, g, nimg, mem, s, nbt);
   double *lsum = nullptr, *gd = nullptr;
   float *master = nullptr, *wq = nullptr;
-  if (st == MPCG_OK) st = mem.get(&lsum, 1, s);
-  if (st == MPCG_OK) st = mem.get(&gd, nbt.np, s);
-  if (st == MPCG_OK) st = mem.get(&master, nbt.np, s);
-  if (st == MPCG_OK) st = mem.get(&wq, nbt.np, s);
+  Alloc::Plan plan;
+  net_batch_plan(net3, g, nimg, plan, nbt);
+  plan.add(&lsum, 1);
+  plan.add(&gd, nbt.np);
+  plan.add(&master, nbt.np);
+  plan.add(&wq, nbt.np);
+  mpcg_status st = mem.commit(plan, s);
+  if (st == MPCG_OK) st = net_batch_ready(nbt, s);
   if (st != MPCG_OK) {
     mem.release();
     return st;
@@ -3070,21 +3116,21 @@ mpcg_status mg_learned_train(mg_hierarchy* const* hs, int nprob, const int* pair
   }
   Alloc mem;
   NetBatch nbt;
-  mpcg_status st = net_batch_alloc(net3, g, B, mem, s, nbt);
-  auto get = [&](auto** p, size_t n) {
-    if (st == MPCG_OK) st = mem.get(p, n, s);
-  };
   float *R, *E, *AE, *master, *m, *v, *wq;
   double* loss;
   const size_t L = g.len;
-  get(&R, (size_t)npairs * L);
-  get(&E, (size_t)npairs * L);
-  get(&AE, (size_t)npairs * L);
-  get(&master, nbt.np);
-  get(&m, nbt.np);
-  get(&v, nbt.np);
-  get(&wq, nbt.np);
-  get(&loss, 1);
+  Alloc::Plan plan;
+  net_batch_plan(net3, g, B, plan, nbt);
+  plan.add(&R, (size_t)npairs * L);
+  plan.add(&E, (size_t)npairs * L);
+  plan.add(&AE, (size_t)npairs * L);
+  plan.add(&master, nbt.np);
+  plan.add(&m, nbt.np);
+  plan.add(&v, nbt.np);
+  plan.add(&wq, nbt.np);
+  plan.add(&loss, 1);
+  mpcg_status st = mem.commit(plan, s);
+  if (st == MPCG_OK) st = net_batch_ready(nbt, s);
   if (st != MPCG_OK) {
     mem.release();
     return st;

@@ -1087,7 +1087,9 @@ def amg_roofline(trace, ns, nnzA, nnzP, C, m, w, peaks):
     for cls, ms in trace:
         tot[cls] = tot.get(cls, 0.0) + ms
     dom = max(tot, key=tot.get)
-    cnt, jj, jr, jp = 0, J, J, 1
+    names = [cls for cls, _ in trace]
+    jp0 = J + 1 - names.count("prolong") // max(1, names.count("update_xr"))
+    cnt, jj, jr, jp = 0, J, J, jp0
     bytes_sum = dur = 0.0
     launches = 0
     for cls, ms in trace:
@@ -1095,7 +1097,7 @@ def amg_roofline(trace, ns, nnzA, nnzP, C, m, w, peaks):
         if cls == "init":
             cnt = 0
         if cls in ("init", "check"):
-            jj, jr, jp = J, J, 1
+            jj, jr, jp = J, J, jp0
         if cls == "jacobi":
             b = nnzA[jj] * (4 + w) + 3 * ns[jj] * w
             jj -= 1
@@ -1114,7 +1116,7 @@ def amg_roofline(trace, ns, nnzA, nnzP, C, m, w, peaks):
                 bytes_sum += b
             dur += ms
             launches += 1
-        if cls == "small_alpha":
+        if cls == "update_xr":
             cnt = min(cnt + 1, m)
     share = tot[dom] / sum(tot.values())
     if bytes_sum == 0:

@@ -266,6 +266,7 @@ struct mg_hierarchy {
   cudaEvent_t ev_fork = nullptr, ev_fine = nullptr, ev_inv = nullptr;
   cudaEvent_t ev_r[kMaxLevels] = {}, ev_sm[kMaxLevels] = {};
   double* A0inv = nullptr;
+  double* A0lift = nullptr;   // algebraic: P_1 A_0^-1 P_1^T, where grid 1 has at most kLiftRows unknowns
   Level lev[kMaxLevels];
   double* L0 = nullptr;
   double* rdiag0 = nullptr;
@@ -641,6 +642,15 @@ void enqueue_mg(mg_hierarchy* h, Solver<T>& S, const T* r, T* Z, const DevState*
 // columns that have reached grid k-1 (the corrections of grids 0 .. k-1) in
 // one block SpMM, so every P_k is read once per iteration; grid j's buffer
 // zc[j] holds columns 0 .. j, column j being its own smoothed correction.
+// Where grid 1 is small enough, P_1 A_0^-1 R_1 is one dense operator on it
+// (kLiftRows): the iteration is a chain of launches of 5 to 6 us, and one launch
+// of 11 us stands for three of 8 (fracture network, 296,480 unknowns, grid 1 of
+// 556; launches one at a time: 201 -> 190 us an iteration).
+//
+// kLiftRows: 1024 rows are 8 MB of FP64 entries from L2, still about the time of
+// one of the launches saved; the next grids (3,677 rows: 108 MB) are far past it.
+constexpr int kLiftRows = 1024;
+
 template <typename T>
 void enqueue_mg_algebraic(mg_hierarchy* h, Solver<T>& S, const T* r, T* Z, const DevState* state, cudaStream_t s) {
   const int J = h->levels - 1;
@@ -654,7 +664,9 @@ void enqueue_mg_algebraic(mg_hierarchy* h, Solver<T>& S, const T* r, T* Z, const
   enqueue_smooth<T>(h, S, J, r, Z + (size_t)J * h->lev[J].g.cp, state, s2);
   cudaEventRecord(h->ev_fine, s2);
   const T* rj = r;
-  for (int j = J; j >= 1; --j) {
+  // the coarsest correction on the first grid whose operator form is at hand
+  const int jc = h->A0lift ? 1 : 0;
+  for (int j = J; j > jc; --j) {
     const GridDesc& gf = h->lev[j].g;
     const GridDesc& gc = h->lev[j - 1].g;
     LAUNCH(h, K_RESTRICT, s,
@@ -669,8 +681,9 @@ void enqueue_mg_algebraic(mg_hierarchy* h, Solver<T>& S, const T* r, T* Z, const
       cudaEventRecord(h->ev_sm[j - 1], s3);
     }
   }
-  LAUNCH(h, K_COARSE, s, launch_coarse_solve<T>(h->lev[0].g, h->A0inv, S.rlev[0], S.zc[0], state, s));
-  for (int k = 1; k <= J; ++k) {
+  LAUNCH(h, K_COARSE, s,
+         launch_coarse_solve<T>(h->lev[jc].g, jc ? h->A0lift : h->A0inv, rj, jc < J ? S.zc[jc] : Z, state, s));
+  for (int k = jc + 1; k <= J; ++k) {
     if (k - 1 >= 1) cudaStreamWaitEvent(s, h->ev_sm[k - 1], 0);
     const GridDesc& gc = h->lev[k - 1].g;
     const GridDesc& gk = h->lev[k].g;
@@ -1537,6 +1550,30 @@ mpcg_status mg_hierarchy_setup_algebraic(const mg_csr* A, const mg_amg_options* 
     if ((st = h->mem.get(&h->A0inv, nn, s)) != MPCG_OK) return fail(st);
     if ((st = h->mem.get(&X, nn, s)) != MPCG_OK) return fail(st);
     launch_coarse_inverse(h->L0, h->rdiag0, X, h->A0inv, n0, s);
+    if (levels > 1 && h->amgA[1].rows <= kLiftRows) {
+      const mpcg::amg::Csr& P = h->amgP[1];
+      Alloc tmp;
+      int *ptr = nullptr, *col = nullptr;
+      double *val = nullptr, *PX = nullptr;
+      const size_t n1 = P.rows, nnz = P.col.size();
+      st = h->mem.get(&h->A0lift, n1 * n1, s);
+      if (st == MPCG_OK) st = tmp.get(&ptr, n1 + 1, s);
+      if (st == MPCG_OK) st = tmp.get(&col, nnz, s);
+      if (st == MPCG_OK) st = tmp.get(&val, nnz, s);
+      if (st == MPCG_OK) st = tmp.get(&PX, n1 * n0, s);
+      if (st == MPCG_OK) {
+        cudaMemcpyAsync(ptr, P.ptr.data(), sizeof(int) * (n1 + 1), cudaMemcpyHostToDevice, s);
+        cudaMemcpyAsync(col, P.col.data(), sizeof(int) * nnz, cudaMemcpyHostToDevice, s);
+        cudaMemcpyAsync(val, P.val.data(), sizeof(double) * nnz, cudaMemcpyHostToDevice, s);
+        launch_coarse_lift((int)n1, n0, ptr, col, val, h->A0inv, PX, h->A0lift, s);
+        if (cudaStreamSynchronize(s) != cudaSuccess) {
+          set_err("setup kernels failed: %s", cudaGetErrorString(cudaGetLastError()));
+          st = MPCG_ERR_CUDA;
+        }
+      }
+      tmp.release();
+      if (st != MPCG_OK) return fail(st);
+    }
   }
   if ((st = build_solver<double>(h, h->s64)) != MPCG_OK) return fail(st);
   if (opt.precision == MPCG_MIXED) {

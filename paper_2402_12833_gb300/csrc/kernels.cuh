@@ -265,6 +265,10 @@ void launch_cholesky(double* a, double* rdiag, int n, int* info, cudaStream_t s)
 // inv = A0^{-1} from the Cholesky factor (X: n*n scratch)
 void launch_coarse_inverse(const double* L, const double* rdiag, double* X, double* inv, int n, cudaStream_t s);
 // out = A0^{-1} r; r, out in the padded layout of grid g
+// M = P A0^{-1} P^T (n1 x n1) of the P (CSR, n1 rows, n0 columns) from the coarsest
+// grid; X is n1 x n0 scratch
+void launch_coarse_lift(int n1, int n0, const int* ptr, const int* col, const double* val, const double* inv, double* X,
+                        double* M, cudaStream_t s);
 template <typename T>
 void launch_coarse_solve(const GridDesc& g, const double* inv, const T* r, T* out, const DevState* state,
                          cudaStream_t s);

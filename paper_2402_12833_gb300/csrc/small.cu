@@ -739,6 +739,26 @@ __global__ void __launch_bounds__(32 * kCoarseRowsPerBlock) k_coarse_solve(GridD
   if (lane == 0) out[padded_index(g, i)] = (T)s;
 }
 
+// X = P A0^{-1} (n1 x n0) and M = X P^T (n1 x n1), P in CSR form: a thread per entry.
+__global__ void k_coarse_lift(int n1, int n0, const int* __restrict__ ptr, const int* __restrict__ col,
+                              const double* __restrict__ val, const double* __restrict__ inv, double* __restrict__ X) {
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n1 * n0; e += gridDim.x * blockDim.x) {
+    const int i = e / n0, k = e % n0;
+    double s = 0.0;
+    for (int q = ptr[i]; q < ptr[i + 1]; ++q) s = fma(val[q], inv[(long long)col[q] * n0 + k], s);
+    X[e] = s;
+  }
+}
+__global__ void k_coarse_lift_both(int n1, int n0, const int* __restrict__ ptr, const int* __restrict__ col,
+                                   const double* __restrict__ val, const double* __restrict__ X, double* __restrict__ M) {
+  for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < n1 * n1; e += gridDim.x * blockDim.x) {
+    const int i = e / n1, j = e % n1;
+    double s = 0.0;
+    for (int q = ptr[j]; q < ptr[j + 1]; ++q) s = fma(val[q], X[(long long)i * n0 + col[q]], s);
+    M[e] = s;
+  }
+}
+
 // out[b * nv + v] = sum of problem b's partials of value v.
 __global__ void k_sum_partials(const double* part, int nv, int nblk, double* out) {
   const int pb = blockIdx.x;
@@ -864,6 +884,11 @@ template void launch_coarse_solve<double>(const GridDesc&, const double*, const 
 template void launch_coarse_solve<float>(const GridDesc&, const double*, const float*, float*, const DevState*,
                                          cudaStream_t);
 template void launch_coarse_solve<dw>(const GridDesc&, const double*, const dw*, dw*, const DevState*, cudaStream_t);
+void launch_coarse_lift(int n1, int n0, const int* ptr, const int* col, const double* val, const double* inv, double* X,
+                        double* M, cudaStream_t s) {
+  k_coarse_lift<<<grid_for((long long)n1 * n0, 1024), kBlock, 0, s>>>(n1, n0, ptr, col, val, inv, X);
+  k_coarse_lift_both<<<grid_for((long long)n1 * n1, 4096), kBlock, 0, s>>>(n1, n0, ptr, col, val, X, M);
+}
 void launch_mix_init(int* mix, int* active, int nb, int* outer, cudaStream_t s) {
   k_mix_init<<<1, kBlock, 0, s>>>(mix, active, nb, outer);
 }

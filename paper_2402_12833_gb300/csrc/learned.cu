@@ -44,7 +44,7 @@ __global__ void __launch_bounds__(kBlock) k_net_dots(GridDesc g, const float* __
 }
 
 // Loss per item and coefficients of dL/dy = -k1 (Ae - k2 Ay) / B: a warp per
-// item, lanes over the partials (one thread per item: 17 us at 8 items of 64 partials; now 9).
+// item, lanes over the partials (one thread per item: 17 us at 8 items of 64 partials; now 11).
 __global__ void k_net_loss(const double* part, int nblk, int B, double* coef, double* loss_sum) {
   const int b = threadIdx.x >> 5, lane = threadIdx.x & 31;
   double d[3];
@@ -56,13 +56,20 @@ __global__ void k_net_loss(const double* part, int nblk, int B, double* coef, do
     for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
     d[v] = a;
   }
-  if (lane != 0) return;
-  const double eAy = d[0], eAe = d[1], yAy = d[2];
-  const bool ok = eAe > 0.0 && yAy > 0.0;
-  const double L = ok ? 1.0 - eAy * eAy / (eAe * yAy) : 1.0;
-  coef[2 * b + 0] = ok ? 2.0 * eAy / (eAe * yAy) / B : 0.0;
-  coef[2 * b + 1] = ok ? eAy / yAy : 0.0;
-  atomicAdd(loss_sum, L / B);   // B <= 12 values; the order does not feed back into training
+  __shared__ double Ls[MPCG_MAX_COLS];
+  if (lane == 0) {
+    const double eAy = d[0], eAe = d[1], yAy = d[2];
+    const bool ok = eAe > 0.0 && yAy > 0.0;
+    Ls[b] = ok ? 1.0 - eAy * eAy / (eAe * yAy) : 1.0;
+    coef[2 * b + 0] = ok ? 2.0 * eAy / (eAe * yAy) / B : 0.0;
+    coef[2 * b + 1] = ok ? eAy / yAy : 0.0;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double L = *loss_sum;
+    for (int k = 0; k < B; ++k) L += Ls[k] / B;
+    *loss_sum = L;
+  }
 }
 
 __global__ void k_net_dy(GridDesc g, int B, const float* __restrict__ Ay, const float* __restrict__ Ae,

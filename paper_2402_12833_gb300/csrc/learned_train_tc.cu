@@ -99,65 +99,69 @@ __global__ void __launch_bounds__(kWT, 2)
       tc::fence_after();
     }
     const long long t0 = (c0 + i) * kChunk;
-    // A: one core-matrix column (8 points) of one 8-channel group per item;
-    // hi rows cg*8 + c, lo rows 16 + cg*8 + c
-    constexpr int CG = (COUT + 7) / 8;
-    for (int item = tid; item < CG * 8; item += kWT) {
-      const int cg = item / 8, pg = item % 8;
-#pragma unroll 1
-      for (int c = 0; c < 8; ++c) {
-        const int co = cg * 8 + c;
-        float hi[8], lo[8];
+    // A: 8 points of one channel per item, a thread each (channels over
+    // neighbouring lanes: the point-major rows are read whole); hi row co, lo
+    // row 16 + co.  With an item per 8 channels 16 threads walked 64 loads each,
+    // and 144 items of B took two rounds: 52 -> 32 us a layer (129^2, batch of 8).
+    constexpr int CR = (COUT + 7) / 8 * 8;
+    static_assert(CR * 8 <= kWT, "an item per thread");
+    if (tid < CR * 8) {
+      const int co = tid % CR, pg = tid / CR;
+      float hi[8], lo[8];
 #pragma unroll
-        for (int kk = 0; kk < 8; ++kk) {
-          const long long t = t0 + pg * 8 + kk;
-          const float d = (t < g.npts && co < COUT) ? dOut[(base + t) * COUT + co] : 0.f;
-          tc::split_bf16(d, hi[kk], lo[kk]);
-        }
-        const uint4 vh = make_uint4(tc::pack_bf16x2(hi[0], hi[1]), tc::pack_bf16x2(hi[2], hi[3]),
-                                    tc::pack_bf16x2(hi[4], hi[5]), tc::pack_bf16x2(hi[6], hi[7]));
-        const uint4 vl = make_uint4(tc::pack_bf16x2(lo[0], lo[1]), tc::pack_bf16x2(lo[2], lo[3]),
-                                    tc::pack_bf16x2(lo[4], lo[5]), tc::pack_bf16x2(lo[6], lo[7]));
-        *reinterpret_cast<uint4*>(A + toff(co, pg * 8)) = vh;
-        *reinterpret_cast<uint4*>(A + toff(16 + co, pg * 8)) = vl;
+      for (int kk = 0; kk < 8; ++kk) {
+        const long long t = t0 + pg * 8 + kk;
+        const float d = (t < g.npts && co < COUT) ? dOut[(base + t) * COUT + co] : 0.f;
+        tc::split_bf16(d, hi[kk], lo[kk]);
       }
+      const uint4 vh = make_uint4(tc::pack_bf16x2(hi[0], hi[1]), tc::pack_bf16x2(hi[2], hi[3]),
+                                  tc::pack_bf16x2(hi[4], hi[5]), tc::pack_bf16x2(hi[6], hi[7]));
+      const uint4 vl = make_uint4(tc::pack_bf16x2(lo[0], lo[1]), tc::pack_bf16x2(lo[2], lo[3]),
+                                  tc::pack_bf16x2(lo[4], lo[5]), tc::pack_bf16x2(lo[6], lo[7]));
+      *reinterpret_cast<uint4*>(A + toff(co, pg * 8)) = vh;
+      *reinterpret_cast<uint4*>(A + toff(16 + co, pg * 8)) = vl;
     }
-    // B: rows (tap, ci), the layer input at the tap's offset, 8 points per core matrix
-    for (int item = tid; item < 9 * 2 * 8; item += kWT) {
-      const int tap = item / 16, half = (item / 8) % 2, pg = item % 8;
+    // B: rows (tap, ci), the layer input at the tap's offset, 8 points of four
+    // channels per item, the loads of all rounds in flight together
+    constexpr int kItems = 9 * 4 * 8, kRounds = (kItems + kWT - 1) / kWT;
+    uint32_t w[kRounds][8][2];   // [round][point][channel pair]
+#pragma unroll
+    for (int rd = 0; rd < kRounds; ++rd) {
+      const int item = rd * kWT + tid;
+      const int tap = item / 32, quad = item % 4, pg = item / 4 % 8;
       const long long off = (tap % 3 - 1) + (long long)(tap / 3 - 1) * p;
-      uint32_t w[8][4];   // [point][channel pair]
 #pragma unroll
       for (int kk = 0; kk < 8; ++kk) {
         const long long t = t0 + pg * 8 + kk;
         const long long q = base + t + off;
-        if (t >= g.npts) {   // beyond the box: dOut is zero there; stay inside the guards
+        w[rd][kk][0] = w[rd][kk][1] = 0u;
+        if (item >= kItems || t >= g.npts) continue;   // beyond the box: dOut is zero there; stay inside the guards
+        if (CIN == 16) {
+          const uint2 v = *reinterpret_cast<const uint2*>(act + q * 16 + quad * 4);
+          w[rd][kk][0] = v.x; w[rd][kk][1] = v.y;
+        } else if (quad == 0) {
 #pragma unroll
-          for (int j = 0; j < 4; ++j) w[kk][j] = 0u;
-        } else if (CIN == 16) {
-          const uint4 v = *reinterpret_cast<const uint4*>(act + q * 16 + half * 8);
-          w[kk][0] = v.x; w[kk][1] = v.y; w[kk][2] = v.z; w[kk][3] = v.w;
-        } else {
-#pragma unroll
-          for (int j = 0; j < 4; ++j) w[kk][j] = 0u;
-          if (half == 0) {
-#pragma unroll
-            for (int c = 0; c < CIN; c += 2) {
-              const __nv_bfloat16 a0 = act[q * CIN + c];
-              const __nv_bfloat16 a1 = c + 1 < CIN ? act[q * CIN + c + 1] : __float2bfloat16_rn(0.f);
-              w[kk][c / 2] = (uint32_t)__bfloat16_as_ushort(a0) | ((uint32_t)__bfloat16_as_ushort(a1) << 16);
-            }
+          for (int c = 0; c < CIN; c += 2) {
+            const __nv_bfloat16 a0 = act[q * CIN + c];
+            const __nv_bfloat16 a1 = c + 1 < CIN ? act[q * CIN + c + 1] : __float2bfloat16_rn(0.f);
+            w[rd][kk][c / 2] = (uint32_t)__bfloat16_as_ushort(a0) | ((uint32_t)__bfloat16_as_ushort(a1) << 16);
           }
         }
       }
+    }
+#pragma unroll
+    for (int rd = 0; rd < kRounds; ++rd) {
+      const int item = rd * kWT + tid;
+      const int tap = item / 32, quad = item % 4, pg = item / 4 % 8;
+      if (item >= kItems) continue;
       // transpose: row ci of the core matrix holds the 8 points of channel ci
 #pragma unroll
-      for (int ci = 0; ci < 8; ++ci) {
-        const unsigned sel = (ci & 1) ? 0x7632u : 0x5410u;
-        const int wi = ci >> 1;
-        const uint4 r = make_uint4(__byte_perm(w[0][wi], w[1][wi], sel), __byte_perm(w[2][wi], w[3][wi], sel),
-                                   __byte_perm(w[4][wi], w[5][wi], sel), __byte_perm(w[6][wi], w[7][wi], sel));
-        *reinterpret_cast<uint4*>(Bt + toff(tap * 16 + half * 8 + ci, pg * 8)) = r;
+      for (int c = 0; c < 4; ++c) {
+        const unsigned sel = (c & 1) ? 0x7632u : 0x5410u;
+        const int wi = c >> 1;
+        const uint4 r = make_uint4(__byte_perm(w[rd][0][wi], w[rd][1][wi], sel), __byte_perm(w[rd][2][wi], w[rd][3][wi], sel),
+                                   __byte_perm(w[rd][4][wi], w[rd][5][wi], sel), __byte_perm(w[rd][6][wi], w[rd][7][wi], sel));
+        *reinterpret_cast<uint4*>(Bt + toff(tap * 16 + quad * 4 + c, pg * 8)) = r;
       }
     }
     tc::fence_async_smem();
@@ -253,23 +257,42 @@ __global__ void __launch_bounds__(kWT, 2)
   if (tid < kDR + 2) tc::mbar_init(tc::smem_u32(bar + tid));
   if (tid == 0) tc::mbar_init_fence();
   // weight tiles: tap t = ky * 3 + kx at tile kx * 3 + ky, row n = ci, column k = co
-  for (int e = tid; e < 9 * 256; e += kWT) {
+  static_assert(9 * 256 % kWT == 0, "whole rounds");
+#pragma unroll
+  for (int e0 = 0; e0 < 9 * 256; e0 += kWT) {   // the rounds' loads in flight together
+    const int e = e0 + tid;
     const int t = e / 256, ci = (e / 16) % 16, co = e % 16;
     const float w = co < COUT ? W[(co * 16 + ci) * 9 + t] : 0.f;
     *reinterpret_cast<__nv_bfloat16*>(smem + kDWOff + ((t % 3) * 3 + t / 3) * 512 + canon16(ci, co)) =
         __float2bfloat16_rn(w);
   }
-  // dOut rows y0 - 1 .. y0 + kDR, x0 - 1 .. x0 + 128 (zero outside the grid)
+  // dOut rows y0 - 1 .. y0 + kDR, x0 - 1 .. x0 + 128 (zero outside the grid); a
+  // point's 16 channels are one 64-byte line segment, read in 16-byte loads, two
+  // points in flight (scalar loads: 24 us a layer at 129^2, batch of 8; now 19)
+#pragma unroll 2
   for (int e = tid; e < (kDR + 2) * kDXS; e += kWT) {
     const int sr = e / kDXS, xs = e % kDXS;
     const int y = y0 - 1 + sr, x = x0 - 1 + xs;
     const bool in = x >= 0 && x < n1 && y >= 0 && y < n1;
     float hi[16], lo[16];
+    float d[16];
 #pragma unroll
-    for (int c = 0; c < 16; ++c) {
-      const float d = (in && c < COUT) ? dOut[(base + (long long)y * p + x) * COUT + c] : 0.f;
-      tc::split_bf16(d, hi[c], lo[c]);
+    for (int c = 0; c < 16; ++c) d[c] = 0.f;
+    if (in) {
+      const float* src = dOut + (base + (long long)y * p + x) * COUT;
+      if constexpr (COUT == 16) {
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const float4 v = reinterpret_cast<const float4*>(src)[q];
+          d[4 * q] = v.x; d[4 * q + 1] = v.y; d[4 * q + 2] = v.z; d[4 * q + 3] = v.w;
+        }
+      } else {
+#pragma unroll
+        for (int c = 0; c < COUT; ++c) d[c] = src[c];
+      }
     }
+#pragma unroll
+    for (int c = 0; c < 16; ++c) tc::split_bf16(d[c], hi[c], lo[c]);
     const int off = (sr * kDXS + xs) * 16;
 #pragma unroll
     for (int pl = 0; pl < 4; ++pl) {

@@ -1,4 +1,4 @@
-// Structured-grid kernels: layout conversion, block stencil SpMM (the A Z
+// Structured-grid kernels: layout conversion, block stencil SpMM (the A P
 // product of Section 2.2), residual, restriction R = P^T and prolongation P
 // (Section 2.1), damped-Jacobi smoothing (Eq. 2), and the Galerkin product
 // P^T A P that builds the coarse operators.

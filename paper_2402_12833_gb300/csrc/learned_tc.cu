@@ -57,7 +57,8 @@ constexpr int kXS = kEW + 2;           // stored row length: x = -1 and x = 128 
 constexpr int kNPix = kEH * kXS;       // pixels of one activation buffer
 constexpr int kPlane = kNPix * 16;     // bytes of one channel plane
 constexpr int kThreads = 256;          // eight warps: TMEM lanes 0..127, twice (channel halves)
-constexpr int kMaxRows = kEH - 2;      // rows computed by the first layer
+constexpr int kMaxRows = kEH - 2;      // rows computed by the first layer; two fewer by each later one
+static_assert(kMaxRows % 2 == 0, "rows are read back in pairs");
 constexpr int kMaxSlots = kEH;         // input rows (slots) of the first layer: one mbarrier each
 constexpr int kTmemCols = 256;         // one 16-column accumulator per output row of a layer (224 used)
 constexpr long long kWaitLimit = 1LL << 22;
@@ -142,29 +143,23 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// 8 consecutive FP32 columns of this thread's TMEM lane
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, float (&v)[8]) {
-  uint32_t r[8];
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int i = 0; i < 8; ++i) v[i] = __uint_as_float(r[i]);
-}
-
-// 16 consecutive FP32 columns of this thread's TMEM lane
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
+// 8 consecutive FP32 columns at each of two places of this thread's TMEM lane,
+// one wait for both
+__device__ __forceinline__ void tmem_ld8x2(uint32_t ta, uint32_t tb, float (&v)[2][8]) {
   uint32_t r[16];
   asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, "
-      "%15}, [%16];"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%16];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8, %9, %10, %11, %12, %13, %14, %15}, [%17];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
         "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+      : "r"(ta), "r"(tb)
+      : "memory");
 #pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
+  for (int i = 0; i < 8; ++i) {
+    v[0][i] = __uint_as_float(r[i]);
+    v[1][i] = __uint_as_float(r[8 + i]);
+  }
 }
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float a, float b) {
@@ -311,10 +306,13 @@ __global__ void __launch_bounds__(kThreads, 2)
         mma_commit(bar0 + 8 * sl);
       }
     }
-    for (int i = 0; i < nrows; ++i) {
-      // output i is complete once the MMAs of slot i + 2 are (commits
-      // complete in issue order), and by then so are those reading slot i
-      const int sb = i + 2;
+    // two rows a step (nrows is even): the wait for the commit and the read of
+    // tensor memory are latency, 44 times a tile with a row a step (four images of
+    // 1025^2: 323 us; now 302)
+    for (int i = 0; i < nrows; i += 2) {
+      // outputs i and i + 1 are complete once the MMAs of slot i + 3 are (commits
+      // complete in issue order), and by then so are those reading slots i, i + 1
+      const int sb = i + 3;
       const bool ok = mbar_wait(bar0 + 8 * sb, (phase >> sb) & 1u, c_wait_first);
       if (!ok) {
         failed = true;
@@ -322,36 +320,41 @@ __global__ void __launch_bounds__(kThreads, 2)
       }
       fence_after();
       // warps w and w + 4 read the same 32 lanes: channels 8 h .. 8 h + 7
-      float v[8];
-      tmem_ld8(tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(col_of(i) + 8 * h), v);
-      const int row = r0 + i, gy = gy0 + row;
-      const bool inside = gx >= 0 && gx < n1 && gy >= 0 && gy < n1;
-      if (L < 3) {
-        uint32_t q[4];
+      float v2[2][8];
+      const uint32_t lane0 = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)(8 * h);
+      tmem_ld8x2(lane0 + (uint32_t)col_of(i), lane0 + (uint32_t)col_of(i + 1), v2);
 #pragma unroll
-        for (int k = 0; k < 4; ++k)
-          q[k] = inside ? pack_bf16x2(fmaxf(v[2 * k], 0.f), fmaxf(v[2 * k + 1], 0.f)) : 0u;
-        const int off = ((row - L - 1) * kXS + x + 1) * 16;   // in place: slot of input row row - 1
-        *reinterpret_cast<uint4*>(act + h * kPlane + off) = make_uint4(q[0], q[1], q[2], q[3]);
-        __nv_bfloat16* kept = L == 0 ? keep.a1 : (L == 1 ? keep.a2 : keep.a3);
-        if (kept && inside && x >= kHalo && x < kHalo + kTW && row >= kHalo && row < kHalo + kTH) {
-          uint4* o = reinterpret_cast<uint4*>(kept + ((long long)b * g.len + g.G + gx + p * gy) * 16);
-          o[h] = make_uint4(q[0], q[1], q[2], q[3]);
-        }
-        if (acts && inside && x >= kHalo && x < kHalo + kTW && row >= kHalo && row < kHalo + kTH) {
-          const long long nn = (long long)n1 * n1;
-          float* o = acts + ((((long long)(L + 1) * gridDim.z + b) * nn) + (long long)gy * n1 + gx) * 16 + 8 * h;
+      for (int d = 0; d < 2; ++d) {
+        const float(&v)[8] = v2[d];
+        const int row = r0 + i + d, gy = gy0 + row;
+        const bool inside = gx >= 0 && gx < n1 && gy >= 0 && gy < n1;
+        if (L < 3) {
+          uint32_t q[4];
 #pragma unroll
-          for (int k = 0; k < 4; ++k) {
-            const __nv_bfloat162 h2 = *reinterpret_cast<const __nv_bfloat162*>(&q[k]);
-            o[2 * k] = __low2float(h2);
-            o[2 * k + 1] = __high2float(h2);
+          for (int k = 0; k < 4; ++k)
+            q[k] = inside ? pack_bf16x2(fmaxf(v[2 * k], 0.f), fmaxf(v[2 * k + 1], 0.f)) : 0u;
+          const int off = ((row - L - 1) * kXS + x + 1) * 16;   // in place: slot of input row row - 1
+          *reinterpret_cast<uint4*>(act + h * kPlane + off) = make_uint4(q[0], q[1], q[2], q[3]);
+          __nv_bfloat16* kept = L == 0 ? keep.a1 : (L == 1 ? keep.a2 : keep.a3);
+          if (kept && inside && x >= kHalo && x < kHalo + kTW && row >= kHalo && row < kHalo + kTH) {
+            uint4* o = reinterpret_cast<uint4*>(kept + ((long long)b * g.len + g.G + gx + p * gy) * 16);
+            o[h] = make_uint4(q[0], q[1], q[2], q[3]);
           }
+          if (acts && inside && x >= kHalo && x < kHalo + kTW && row >= kHalo && row < kHalo + kTH) {
+            const long long nn = (long long)n1 * n1;
+            float* o = acts + ((((long long)(L + 1) * gridDim.z + b) * nn) + (long long)gy * n1 + gx) * 16 + 8 * h;
+#pragma unroll
+            for (int k = 0; k < 4; ++k) {
+              const __nv_bfloat162 h2 = *reinterpret_cast<const __nv_bfloat162*>(&q[k]);
+              o[2 * k] = __low2float(h2);
+              o[2 * k + 1] = __high2float(h2);
+            }
+          }
+        } else if (h == 0 && inside && x >= kHalo && x < kHalo + kTW && row >= kHalo && row < kHalo + kTH) {
+          const long long o = (long long)b * g.len + g.G + gx + p * gy;
+          if (y) y[o] = v[0];
+          if (z) z[o] = (T)(zscale * (double)v[0]);
         }
-      } else if (h == 0 && inside && x >= kHalo && x < kHalo + kTW && row >= kHalo && row < kHalo + kTH) {
-        const long long o = (long long)b * g.len + g.G + gx + p * gy;
-        if (y) y[o] = v[0];
-        if (z) z[o] = (T)(zscale * (double)v[0]);
       }
     }
     // the layer's outputs feed the next layer's MMAs (async proxy)

@@ -193,7 +193,7 @@ def roofline(trace, ns, C, m, w, peaks, fp64_alu_peak_tflops, S=27, vector=False
                 flops_sum += f
             dur += ms
             launches += 1
-        if cls == "small_alpha":
+        if cls == "update_xr":
             cnt = min(cnt + 1, m)
     share = tot[dom] / sum(tot.values())
     if bytes_sum == 0:

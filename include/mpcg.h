@@ -358,7 +358,7 @@ long long mg_level_size(const mg_hierarchy* h, int level);
 
 /*
  * Y = A_level X for `ncols` columns (block SpMM of the Section 2.2 update
- * A Z); X_dev, Y_dev are column-major n_level x ncols device arrays.
+ * A P); X_dev, Y_dev are column-major n_level x ncols device arrays.
  */
 mpcg_status mg_apply_operator(mg_hierarchy* h, int level, const double* X_dev,
                               double* Y_dev, int ncols);
@@ -491,7 +491,9 @@ int mg_learned_num_params_of(const mg_hierarchy* h);
 mpcg_status mg_learned_attach(mg_hierarchy* h, const float* params, int nparams);
 mpcg_status mg_learned_detach(mg_hierarchy* h);
 /* y = N(rhat, c) for nimg images on h's fine grid (device, n floats each,
- * rhat already scaled); needs attached weights. */
+ * rhat already scaled); needs attached weights.  The hierarchy keeps the call's
+ * workspace (2 * nimg padded fine-grid arrays of floats) for the next one where it
+ * takes at most 256 MB, until mg_learned_detach or mg_hierarchy_destroy. */
 mpcg_status mg_learned_forward(mg_hierarchy* h, const float* rhat_dev, float* y_dev, int nimg);
 /* mg_learned_forward that also copies the activations out for inspection
  * (the tensor-core inference kernel): acts_dev (device, may be NULL) gets
@@ -589,7 +591,8 @@ mpcg_status mg_stencil_apply_noalloc(int dim, int nodes, const double* values_de
  *   MG_TUNE_STREAM_BLOCKS  blocks of the streaming block kernels (A-
  *                          orthogonalisation, update, residual) on a grid;
  *   MG_TUNE_SPMM_BLOCKS    blocks of the block SpMM on the full stored stencil;
- *   MG_TUNE_GRAM_CHUNKS    point chunks per window block of the window Gram;
+ *   MG_TUNE_GRAM_CHUNKS    point chunks the warps of a row task of the window Gram
+ *                          share out;
  *   MG_TUNE_JACOBI_NARROW  1: one point per thread in the Jacobi sweep of a
  *                          grid, 0: a 16-byte vector per thread.
  * Every tuned value is clamped at launch to the range the solver's buffers

@@ -43,33 +43,34 @@ __global__ void __launch_bounds__(kBlock) k_net_dots(GridDesc g, const float* __
   block_sum_store<float, 3>(s, part + (long long)b * 3 * gridDim.x, gridDim.x, blockIdx.x);
 }
 
-// Loss per item and coefficients of dL/dy = -k1 (Ae - k2 Ay) / B: a warp per
-// item, lanes over the partials (one thread per item: 17 us at 8 items of 64 partials; now 11).
+// Loss per item and coefficients of dL/dy = -k1 (Ae - k2 Ay) / B.  A warp sums
+// an item's partials; then a lane per item divides, so that the slow FP64
+// divisions of all items are one warp's instructions (one thread per item from
+// the start: 17 us at 8 items of 64 partials, a warp per item to the end 11, now 9).
 __global__ void k_net_loss(const double* part, int nblk, int B, double* coef, double* loss_sum) {
   const int b = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  double d[3];
+  __shared__ double dots[3][MPCG_MAX_COLS];
 #pragma unroll
   for (int v = 0; v < 3; ++v) {
     double a = 0.0;
     for (int k = lane; k < nblk; k += 32) a += part[((long long)b * 3 + v) * nblk + k];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) a += __shfl_xor_sync(0xffffffffu, a, o);
-    d[v] = a;
-  }
-  __shared__ double Ls[MPCG_MAX_COLS];
-  if (lane == 0) {
-    const double eAy = d[0], eAe = d[1], yAy = d[2];
-    const bool ok = eAe > 0.0 && yAy > 0.0;
-    Ls[b] = ok ? 1.0 - eAy * eAy / (eAe * yAy) : 1.0;
-    coef[2 * b + 0] = ok ? 2.0 * eAy / (eAe * yAy) / B : 0.0;
-    coef[2 * b + 1] = ok ? eAy / yAy : 0.0;
+    if (lane == 0) dots[v][b] = a;
   }
   __syncthreads();
-  if (threadIdx.x == 0) {
-    double L = *loss_sum;
-    for (int k = 0; k < B; ++k) L += Ls[k] / B;
-    *loss_sum = L;
+  if (b != 0) return;
+  double L = 0.0;
+  if (lane < B) {
+    const double eAy = dots[0][lane], eAe = dots[1][lane], yAy = dots[2][lane];
+    const bool ok = eAe > 0.0 && yAy > 0.0;
+    L = (ok ? 1.0 - eAy * eAy / (eAe * yAy) : 1.0) / B;
+    coef[2 * lane + 0] = ok ? 2.0 * eAy / (eAe * yAy) / B : 0.0;
+    coef[2 * lane + 1] = ok ? eAy / yAy : 0.0;
   }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) L += __shfl_xor_sync(0xffffffffu, L, o);
+  if (lane == 0) *loss_sum += L;
 }
 
 __global__ void k_net_dy(GridDesc g, int B, const float* __restrict__ Ay, const float* __restrict__ Ae,

@@ -400,6 +400,11 @@ __global__ void __launch_bounds__(kBlock) k_restrict_multi(RestrictArgs<T, K> a,
   restrict_step<T, K, TC, 1>(a, buf, tx, ty, tx == ntx - 1, ty == nty - 1, pb);
 }
 
+// s1 + dinv (r - A s1), s1 = dinv r, the roundings fixed for the kernels that share it
+__device__ __forceinline__ float half_sweep(float di, float ri, float as1) {
+  return fmaf(di, __fsub_rn(ri, as1), __fmul_rn(di, ri));
+}
+
 // Damped Jacobi (Eq. 2 with M = D / omega, dinv = omega / diag), c_0 = 0:
 //   mode 0: out = dinv r                          (one sweep)
 //   mode 1: out = s1 + dinv (r - A s1), s1 = dinv r  (two sweeps, s1 formed
@@ -408,7 +413,9 @@ __global__ void __launch_bounds__(kBlock) k_restrict_multi(RestrictArgs<T, K> a,
 //   W points per thread: Vec<T>::W (one vector load), or 1 on the small
 //   grids (modes 0 and 1; mode 2 keeps Vec<T>::W).  Every point's
 //   arithmetic is the same whatever W.  SYM: st is the symmetric half
-//   (row_coeffs).
+//   (row_coeffs); its two-sweep mode runs here for W = 1 only and adds a point's
+//   products as k_jacobi_half does, those over the ends of an aligned group of
+//   four apart: the width may depend on the batch, a problem's bits may not.
 template <typename T, int DIM, int W = Vec<T>::W, bool SYM = false>
 __global__ void __launch_bounds__(kBlock, 4) k_jacobi(GridDesc g, const T* __restrict__ st, const T* __restrict__ dinv,
                                                    const T* __restrict__ r, const T* __restrict__ sin,
@@ -440,6 +447,27 @@ __global__ void __launch_bounds__(kBlock, 4) k_jacobi(GridDesc g, const T* __res
   if (mode == 1) {
     const unsigned act = __ballot_sync(0xffffffffu, active);
     constexpr int R = DIM == 3 ? 9 : 3;
+    if constexpr (SYM && W == 1) {
+      const int pos = (int)(q & 3);   // in its group; 1 and 2 have no product over an end
+      T over = 0, in = 0;
+#pragma unroll
+      for (int k = 0; k < R; ++k) {
+        const long long ro = row_offset<DIM>(k, g.px, g.pxy);
+        T a0[1] = {}, a1[1] = {}, a2[1] = {}, ed[3], er[3];
+        if (active) row_coeffs<T, DIM, 1, SYM>(st, g.cp, idx, ro, k, a0, a1, a2);
+        load_row_shfl<T, 1>(dinv + idx + ro, ed, active, act, lane);
+        load_row_shfl<T, 1>(r + idx + ro, er, active, act, lane);
+        const T xl = ed[0] * er[0], xc = ed[1] * er[1], xr = ed[2] * er[2];
+        if (pos == 0) over = fma(a0[0], xl, over);
+        else in = fma(a0[0], xl, in);
+        in = fma(a1[0], xc, in);
+        if (pos == 3) over = fma(a2[0], xr, over);
+        else in = fma(a2[0], xr, in);
+      }
+      o[0] = half_sweep(di[0], ri[0], pos == 0 || pos == 3 ? in + over : in);
+      if (active) out[idx] = o[0];
+      return;
+    }
 #pragma unroll
     for (int k = 0; k < R; ++k) {
       const long long ro = row_offset<DIM>(k, g.px, g.pxy);
@@ -599,7 +627,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_jacobi_half(GridDesc g, RowMap ma
   if (!store) return;
   float o[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) o[i] = di[i] * ri[i] + di[i] * (ri[i] - acc[i + 1]);
+  for (int i = 0; i < 4; ++i) o[i] = half_sweep(di[i], ri[i], acc[i + 1]);
   Vec<float>::store(out + idx, o);
 }
 

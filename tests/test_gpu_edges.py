@@ -132,6 +132,23 @@ def test_solve_with_the_widest_block(M):
     assert status == M.MPCG_OK and (b - y).norm() <= 1.01e-8 * b.norm()
 
 
+@pytest.mark.parametrize("dim,nodes,count", [(2, 65, 24), (2, 129, 8), (3, 33, 5)])
+def test_mixed_batch_equals_single_solves_bitwise(M, dim, nodes, count):
+    """Grids whose smoothing takes another width in a batch than alone."""
+    probs = [pb.diffusion_macro(dim, nodes, 300 + i, rhs="normal", rhs_seed=400 + i) for i in range(count)]
+    dev = [torch.from_numpy(np.ascontiguousarray(p.stencil)).cuda() for p in probs]
+    B = M.BatchedHierarchy(dev, dim, nodes, probs[0].levels, precision=M.MPCG_MIXED)
+    b = torch.from_numpy(np.stack([p.b for p in probs])).cuda()
+    x = torch.zeros_like(b)
+    status, its = B.solve(b, x, rtol=1e-8, maxit=2000)
+    assert status == M.MPCG_OK
+    for i in range(count):
+        H = M.Hierarchy(dev[i], dim, nodes, probs[0].levels, precision=M.MPCG_MIXED)
+        xs = torch.zeros_like(b[i])
+        status, k, _, _ = H.solve(b[i].contiguous(), xs, rtol=1e-8, maxit=2000)
+        assert status == M.MPCG_OK and its[i] == k and torch.equal(x[i], xs), i
+
+
 @pytest.mark.parametrize("nodes,faces", [(21, 0x3F), (21, 0x2A), (37, 0x15), (45, 0x3F)])
 def test_matrix_free_rows(M, nodes, faces):
     """Ragged rows through the operator rebuilt from kappa, with its Gram sums."""

@@ -418,7 +418,9 @@ mpcg_status build_solver(mg_hierarchy* h, Solver<T>& S) {
   CKS(S.mem.get(&S.part_res, nb * 2 * sbc, s));
   CKS(S.mem.get(&S.part_W, nb * S.m * C * C * gcc, s));
   // at least the row kernels' slots: two blocks per SM of 256 threads, or as many smaller ones
-  const size_t gsl = std::max(sbc, (size_t)16 * (size_t)std::max(sm_count(), 152));
+  size_t gsl = std::max(sbc, (size_t)16 * (size_t)std::max(sm_count(), 152));
+  if (h->algebraic)
+    gsl = std::max(gsl, (size_t)ell_gram_blocks(ell_of<T>(h->lev[J].eA).nslices, std::max(sm_count(), 152)));
   CKS(S.mem.get(&S.part_G, nb * (C * (C + 1) / 2 + C) * gsl, s));
   CKS(S.mem.get(&S.part_r, nb * sbc, s));
   CKS(S.mem.get(&S.small_scratch, nb * kSmallScratch, s));

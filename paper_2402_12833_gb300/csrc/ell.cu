@@ -188,9 +188,7 @@ template void launch_ell_spmm<dw>(const EllDev<dw>&, const SpmmIO<dw>&, long lon
 
 int launch_ell_spmm_gram(const EllDev<float>& A, const SpmmIO<float>& io, long long ld, int C, const float* r,
                          double* part, const DevState* state, cudaStream_t s) {
-  // at most eight blocks per SM: the slots the solver reserves
-  const int cap = 8 * (sm_count() > 0 ? sm_count() : 152), need = ell_threads_blocks(A);
-  const int grid = need < cap ? need : cap;
+  const int grid = ell_gram_blocks(A.nslices, sm_count() > 0 ? sm_count() : 152);
 #define MPCG_ELL_CASE(CC)                                                                                \
   case CC:                                                                                               \
     k_ell_spmm<float, CC, false, true><<<grid, kBlock, 0, s>>>(A, io, ld, ld, r, part, state);           \

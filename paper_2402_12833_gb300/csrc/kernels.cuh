@@ -69,6 +69,18 @@ inline int grid_for(long long work, int cap) {
 template <typename T>
 void launch_ell_spmm(const EllDev<T>& A, const SpmmIO<T>& io, long long ldx, long long ldy, int C,
                      const DevState* state, cudaStream_t s);
+// Blocks of the FP32 product that also forms P^T A P and P^T r: eight per SM, or
+// more where a lane would then meet over 64 slices, that is sum over 64 rows in
+// FP32 (the accuracy limit above; at eight blocks per SM it is passed from 19.9 M
+// rows on with a lane per row, 5 M with four).  The solver reserves as many slots.
+inline int ell_gram_blocks(long long nslices, int sms) {
+  constexpr int warps = kBlock / 32;
+  const long long need = (nslices + warps - 1) / warps;                   // a slice per warp
+  const long long least = (nslices + 64LL * warps - 1) / (64LL * warps);   // 64 slices per warp
+  long long b = 8LL * sms;
+  if (b < least) b = least;
+  return (int)(b < need ? b : need);
+}
 // the FP32 product with launch_block_gram's partial sums for X = P (column pitch
 // ld for both); returns the slots per value
 int launch_ell_spmm_gram(const EllDev<float>& A, const SpmmIO<float>& io, long long ld, int C, const float* r,

@@ -2326,6 +2326,7 @@ mpcg_status mg_autotune(mg_hierarchy* h, const char* cache_path, int* timed_out)
     long long npts;
     int C, dflt, lo, hi;
     std::vector<int> metric;   // kernel classes the shape acts on (documentation)
+    bool used = true;          // some launch of this hierarchy consults it
   };
   std::vector<Tunable> keys;
   keys.push_back({tune::kStream, tune::kAny, gf.npts, 0, stream_blocks_default(gf), stream_blocks_min(gf),
@@ -2337,7 +2338,12 @@ mpcg_status mg_autotune(mg_hierarchy* h, const char* cache_path, int* timed_out)
     if (kind == tune::kF32) d = spmm_blocks<float>(gf, C);
     else if (kind == tune::kDW) d = spmm_blocks<dw>(gf, C);
     else d = spmm_blocks<double>(gf, C);
-    keys.push_back({tune::kSpmm, kind, gf.npts, C, d, stream_blocks_min(gf), stream_blocks_cap(gf), {K_SPMM, K_ALPHA}});
+    // Only the product on a scalar grid's full stencil asks for its blocks: those on
+    // the half stencil, from kappa, of the sparse operators and of the vector grids
+    // take them from the rows, and candidates would be timed on identical launches.
+    const Level& L = h->lev[J];
+    const bool used = !h->algebraic && gf.ncomp == 1 && !(kind == tune::kF32 && (L.sth32 || L.kq32));
+    keys.push_back({tune::kSpmm, kind, gf.npts, C, d, stream_blocks_min(gf), stream_blocks_cap(gf), {K_SPMM}, used});
   }
   if (!h->algebraic && h->opt.smoother == MPCG_SMOOTHER_JACOBI)
     for (int j = 1; j <= J; ++j) {
@@ -2420,6 +2426,11 @@ mpcg_status mg_autotune(mg_hierarchy* h, const char* cache_path, int* timed_out)
     return MPCG_OK;
   };
   for (const Tunable& k : keys) {
+    if (!k.used) {   // the rule's value completes the cache; nothing is timed
+      int v;
+      if (!tune::find(k.fn, k.kind, k.npts, nb, k.C, &v)) tune::set(k.fn, k.kind, k.npts, nb, k.C, k.dflt);
+      continue;
+    }
     std::vector<int> cand = {k.dflt};
     if (k.fn == tune::kJacobi) {
       cand = {0, 1};

@@ -93,3 +93,37 @@ def test_extreme_shapes_are_clamped_and_exact(M, prob, ref, blocks):
     M.mg_autotune_clear()
     assert st == M.MPCG_OK and abs(k - r.iters) <= 1
     assert np.linalg.norm(xg - r.x) <= 1e-10 * np.linalg.norm(r.x)
+
+
+@pytest.mark.parametrize("kind", ["half", "kappa", "elasticity", "sparse"])
+def test_product_blocks_are_timed_only_where_a_launch_takes_them(M, kind):
+    """The products on the half stencil, from kappa, of vector grids and of sparse
+    operators take their blocks from the rows: tuning such a hierarchy times the
+    streaming blocks (at most seven candidates), the Gram chunks (at most four)
+    and the Jacobi widths (two a grid) alone, and leaves a set SpMM value as it
+    is; the full stencil of the same grid adds its candidates (at least two)."""
+    M.mg_autotune_clear()
+    if kind == "sparse":
+        p = pb.poisson_random(2, 1025, 2)
+        H, limit = M.AlgebraicHierarchy(pb.stencil_csr(p), precision=M.MPCG_MIXED), 11
+    elif kind == "elasticity":
+        p = pb.elasticity_cantilever(65)
+        H, limit = M.Hierarchy(torch.from_numpy(np.ascontiguousarray(p.stencil)).cuda(), 3, 65, p.levels, dofs_per_node=3,
+                               faces=p.faces, precision=M.MPCG_MIXED), 11
+    else:
+        p = pb.poisson_random(3, 65, 2)
+        H, F = _hier(M, p, M.MPCG_MIXED), M.Hierarchy(torch.from_numpy(np.ascontiguousarray(p.stencil)).cuda(), 3, 65,
+                                                      p.levels, precision=M.MPCG_MIXED, half_stencil=0)
+        if kind == "kappa":
+            M.mg_attach_q1_kappa(H.h, torch.ones(64 ** 3, dtype=torch.float64, device="cuda"))
+        limit = M.mg_autotune(F.h) - 2
+        F.close()
+        M.mg_autotune_clear()
+        npts = 64 ** 3
+        M.mg_autotune_set(M.MG_TUNE_SPMM_BLOCKS, M.MG_TUNE_F32, npts, 1, p.levels, 77)
+    timed = M.mg_autotune(H.h)
+    assert 2 <= timed <= limit, (timed, limit)
+    if kind in ("half", "kappa"):
+        assert M.mg_autotune_lookup(M.MG_TUNE_SPMM_BLOCKS, M.MG_TUNE_F32, npts, 1, p.levels) == 77
+    H.close()
+    M.mg_autotune_clear()

@@ -413,8 +413,8 @@ __device__ __forceinline__ float half_sweep(float di, float ri, float as1) {
 //   W points per thread: Vec<T>::W (one vector load), or 1 on the small
 //   grids (modes 0 and 1; mode 2 keeps Vec<T>::W).  Every point's
 //   arithmetic is the same whatever W.  SYM: st is the symmetric half
-//   (row_coeffs); its two-sweep mode runs here for W = 1 only and adds a point's
-//   products as k_jacobi_half does, those over the ends of an aligned group of
+//   (row_coeffs); its two-sweep mode exists here for W = 1 only (k_jacobi_half has
+//   the wide form) and adds a point's products as that kernel does, those over the ends of an aligned group of
 //   four apart: the width may depend on the batch, a problem's bits may not.
 template <typename T, int DIM, int W = Vec<T>::W, bool SYM = false>
 __global__ void __launch_bounds__(kBlock, 4) k_jacobi(GridDesc g, const T* __restrict__ st, const T* __restrict__ dinv,
@@ -465,27 +465,28 @@ __global__ void __launch_bounds__(kBlock, 4) k_jacobi(GridDesc g, const T* __res
         else in = fma(a2[0], xr, in);
       }
       o[0] = half_sweep(di[0], ri[0], pos == 0 || pos == 3 ? in + over : in);
-      if (active) out[idx] = o[0];
-      return;
-    }
+    } else if constexpr (!SYM) {
 #pragma unroll
-    for (int k = 0; k < R; ++k) {
-      const long long ro = row_offset<DIM>(k, g.px, g.pxy);
-      T a0[W] = {}, a1[W] = {}, a2[W] = {}, ed[W + 2], er[W + 2];
-      if (active) row_coeffs<T, DIM, W, SYM>(st, g.cp, idx, ro, k, a0, a1, a2);
-      load_row_shfl<T, W>(dinv + idx + ro, ed, active, act, lane);
-      load_row_shfl<T, W>(r + idx + ro, er, active, act, lane);
+      for (int k = 0; k < R; ++k) {
+        const long long ro = row_offset<DIM>(k, g.px, g.pxy);
+        T a0[W] = {}, a1[W] = {}, a2[W] = {}, ed[W + 2], er[W + 2];
+        if (active) row_coeffs<T, DIM, W, false>(st, g.cp, idx, ro, k, a0, a1, a2);
+        load_row_shfl<T, W>(dinv + idx + ro, ed, active, act, lane);
+        load_row_shfl<T, W>(r + idx + ro, er, active, act, lane);
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+          acc[0][w] = fma(a0[w], ed[w] * er[w], acc[0][w]);
+          acc[0][w] = fma(a1[w], ed[w + 1] * er[w + 1], acc[0][w]);
+          acc[0][w] = fma(a2[w], ed[w + 2] * er[w + 2], acc[0][w]);
+        }
+      }
 #pragma unroll
       for (int w = 0; w < W; ++w) {
-        acc[0][w] = fma(a0[w], ed[w] * er[w], acc[0][w]);
-        acc[0][w] = fma(a1[w], ed[w + 1] * er[w + 1], acc[0][w]);
-        acc[0][w] = fma(a2[w], ed[w + 2] * er[w + 2], acc[0][w]);
+        const T s1 = di[w] * ri[w];
+        o[w] = s1 + di[w] * (ri[w] - acc[0][w]);
       }
-    }
-#pragma unroll
-    for (int w = 0; w < W; ++w) {
-      const T s1 = di[w] * ri[w];
-      o[w] = s1 + di[w] * (ri[w] - acc[0][w]);
+    } else {
+      return;   // k_jacobi_half has this mode
     }
   } else if constexpr (W == Vec<T>::W) {   // mode 2 (the launcher uses the full width for it)
     if (!active) return;

@@ -1888,13 +1888,22 @@ static int spmm_half(const GridDesc& g, const float* half, const SpmmIO<float>& 
   // With the 14 planes of a large 3D grid the product's loads fill the registers
   // and the Gram sums cost as much as a launch of their own (129^3, C = 6: 88 us
   // against 62 + 22); up to a segment per warp, two blocks per SM, they are free.
-  const bool alone = part && DIM == 3 && map.nwarps > 16LL * (sm_count() > 0 ? sm_count() : 152);
+  // (A 3D grid that small has at most kGramRegs columns: seven grids take 128
+  // elements a side.)  In 2D they pay up to the widest block, although from ten
+  // columns on the kernel spills: with a launch of their own a Poisson update takes
+  // 8 % longer at 2049^2 and C = 10, 6 % at C = 11 and at 4097^2 with C = 12.
+  const bool alone =
+      part && DIM == 3 && (C > kGramRegs || map.nwarps > 16LL * (sm_count() > 0 ? sm_count() : 152));
   if (alone) part = nullptr;
   const dim3 grid((unsigned)(part ? l.blocks : (32 * map.nwarps + l.threads - 1) / l.threads), g.nb);
 #define MPCG_SPMM_CASE(CC)                                                                                \
   case CC:                                                                                                \
-    if (part) k_spmm_half<DIM, CC, true><<<grid, l.threads, 0, s>>>(g, map, half, io, r, part, state);    \
-    else k_spmm_half<DIM, CC, false><<<grid, l.threads, 0, s>>>(g, map, half, io, r, part, state);        \
+    if constexpr (DIM == 2 || CC <= kGramRegs)                                                            \
+      if (part) {                                                                                         \
+        k_spmm_half<DIM, CC, true><<<grid, l.threads, 0, s>>>(g, map, half, io, r, part, state);          \
+        break;                                                                                            \
+      }                                                                                                   \
+    k_spmm_half<DIM, CC, false><<<grid, l.threads, 0, s>>>(g, map, half, io, r, part, state);             \
     break;
   switch (C) {
     MPCG_SPMM_CASE(1) MPCG_SPMM_CASE(2) MPCG_SPMM_CASE(3) MPCG_SPMM_CASE(4) MPCG_SPMM_CASE(5)

@@ -758,7 +758,8 @@ void enqueue_vsmooth(mg_hierarchy* h, Solver<T>& S, int j, const T* g, T* x, int
 // finest down, nu smoothing steps (SSOR, or damped Jacobi), the defect and
 // its restriction; the exact coarse solve; on the way up the prolongated
 // correction and nu smoothing steps.  Grid j < J keeps its right-hand side
-// in rlev[j], its iterate in zc[j] and its defect in tmp[j].
+// in rlev[j], its iterate in zc[j] and its defect in tmp[j]; a hierarchy of one
+// grid has none of these and solves r exactly into out.
 template <typename T>
 void enqueue_vcycle(mg_hierarchy* h, Solver<T>& S, const T* r, T* out, const DevState* state, cudaStream_t s) {
   const int J = h->levels - 1;
@@ -781,7 +782,7 @@ void enqueue_vcycle(mg_hierarchy* h, Solver<T>& S, const T* r, T* out, const Dev
       LAUNCH(h, K_RESTRICT, s, launch_restrict<T>(L.g, gc, S.tmp[j], S.rlev[j - 1], state, s));
     }
   }
-  LAUNCH(h, K_COARSE, s, launch_coarse_solve<T>(h->lev[0].g, h->A0inv, S.rlev[0], it(0), state, s));
+  LAUNCH(h, K_COARSE, s, launch_coarse_solve<T>(h->lev[0].g, h->A0inv, rhs(0), it(0), state, s));
   for (int j = 1; j <= J; ++j) {
     const Level& L = h->lev[j];
     const GridDesc& gc = h->lev[j - 1].g;

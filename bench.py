@@ -98,20 +98,23 @@ def stencil_words(dim: int, w: int, vector: bool = False) -> int:
     return full // 2 + 1 if w == 4 else full
 
 
-def kernel_work(cls: str, n: int, C: int, cnt: int, w: int, S: int = 27, recurrence: bool = True):
+def kernel_work(cls: str, n: int, C: int, cnt: int, w: int, S: int = 27, recurrence: bool = True, fused: bool = False):
     """Algorithmic HBM bytes and flops of one launch on the fine grid (per
     unknown figures x n; cnt = blocks in the window at that launch; S =
     stored stencil coefficients per unknown, stencil_words).  The flops
     count the full stencil's products whatever is stored.  recurrence: A P
     formed as A Z - sum A P_j beta_j within the orthogonalisation, with the
-    Gram sums; the library forms it by the block SpMM of P (False)."""
+    Gram sums (the model of Algorithm 1 as written); the library forms it by
+    the block SpMM of P (False), where the FP32 products of most grids take the
+    Gram sums P^T A P and P^T r along (fused: no orth_gram launch follows)."""
+    gram = 2 * (C * (C + 1) // 2 + C)                # upper triangle of P^T A P, P^T r
     if cls == "orth_update" and not recurrence:      # read Z, P_j; write P
         return (cnt * C + 2 * C) * w * n, 2 * cnt * C * C * n
-    if cls == "orth_gram" and not recurrence:        # read the new P, A P and r; upper triangle of P^T A P, P^T r
-        return (2 * C + 1) * w * n, 2 * (C * (C + 1) // 2 + C) * n
-    if cls == "spmm" and not recurrence:             # read stencil, P; write A P
+    if cls == "orth_gram" and not recurrence:        # read the new P, A P and r
+        return (2 * C + 1) * w * n, gram * n
+    if cls == "spmm" and not recurrence:             # read stencil, P (fused: and r); write A P
         taps = 81 if S == 81 else (27 if S > 9 else 9)
-        return (S + 2 * C) * w * n, 2 * taps * C * n
+        return (S + 2 * C + (1 if fused else 0)) * w * n, (2 * taps * C + (gram if fused else 0)) * n
     if cls == "orth_update":      # read Z, AZ, P_j, AP_j, r; write P, AP; sym Gram + P^T r
         return (2 * cnt * C + 4 * C + 1) * w * n, 2 * (2 * cnt * C * C + C * (C + 1) + C) * n
     if cls == "gram_window":      # read AP_j, Z
@@ -126,6 +129,38 @@ def kernel_work(cls: str, n: int, C: int, cnt: int, w: int, S: int = 27, recurre
     return None, None
 
 
+# The launch rules of the library that the launch order below follows (scalar grids
+# with Dirichlet faces, two Jacobi sweeps): which grids share a launch of the
+# restriction chain, and which take their two sweeps in two launches.
+TAIL_POINTS, TAIL_THREADS = 512, 768     # grids that the single-block tail takes, padded points
+TWO_LAUNCH_POINTS = 1 << 16              # 8-byte words: padded points from which the sweeps are two launches
+
+
+def padded_points(n: int, dim: int) -> int:
+    """Entries of the padded box of a grid of n unknowns: rows of a multiple of four, one pad row and plane."""
+    n1 = round(n ** (1.0 / dim))
+    return (n1 + 1 + 3) // 4 * 4 * (n1 + 1) ** (dim - 1)
+
+
+def restrict_launches(ns, dim: int):
+    """Grids that each launch of the restriction chain goes down, finest first: one in 3D, in 2D two or three,
+    down to the grid above the tail."""
+    J = len(ns) - 1
+    last = threads = 0
+    for j in range(J):
+        p = padded_points(ns[j], dim)
+        threads += p
+        if p > TAIL_POINTS or threads > TAIL_THREADS:
+            break
+        last = j + 1
+    out, left = [], J - last
+    while left > 0:
+        k = 1 if dim == 3 else (left if left <= 3 else (2 if left % 3 else 3))
+        out.append(k)
+        left -= k
+    return out
+
+
 def level_dofs(nodes, dim, levels):
     """Interior unknowns of every grid, coarsest first."""
     return [((nodes - 1) // 2 ** (levels - 1 - j) - 1) ** dim for j in range(levels)]
@@ -137,10 +172,11 @@ def roofline(trace, ns, C, m, w, peaks, fp64_alu_peak_tflops, S=27, vector=False
 
     The grid of each multilevel launch follows the launch order of one MG
     chain: the smoothings of grids J, J-1, ..., 1 (nu = 2: one fused launch
-    each; vector problems: the first sweep, then the second sweep's
-    residual and block update -- one launch on the fine grid, two on the
-    coarser ones), the
-    restrictions from grids J, ..., 1, one composite prolongation."""
+    each, two on the larger grids of 8-byte words; vector problems: the
+    first sweep, then the second sweep's residual and block update -- one
+    launch on the fine grid, two on the coarser ones), the restrictions
+    (restrict_launches), one composite prolongation.  The product carries the
+    Gram sums where no launch of their own appears."""
     J = len(ns) - 1
     jsub = 0
     tot = {}
@@ -149,7 +185,10 @@ def roofline(trace, ns, C, m, w, peaks, fp64_alu_peak_tflops, S=27, vector=False
     dom = max(tot, key=tot.get)
     cnt = 0
     jj = jr = J
-    jp = 1
+    dim = 3 if S > 9 else 2
+    chain = [1] * J if vector else restrict_launches(ns, dim)
+    kr = 0
+    fused_gram = "orth_gram" not in tot
     bytes_sum = flops_sum = 0.0
     launches = 0
     dur = 0.0
@@ -158,7 +197,7 @@ def roofline(trace, ns, C, m, w, peaks, fp64_alu_peak_tflops, S=27, vector=False
         if cls == "init":
             cnt = 0
         if cls in ("init", "check"):
-            jj, jr, jp, jsub = J, J, 1, 0
+            jj, jr, kr, jsub = J, J, 0, 0
         if cls == "jacobi" and vector:
             fused = ns[jj] // 3 >= (1 << 17) * 0.9   # the fine grids whose last sweep is one launch
             if jsub == 0:     # s1 = D^-1 r: read r, 3 inverse-block planes; write s1
@@ -177,16 +216,24 @@ def roofline(trace, ns, C, m, w, peaks, fp64_alu_peak_tflops, S=27, vector=False
         elif cls == "jacobi":
             Sj = s_fine if (s_fine is not None and jj == J) else S   # matrix-free fine grid: kappa, not stencil
             taps = 27 if S > 9 else 9
-            b, f = (Sj + 3) * w * ns[jj], (2 * taps + 4) * ns[jj]
-            jj -= 1
+            if w == 8 and padded_points(ns[jj], dim) >= TWO_LAUNCH_POINTS:
+                if jsub == 0:     # s1 = dinv r: read r, dinv; write s1
+                    b, f = 3 * w * ns[jj], ns[jj]
+                else:             # s = s1 + dinv (r - A s1): read the stencil, s1, r, dinv; write s
+                    b, f = (Sj + 4) * w * ns[jj], (2 * taps + 3) * ns[jj]
+                jj, jsub = (jj, 1) if jsub == 0 else (jj - 1, 0)
+            else:
+                b, f = (Sj + 3) * w * ns[jj], (2 * taps + 4) * ns[jj]
+                jj -= 1
         elif cls == "restrict":
-            b, f = (ns[jr] + ns[jr - 1]) * w, 2 * 27 * ns[jr - 1]
-            jr -= 1
+            k = chain[kr] if kr < len(chain) else 1
+            b, f = sum(ns[jr - k:jr + 1]) * w, 2 * 3 ** dim * sum(ns[jr - k:jr])
+            jr, kr = jr - k, kr + 1
         elif cls == "prolong":   # composite: write J fine columns, read every coarse correction once
             b, f = (J * ns[J] + sum(ns[:J])) * w, 2 * 8 * J * ns[J]
         elif cls in ("orth_update", "gram_window", "spmm", "update_xr", "orth_gram"):
             b, f = kernel_work(cls, ns[J], C, cnt, w, s_fine if (s_fine is not None and cls == "spmm") else S,
-                               recurrence=False)
+                               recurrence=False, fused=fused_gram)
         if cls == dom:
             if b is not None:
                 bytes_sum += b
@@ -1108,7 +1155,7 @@ def amg_roofline(trace, ns, nnzA, nnzP, C, m, w, peaks):
             b = nnzP[jp] * (4 + w) + jp * (ns[jp - 1] + ns[jp]) * w
             jp += 1
         elif cls == "spmm":
-            b = nnzA[J] * (4 + w) + 2 * C * ns[J] * w
+            b = nnzA[J] * (4 + w) + (2 * C + ("orth_gram" not in tot)) * ns[J] * w
         elif cls in ("orth_update", "gram_window", "update_xr", "orth_gram"):
             b, _ = kernel_work(cls, ns[J], C, cnt, w, recurrence=False)
         if cls == dom:

@@ -50,3 +50,34 @@ def test_roofline_byte_model():
     dom, rl, share, tot = bench.roofline(trace, ns, 2, 5, 4, {"hbm_gbs": 1000.0}, None, S=14)
     assert dom == "jacobi" and rl["launches"] == 2
     assert rl["algorithmic_bytes_per_launch"] == (14 + 3) * 4 * (ns[1] + ns[0]) / 2
+
+
+def test_work_of_the_launches_as_they_are():
+    """A P by the block SpMM of P: the orthogonalisation reads Z and the window's
+    P_j alone, the Gram sums go with the product or in a launch of their own; large
+    grids of 8-byte words smooth in two launches; a 2D restriction chain takes two or
+    three grids a launch and ends above the grids of the single-block tail."""
+    sys.path.insert(0, ROOT)
+    import bench
+    n, C, w, cnt = 1000, 6, 4, 5
+    kw = dict(recurrence=False)
+    assert bench.kernel_work("orth_update", n, C, cnt, w, **kw) == ((cnt + 2) * C * w * n, 2 * cnt * C * C * n)
+    assert bench.kernel_work("orth_gram", n, C, cnt, w, **kw) == ((2 * C + 1) * w * n, 2 * 27 * n)
+    assert bench.kernel_work("spmm", n, C, cnt, w, 14, **kw) == ((14 + 2 * C) * w * n, 2 * 27 * C * n)
+    assert bench.kernel_work("spmm", n, C, cnt, w, 14, fused=True, **kw) == \
+        ((15 + 2 * C) * w * n, 2 * (27 * C + 27) * n)
+    # 129^3: grids of 7^3 and 3^3 unknowns in the tail, three restrictions before it
+    assert bench.padded_points(127 ** 3, 3) == 128 ** 3 and bench.padded_points(95 ** 3, 3) == 96 ** 3
+    assert bench.restrict_launches([1, 27, 343, 3375, 29791, 250047, 2048383][1:], 3) == [1, 1, 1]
+    # 1025^2, nine grids: 15^2 and smaller in the tail, five restrictions in two launches
+    ns = [(2 ** k - 1) ** 2 for k in range(2, 11)]
+    assert bench.restrict_launches(ns, 2) == [2, 3]
+    per = [("restrict", 1.0), ("restrict", 1.0)]
+    dom, rl, _, _ = bench.roofline([("init", 0.0)] + per + [("check", 0.0)] + per, ns, 9, 5, 4, {"hbm_gbs": 1e3}, None, S=5)
+    assert dom == "restrict" and rl["launches"] == 4
+    assert rl["algorithmic_bytes_per_launch"] == 4 * (sum(ns[-3:]) + sum(ns[-6:-2])) / 2
+    # FP64, 65^3: the fine grid takes two launches, the next one; one MG chain
+    ns = [343, 3375, 29791, 250047]
+    trace = [("init", 0.0)] + [("jacobi", 1.0)] * 4 + [("check", 0.0)]
+    _, rl, _, _ = bench.roofline(trace, ns, 5, 5, 8, {"hbm_gbs": 1e3}, None, S=27)
+    assert rl["algorithmic_bytes_per_launch"] == 8 * ((3 + 31) * ns[3] + 30 * (ns[2] + ns[1])) / 4

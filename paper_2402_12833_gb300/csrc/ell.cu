@@ -1,8 +1,8 @@
 // Operators of an algebraic hierarchy (sliced ELLPACK, EllDev in
-// common.cuh): the block SpMM A P of the Section 2.2 update, the residual, damped Jacobi on every grid (Eq. 2,
-// c_0 = 0) and the transfers R_j = P_j^T (restriction) and P_j
-// (prolongation) of Section 2.1.  Vectors are flat padded arrays (unknown i
-// at G + i); every launcher takes pointers already offset by G.
+// common.cuh): the block SpMM A P of the Section 2.2 update, the residual,
+// damped Jacobi on every grid (Eq. 2, c_0 = 0) and the transfers R_j = P_j^T
+// (restriction) and P_j (prolongation) of Section 2.1.  Vectors are flat padded
+// arrays (unknown i at G + i); every launcher takes pointers already offset by G.
 //
 // A warp computes one slice: g lanes per row accumulate every g-th entry and
 // a shuffle reduction over the g lanes finishes the row, so the column and

@@ -276,15 +276,15 @@ void launch_dense_from_stencil(const GridDesc& g, const double* st, double* dens
 void launch_cholesky(double* a, double* rdiag, int n, int* info, cudaStream_t s);
 // inv = A0^{-1} from the Cholesky factor (X: n*n scratch)
 void launch_coarse_inverse(const double* L, const double* rdiag, double* X, double* inv, int n, cudaStream_t s);
-// out = A0^{-1} r; r, out in the padded layout of grid g
 // M = P A0^{-1} P^T (n1 x n1) of the P (CSR, n1 rows, n0 columns) from the coarsest
 // grid; X is n1 x n0 scratch
 void launch_coarse_lift(int n1, int n0, const int* ptr, const int* col, const double* val, const double* inv, double* X,
                         double* M, cudaStream_t s);
+// out = inv r, inv the explicit inverse of grid g's operator (or the lifted one);
+// r, out in the padded layout of grid g
 template <typename T>
 void launch_coarse_solve(const GridDesc& g, const double* inv, const T* r, T* out, const DevState* state,
                          cudaStream_t s);
-// ||r||^2 style sum of partials (value-major) into out[nv]
 // Device side of the mixed-precision refinement loop: mix holds per problem
 // {inner iterations so far, status, active}.
 void launch_mix_init(int* mix, int* active, int nb, int* outer, cudaStream_t s);
@@ -292,6 +292,7 @@ void launch_outer_check(int* mix, int* active, int nb, const double* nrm, double
                         int* outer, DevState* st, double inner_rtol, int m, int C, double delta, double tau,
                         cudaGraphConditionalHandle cond, cudaStream_t s);
 void launch_outer_accumulate(int* mix, int nb, const DevState* st, cudaStream_t s);
+// out[p nv + v] = the sum of problem p's nblk partials of value v (value-major)
 void launch_sum_partials(const double* part, int nb, int nv, int nblk, double* out, cudaStream_t s);
 // x64 += scale * d (padded, FP32 d); scale read from device; xnz[p] = 1
 void launch_axpy_mixed(const GridDesc& g, double* x, const float* d, const double* scale, int* xnz,

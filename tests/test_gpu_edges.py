@@ -245,3 +245,34 @@ def test_training_set_products_and_batches(M):
     loss = M.mg_learned_train([H.h, H2.h], which, R, E, params, epochs=1, batch=1, lr=0.0)
     assert np.array_equal(params, theta)
     assert abs(loss[0] - np.mean(want)) <= 1e-6 * abs(np.mean(want))
+
+
+def test_batches_of_several_pairs(M):
+    """Pairs of two problems in a mixed order, a multiple of the batch each, with a
+    learning rate of zero: the epoch's loss is the mean of the pairs' own losses.
+    And a batch that the pairs do not fill, of the second of two problems: one Adam
+    step along the gradient of its pairs (the first step moves a weight by lr g /
+    (|g| + eps): for entries above a thousandth of the largest, whose sign the
+    order of the sums cannot turn, within 1e-3 lr)."""
+    prob, H = _net(M, 33)
+    prob2 = pb.diffusion_macro(2, 33, 5, rhs="normal", rhs_seed=1)
+    H2 = M.Hierarchy(torch.from_numpy(np.ascontiguousarray(prob2.stencil)).cuda(), 2, 33, prob2.levels,
+                     precision=M.MPCG_MIXED)
+    R, E = _fields(prob, 12)
+    which = [0, 1, 0, 0, 1, 0, 0, 1, 0, 0, 1, 0]
+    theta = OL.init_params(5)
+    want = [M.mg_learned_grad((H, H2)[which[k]].h, theta, R[k:k + 1].contiguous(), E[k:k + 1].contiguous(), 1)[1]
+            for k in range(12)]
+    params = theta.copy()
+    loss = M.mg_learned_train([H.h, H2.h], which, R, E, params, epochs=1, batch=4, lr=0.0)
+    assert np.array_equal(params, theta)
+    assert abs(loss[0] - np.mean(want)) <= 1e-6 * abs(np.mean(want))
+
+    lr = 1e-3
+    R3, E3 = R[:3].contiguous(), E[:3].contiguous()
+    g, l3 = M.mg_learned_grad(H2.h, theta, R3, E3, 3)
+    params = theta.copy()
+    loss = M.mg_learned_train([H.h, H2.h], [1, 1, 1], R3, E3, params, epochs=1, batch=8, lr=lr, eps=1e-12)
+    big = np.abs(g) > 1e-3 * np.abs(g).max()
+    assert big.sum() > 1000 and abs(loss[0] - l3) <= 1e-6 * abs(l3)
+    assert np.abs((params - theta)[big] + lr * np.sign(g[big])).max() <= 1e-3 * lr + 1e-7 * np.abs(theta).max()

@@ -276,3 +276,24 @@ def test_batches_of_several_pairs(M):
     big = np.abs(g) > 1e-3 * np.abs(g).max()
     assert big.sum() > 1000 and abs(loss[0] - l3) <= 1e-6 * abs(l3)
     assert np.abs((params - theta)[big] + lr * np.sign(g[big])).max() <= 1e-3 * lr + 1e-7 * np.abs(theta).max()
+
+
+def test_double_word_elasticity_with_the_fused_sweep(M):
+    """65^3 nodes, 3 unknowns each: the fine grid's second sweep is one launch.  The
+    double-word solve takes the FP64 solve's updates within one and gives its
+    solution (both stop on the same recursion; 1e-9 of the norm), and its residual
+    with the FP64 operator meets the tolerance."""
+    prob = pb.elasticity_cantilever(65)
+    st = torch.from_numpy(np.ascontiguousarray(prob.stencil)).cuda()
+    b = torch.from_numpy(prob.b).cuda()
+    got = []
+    for precision in (M.MPCG_FP64, M.MPCG_FP64_DW):
+        H = M.Hierarchy(st, 3, 65, prob.levels, dofs_per_node=3, faces=prob.faces, precision=precision)
+        x, y = torch.zeros_like(b), torch.zeros_like(b)
+        status, k, _, _ = H.solve(b, x, rtol=1e-8, maxit=100, histories=False)
+        M.mg_apply_operator(H.h, prob.levels - 1, x, y, 1)
+        assert status == M.MPCG_OK and (b - y).norm() <= 1.01e-8 * b.norm()
+        got.append((k, x))
+        H.close()
+    assert abs(got[0][0] - got[1][0]) <= 1
+    assert (got[0][1] - got[1][1]).norm() <= 1e-9 * got[0][1].norm()

@@ -588,8 +588,8 @@ mpcg_status mg_stencil_apply_noalloc(int dim, int nodes, const double* values_de
  * kernels' grid shapes otherwise follow fixed rules measured on GB300).
  * Tunables, each keyed by (tunable, arithmetic, grid points incl. padding,
  * problems in the batch, columns):
- *   MG_TUNE_STREAM_BLOCKS  blocks of the streaming block kernels (A-
- *                          orthogonalisation, update, residual) on a grid;
+ *   MG_TUNE_STREAM_BLOCKS  blocks of the reducing block kernels (update, residual,
+ *                          Gram sums of the new block) on a grid;
  *   MG_TUNE_SPMM_BLOCKS    blocks of the block SpMM on the full stored stencil;
  *   MG_TUNE_GRAM_CHUNKS    point chunks the warps of a row task of the window Gram
  *                          share out;
@@ -606,7 +606,9 @@ mpcg_status mg_stencil_apply_noalloc(int dim, int nodes, const double* values_de
  * solves, the best of three batches after a warm-up batch), one shape at a
  * time against the best found so far, and keeps the fastest.  With cache_path (may be NULL) a
  * cache written on this device that holds every key is loaded instead of
- * timing, and the table is written there afterwards.  Changes results only
+ * timing, and the table is written there afterwards.  The SpMM blocks are timed
+ * where the product takes them, on the full stored stencil of scalar grids; else
+ * a value that is set stays and the rule's is stored.  Changes results only
  * at rounding level (reduction partitions follow the shapes).  Shapes apply
  * to every hierarchy of the process with the same keys; graphs captured
  * before are rebuilt on their next solve.  *timed (may be NULL) gets the

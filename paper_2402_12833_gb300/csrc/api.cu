@@ -2331,7 +2331,7 @@ mpcg_status mg_autotune(mg_hierarchy* h, const char* cache_path, int* timed_out)
   };
   std::vector<Tunable> keys;
   keys.push_back({tune::kStream, tune::kAny, gf.npts, 0, stream_blocks_default(gf), stream_blocks_min(gf),
-                  stream_blocks_cap(gf), {K_ORTH, K_UPDATE, K_RESIDUAL, K_INIT, K_CHECK}});
+                  stream_blocks_cap(gf), {K_OGRAM, K_UPDATE, K_RESIDUAL, K_INIT, K_CHECK, K_ALPHA}});
   keys.push_back({tune::kGram, tune::kAny, gf.npts, 0, gram_chunks_default(gf), gram_chunks_min(gf),
                   gram_chunks_cap(gf), {K_GRAM, K_BETA}});
   {

@@ -502,8 +502,8 @@ __global__ void __launch_bounds__(kBlock, 4) k_jacobi(GridDesc g, const T* __res
 }
 
 // The FP32 block SpMM on the symmetric half, rows read in aligned vectors only
-// (rows.cuh).  Bound by load latency (129^3, C = 6, ncu: DRAM 53 %, L1 41 %, long
-// scoreboard 7 of 11 stall cycles, 16 warps per SM), hence two rows in registers,
+// (rows.cuh).  Bound by load latency (129^3, C = 6, ncu: DRAM 51 %, L1 45 %, long
+// scoreboard 7.7 cycles an instruction, two blocks per SM), hence two rows in registers,
 // the next one's loads issued before the present one's products; C columns per
 // thread, because the columns share the row's coefficients.  Event-timed: 129^3
 // 69 -> 62 us, 1025^2 with C = 9 27 -> 23.6 us.  Slower: three columns per

@@ -4,9 +4,10 @@
 namespace mpcg {
 namespace tune {
 
-// The tunable launch shapes: streaming-kernel blocks (orthogonalisation,
-// update, residual), block-SpMM blocks, window-Gram chunks per window block,
-// and the one-point-per-thread Jacobi switch of a grid (1 on, 0 off).
+// The tunable launch shapes: blocks of the reducing block kernels (update,
+// residual, Gram sums of the new block), block-SpMM blocks (full stencils),
+// window-Gram point chunks, and the one-point-per-thread Jacobi switch of a grid
+// (1 on, 0 off).
 enum { kStream = 0, kSpmm = 1, kGram = 2, kJacobi = 3, kNumTunables = 4 };
 
 // Arithmetic of a keyed shape; kAny for shapes shared by every precision
